@@ -400,7 +400,8 @@ void enqueue_sort(sph_ctx* ctx, bool superset = false)
         ctx->launches += launch_reset_red(L, ctx->npatch, ctx->red);
         ctx->launches += launch_reduce_bbox(L, s, ctx->items, ctx->nitems, ctx->red);
         ctx->launches += launch_h_hist(L, s, ctx->items, ctx->nitems, ctx->red);
-        ctx->launches += launch_grid_params(L, ctx->npatch, ctx->red, ctx->pd, ctx->cell_factor, ctx->status);
+        ctx->launches += launch_grid_params(L, ctx->npatch, ctx->red, ctx->pd, ctx->cell_factor, ctx->status,
+                                            ctx->cf_vote);
     }
     {
         Phase p(ctx, SPH_PHASE_KEYS);
@@ -421,9 +422,8 @@ void enqueue_sort(sph_ctx* ctx, bool superset = false)
                                        superset ? RowHint{ctx->cnt_s, ctx->hint_ok_s, ctx->rowcap}
                                                 : RowHint{ctx->cnt, ctx->hint_ok, ctx->rowcap},
                                        superset ? ctx->hsearch_pre : nullptr, superset ? ctx->skinref.h0 : nullptr);
-        ctx->launches += launch_cell_boxes(L, ctx->npatch, ctx->pd, ctx->grid, ctx->rec.r4);
-        ctx->launches += launch_cell_hnb(L, ctx->npatch, ctx->pd, ctx->grid, stencil_k(ctx->cell_factor), ctx->hnb_tmp);
-        ctx->launches += launch_cell_vote(L, ctx->npatch, ctx->pd, ctx->grid, ctx->cf_vote);
+        ctx->launches += launch_cell_tables(L, ctx->npatch, ctx->pd, ctx->grid, ctx->rec.r4, stencil_k(ctx->cell_factor),
+                                            ctx->hnb_tmp, ctx->cf_vote);
         ctx->cur = nxt;
     }
     ctx->fresh = false;
@@ -440,7 +440,7 @@ void enqueue_lists(sph_ctx* ctx)
     ctx->canon_valid = false;
     {
         Phase p(ctx, SPH_PHASE_NB);
-        ctx->launches += launch_nb_lists(L, a, stencil_k(ctx->cell_factor), 1);
+        ctx->launches += launch_nb_lists(L, a, 1);
     }
     ctx->bins_valid = false;
     // the row lengths now belong to the current order: hints for the next sort
@@ -474,8 +474,7 @@ void enqueue_density(sph_ctx* ctx)
             cudaMemsetAsync(ctx->pool_used + 1, 0, sizeof(unsigned long long), ctx->stream);
         }
         Phase p(ctx, SPH_PHASE_DENSITY);
-        ctx->launches += launch_fused_density(launch_of(ctx), nb_args(ctx), pair_args(ctx),
-                                              stencil_k(ctx->cell_factor), ctx->mixed);
+        ctx->launches += launch_fused_density(launch_of(ctx), nb_args(ctx), pair_args(ctx), ctx->mixed);
         // cnt now holds the row lengths of the current order: hints for the next sort
         cudaMemsetAsync(ctx->hint_ok, 1, sizeof(int), ctx->stream);
         return;
@@ -493,8 +492,7 @@ void enqueue_momentum(sph_ctx* ctx)
 {
     Phase p(ctx, SPH_PHASE_MOMENTUM);
     if (ctx->fused)
-        ctx->launches += launch_fused_momentum(launch_of(ctx), nb_args(ctx), pair_args(ctx),
-                                               stencil_k(ctx->cell_factor), ctx->mixed);
+        ctx->launches += launch_fused_momentum(launch_of(ctx), nb_args(ctx), pair_args(ctx), ctx->mixed);
     else if (ctx->bins_pair) {
         enqueue_bins(ctx);
         ctx->launches += launch_momentum_binned(launch_of(ctx), binned_args(ctx), ctx->bins_pair, ctx->mixed);
@@ -519,7 +517,7 @@ void enqueue_superset(sph_ctx* ctx)
     }
     {
         Phase p(ctx, SPH_PHASE_NB);
-        ctx->launches += launch_nb_lists(L, a, stencil_k(ctx->cell_factor), 0);
+        ctx->launches += launch_nb_lists(L, a, 0);
         ctx->launches += launch_skin_snapshot(L, ctx->n, ctx->st[ctx->cur], ctx->skinref);
     }
     cudaMemsetAsync(ctx->hint_ok_s, 1, sizeof(int), ctx->stream);
@@ -887,7 +885,8 @@ sph_status sph_create(const sph_config* cfg_in, sph_ctx** out)
     uint4* cellrec = nullptr;
     uint32_t* cellxyz = nullptr;
     ok = ok && dalloc(ctx, cellrec, (size_t)ctx->cap_cells) && dalloc(ctx, cellxyz, N) &&
-         dalloc(ctx, ctx->grid.hnb, (size_t)ctx->cap_cells) && dalloc(ctx, ctx->hnb_tmp, (size_t)ctx->cap_cells);
+         dalloc(ctx, ctx->grid.row, (size_t)ctx->cap_cells) && dalloc(ctx, ctx->grid.row_rec, N + 16) &&
+         dalloc(ctx, ctx->grid.row_id, N + 16) && dalloc(ctx, ctx->grid.hnb, (size_t)ctx->cap_cells) && dalloc(ctx, ctx->hnb_tmp, (size_t)ctx->cap_cells);
     ctx->grid.cell = cellrec;
     ctx->grid.cellxyz = cellxyz;
     // kGroup-style padding: the list search reads groups of records past a cell

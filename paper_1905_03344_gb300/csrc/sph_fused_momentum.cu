@@ -5,13 +5,13 @@
 
 namespace sphg {
 
-int launch_fused_momentum(const Launch& L, const NbArgs& a, const PairArgs& pa, int K, int mixed)
+int launch_fused_momentum(const Launch& L, const NbArgs& a, const PairArgs& pa, int mixed)
 {
     if (a.n <= 0 || a.nunits <= 0) return 0;
     if (mixed) {
-        SPH_FUSED_DISPATCH(k_fused_momentum_mixed, K, L, a, pa);
+        SPH_FUSED_DISPATCH(k_fused_momentum_mixed, L, a, pa);
     } else {
-        SPH_FUSED_DISPATCH(k_fused_momentum_fp64, K, L, a, pa);
+        SPH_FUSED_DISPATCH(k_fused_momentum_fp64, L, a, pa);
     }
     return 1;
 }

@@ -7,8 +7,8 @@
 // patch is big).  A uniform grid of cells with edge s >= 2 h_s cell_factor
 // covers the bounding box in x, y and the period lz in z; a small particle
 // searches the (2K+1)^3 cells around its own (K = 1 for cell_factor >= 1,
-// 2 for >= 1/2, 3 below) for small neighbours, pruned by the largest h
-// around its cell and by each cell's own largest h.  Big
+// 2 for >= 1/2, 3 below) for small neighbours, row by row, pruned by the
+// largest h around its cell.  Big
 // particles are indexed separately by coarse cells (aligned blocks of 2^kc
 // fine cells with edge >= 2 h_max), which every particle searches for big
 // neighbours; a big particle searches the fine grid as far as its own 2 h.
@@ -73,6 +73,7 @@ struct PatchDev {
     int32_t ncx, ncy, ncz, K;
     int32_t zmode;               // 0: 2K+1 distinct z cells; 1: all z cells + float wrap
     int32_t nbig;                // big particles (h > hs), counted by the key kernel
+    uint32_t row_fill;           // slots of the row copy handed out so far
     double hs;                   // class threshold: small iff h <= hs
     float hs_f;
     double hmed;                 // median of h (histogram bin centre)
@@ -104,14 +105,19 @@ struct State {
 
 // Cell record, 16 bytes: particles [x, y) of the sorted order (x = y: empty;
 // fine cells hold small particles, coarse cells big ones), z = the largest h
-// in the cell (FP32 bits), w = for fine cells the tight box of the cell's
-// particles, as insets from the cell faces in 1/kBoxQ of the cell edge:
-// bits 0-4 low x, 5-9 high x, 10-14 low y, 15-19 high y, 20-24 low z,
-// 25-29 high z (a particle with offset o lies in [lo, kBoxQ - hi) / kBoxQ of
-// the edge, up to the FP32 rounding of o).
-constexpr int kBoxQ = 32;
+// in the cell (FP32 bits).
+//
+// The search reads its small candidates from a second copy of the records, in
+// which the particles of a row of fine cells (all x at one y, z) are
+// contiguous and ordered by cell: row[fine cell] = {first, end} slot of the
+// cell in that copy, row_rec = {x from the grid's origin, oy, oz, 4 h^2} and
+// row_id = sorted slot | x cell << kColBits.  A row of the search sphere is
+// then one run of slots, where the Morton order holds one run per cell.
 struct Grid {
     uint4* cell;         // [cell] record above
+    uint2* row;          // [fine cell]
+    float4* row_rec;     // [slot], padded past the end (read in groups)
+    uint32_t* row_id;    // [slot], padded likewise
     uint32_t* cellxyz;   // [particle] cx | cy << 8 | cz << 16
     const uint16_t* patch_of;  // [particle] patch index
     float* hnb;          // [fine cell] the largest h of the fine cells within
@@ -183,7 +189,7 @@ int launch_reduce_bbox(const Launch& L, const State& s, const WorkItem* items, i
                        PatchRed* red);
 int launch_h_hist(const Launch& L, const State& s, const WorkItem* items, int nitems, PatchRed* red);
 int launch_grid_params(const Launch& L, int npatch, const PatchRed* red, PatchDev* pd,
-                       double cell_factor, int* status);
+                       double cell_factor, int* status, unsigned long long* vote);
 int launch_keys(const Launch& L, int64_t n, const State& s, const uint16_t* patch_of,
                 PatchDev* pd, uint32_t* keys, uint32_t* vals);
 // LSD radix sort of (keys, vals); result in (keys, vals); uses alternates.
@@ -211,14 +217,13 @@ int launch_gather(const Launch& L, int64_t n, const uint32_t* skeys, const uint3
 // grid of the last sort (what the gather writes, with the unscaled h)
 int launch_refresh_records(const Launch& L, int64_t n, const State& s, const uint16_t* patch_of,
                            const PatchDev* pd, const uint32_t* cellxyz, const Recs& r, const Fp64& f, int mixed);
-// tight boxes of the fine cells (after the gather)
-int launch_cell_boxes(const Launch& L, int npatch, const PatchDev* pd, const Grid& g, const float4* r4);
-// g.hnb for stencil half-extent K (tmp: one float per cell)
-int launch_cell_hnb(const Launch& L, int npatch, const PatchDev* pd, const Grid& g, int K, float* tmp);
-// the state's vote for the grid of the next sort (vote[0]: non-empty fine
-// cells, vote[1]: those whose hnb is below 0.8 h_s in a patch with h_s above
-// 1.4 h_median); vote is cleared here
-int launch_cell_vote(const Launch& L, int npatch, const PatchDev* pd, const Grid& g, unsigned long long* vote);
+// after the gather: the row copy of the small particles' search records,
+// g.hnb for stencil half-extent K (tmp: one float per cell) and the state's
+// vote for the grid of the next sort (vote[0]: non-empty fine cells, vote[1]:
+// those whose hnb is below 0.8 h_s in a patch with h_s above 1.4 h_median;
+// cleared by launch_grid_params)
+int launch_cell_tables(const Launch& L, int npatch, PatchDev* pd, const Grid& g, const float4* r4, int K, float* tmp,
+                       unsigned long long* vote);
 // temporary words of the device-wide exclusive scan over n values
 int64_t scan_tmp_words(int64_t n);
 
@@ -240,10 +245,9 @@ struct NbArgs {
     int64_t pool_cap;                    // entries the pool holds (max_pairs + slack)
     int* status;
 };
-// K: stencil half-extent of every patch (1 for cell_factor >= 1, 2 for >= 1/2, else 3)
 // exact = 1: the neighbour lists and n_i; exact = 0: the candidate superset
 // of reused lists (every candidate within the grid's scaled search radius)
-int launch_nb_lists(const Launch& L, const NbArgs& a, int K, int exact);
+int launch_nb_lists(const Launch& L, const NbArgs& a, int exact);
 // exact lists (a.col, a.cnt, a.nown; rows at a.rowstart) from the superset
 // rows col_s / cnt_s at the same offsets, on the current records and state
 int launch_nb_filter(const Launch& L, const NbArgs& a, const uint32_t* col_s, const uint32_t* cnt_s);
@@ -297,11 +301,10 @@ int launch_pair_bins(const Launch& L, int64_t n, const uint32_t* cnt, uint32_t* 
 // distinct lanes-per-particle value)
 int launch_density_binned(const Launch& L, PairArgs a, int w, int mixed);
 int launch_momentum_binned(const Launch& L, PairArgs a, int w, int mixed);
-// list-free pair sums over the search of the current grid (stencil
-// half-extent K); the density pass also writes |N(i)| and n_i and adds the
+// list-free pair sums over the search of the current grid; the density pass also writes |N(i)| and n_i and adds the
 // pairs to pool_used[1]
-int launch_fused_density(const Launch& L, const NbArgs& a, const PairArgs& pa, int K, int mixed);
-int launch_fused_momentum(const Launch& L, const NbArgs& a, const PairArgs& pa, int K, int mixed);
+int launch_fused_density(const Launch& L, const NbArgs& a, const PairArgs& pa, int mixed);
+int launch_fused_momentum(const Launch& L, const NbArgs& a, const PairArgs& pa, int mixed);
 
 struct StepArgs {
     int64_t n;

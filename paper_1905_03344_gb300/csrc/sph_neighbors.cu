@@ -22,11 +22,11 @@ namespace sphg {
 
 // counting walk (col = nullptr) and repair walk (straight to the pool): one
 // out-of-line copy serves both
-template <int K, bool EXACT>
+template <bool EXACT>
 __device__ __noinline__ RowSink<kWalkFlat, EXACT> walk_all_flat(const NbArgs& a, const PatchDev* P, int64_t i,
                                                              bool big, RowSink<kWalkFlat, EXACT> row)
 {
-    walk_all<RowSink<kWalkFlat, EXACT>, K>(a, P, i, big, row);
+    walk_all<RowSink<kWalkFlat, EXACT>>(a, P, i, big, row);
     return row;
 }
 
@@ -39,10 +39,9 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, int lane)
     return v;
 }
 
-// K: stencil half-extent, the same for every patch (it follows cell_factor);
 // EXACT = false: the candidate superset (every candidate within the scaled
 // search radius in FP32, no n_i)
-template <int K, bool EXACT>
+template <bool EXACT>
 __global__ void __launch_bounds__(32 * kNbtWarps, SPH_NB_MINB) k_nb_thread(NbArgs a)
 {
     extern __shared__ __align__(16) uint32_t nb_ring[];
@@ -63,7 +62,7 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_NB_MINB) k_nb_thread(NbArg
             const uint32_t hint = a.rowcap[i];
             if (hint == kNoHint) {
                 const RowSink<kWalkFlat, EXACT> rc =
-                    walk_all_flat<K, EXACT>(a, P, i, big, RowSink<kWalkFlat, EXACT>{nullptr, nullptr, 0u, 0u, 0u, 0u});
+                    walk_all_flat<EXACT>(a, P, i, big, RowSink<kWalkFlat, EXACT>{nullptr, nullptr, 0u, 0u, 0u, 0u});
                 res = round8(rc.cnt);
             } else {
                 const uint32_t c = min(hint, (uint32_t)a.n);
@@ -80,7 +79,7 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_NB_MINB) k_nb_thread(NbArg
         unsigned long long r0 = base + (inc - res);
         RowSink<kWalkRing, EXACT> row = {a.col + r0, ring, ok ? res : 0u, 0u, 0u, 0u};
         if (act) {
-            walk_all<RowSink<kWalkRing, EXACT>, K>(a, P, i, big, row);
+            walk_all<RowSink<kWalkRing, EXACT>>(a, P, i, big, row);
             row.finish();
             // only a row that is in the pool (within the sink's reservation,
             // which is 0 for a warp whose reservation did not fit)
@@ -92,7 +91,7 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_NB_MINB) k_nb_thread(NbArg
             const uint32_t need = round8(row.cnt);
             r0 = atomicAdd(&a.pool_used[0], (unsigned long long)need);
             if (r0 + need <= pool_cap) {
-                const RowSink<kWalkFlat, EXACT> rr = walk_all_flat<K, EXACT>(
+                const RowSink<kWalkFlat, EXACT> rr = walk_all_flat<EXACT>(
                     a, P, i, big, RowSink<kWalkFlat, EXACT>{a.col + r0, nullptr, need, 0u, 0u, 0u});
                 row.cnt = rr.cnt;
                 row.own = rr.own;
@@ -113,13 +112,13 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_NB_MINB) k_nb_thread(NbArg
     }
 }
 
-template <int K, bool EXACT>
+template <bool EXACT>
 void launch_nb_thread(const Launch& L, const NbArgs& a)
 {
     const size_t smem = sizeof(uint32_t) * 32 * (kRing + kPend) * kNbtWarps;
     static int per_sm = 0;
     if (!per_sm) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_nb_thread<K, EXACT>, 32 * kNbtWarps, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_nb_thread<EXACT>, 32 * kNbtWarps, smem);
         if (per_sm < 1) per_sm = 1;
         // shared memory only for the rings of the resident CTAs: the rest is L1
         int smem_max = 0, dev = 0;
@@ -129,24 +128,17 @@ void launch_nb_thread(const Launch& L, const NbArgs& a)
             const size_t need = (size_t)per_sm * (smem + 1024);
             int pct = (int)((need * 100 + (size_t)smem_max - 1) / (size_t)smem_max);
             pct = pct < 1 ? 1 : (pct > 100 ? 100 : pct);
-            cudaFuncSetAttribute(k_nb_thread<K, EXACT>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+            cudaFuncSetAttribute(k_nb_thread<EXACT>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
         }
     }
-    k_nb_thread<K, EXACT><<<L.sms * per_sm, 32 * kNbtWarps, smem, L.stream>>>(a);
+    k_nb_thread<EXACT><<<L.sms * per_sm, 32 * kNbtWarps, smem, L.stream>>>(a);
 }
 
-int launch_nb_lists(const Launch& L, const NbArgs& a, int K, int exact)
+int launch_nb_lists(const Launch& L, const NbArgs& a, int exact)
 {
     if (a.n <= 0 || a.nunits <= 0) return 0;
-    if (exact) {
-        if (K == 1) launch_nb_thread<1, true>(L, a);
-        else if (K == 2) launch_nb_thread<2, true>(L, a);
-        else launch_nb_thread<3, true>(L, a);
-    } else {
-        if (K == 1) launch_nb_thread<1, false>(L, a);
-        else if (K == 2) launch_nb_thread<2, false>(L, a);
-        else launch_nb_thread<3, false>(L, a);
-    }
+    if (exact) launch_nb_thread<true>(L, a);
+    else launch_nb_thread<false>(L, a);
     return 1;
 }
 

@@ -163,9 +163,10 @@ int launch_reset_red(const Launch& L, int npatch, PatchRed* red)
 // every z cell is visited once and the minimum image is taken in FP32.
 // ---------------------------------------------------------------------------
 __global__ void k_grid_params(int npatch, const PatchRed* red, PatchDev* pd, double cell_factor,
-                              int* status)
+                              int* status, unsigned long long* vote)
 {
     int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < 2) vote[p] = 0ull;          // counted afresh by k_cell_hnb
     if (p >= npatch) return;
     PatchDev P = pd[p];
     const int K = stencil_k(cell_factor);
@@ -273,6 +274,7 @@ __global__ void k_grid_params(int npatch, const PatchRed* red, PatchDev* pd, dou
     P.hs_f = (float)hs;
     P.hmed = hmed;
     P.nbig = 0;
+    P.row_fill = 0;
     P.kc = kc;
     P.ncxc = (int)ncxc;
     P.ncyc = (int)ncyc;
@@ -283,9 +285,9 @@ __global__ void k_grid_params(int npatch, const PatchRed* red, PatchDev* pd, dou
 }
 
 int launch_grid_params(const Launch& L, int npatch, const PatchRed* red, PatchDev* pd,
-                       double cell_factor, int* status)
+                       double cell_factor, int* status, unsigned long long* vote)
 {
-    k_grid_params<<<(npatch + 127) / 128, 128, 0, L.stream>>>(npatch, red, pd, cell_factor, status);
+    k_grid_params<<<(npatch + 127) / 128, 128, 0, L.stream>>>(npatch, red, pd, cell_factor, status, vote);
     return 1;
 }
 
@@ -767,101 +769,110 @@ int launch_refresh_records(const Launch& L, int64_t n, const State& s, const uin
 }
 
 // ---------------------------------------------------------------------------
-// The tight box of each non-empty fine cell, from its particles' FP32
-// offsets, quantised outward to 1/kBoxQ of the cell edge (see Grid).  One
-// thread per cell; blockIdx.y is the patch.
+// The row copy of the small particles' search records (see Grid): one warp
+// per row of fine cells, which reserves the row's slots (where in the copy a
+// row lies depends on scheduling, its contents do not), scans the cells'
+// counts and copies their particles: 36 bytes a particle, 0.11 ms at 8 M.
+// The warp also leaves the row's running maximum of h over K cells to each
+// side in hnb_x.  blockIdx.y is the patch.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int box_q(float o, float inv_edge)
+__global__ void __launch_bounds__(256) k_cell_rows(PatchDev* pd, Grid g, const float4* r4, int K, float* hnb_x)
 {
-    const int q = (int)floorf(o * inv_edge * (float)kBoxQ);
-    return min(max(q, 0), kBoxQ - 1);
-}
-
-__global__ void __launch_bounds__(256) k_cell_boxes(const PatchDev* pd, Grid g, const float4* r4)
-{
-    const PatchDev* P = pd + blockIdx.y;
-    const int64_t nfine = (int64_t)P->ncx * P->ncy * P->ncz;
-    const float inv_s = P->inv_s_f, inv_sz = P->inv_sz_f;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nfine; c += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t lin = P->cell_base + c;
-        const uint32_t b = g.cell[lin].x, e = g.cell[lin].y;
-        if (b >= e) continue;
-        int lx = kBoxQ, ly = kBoxQ, lz = kBoxQ, hx = 0, hy = 0, hz = 0;
-        for (uint32_t k = b; k < e; k++) {
-            const float4 q = r4[k];
-            const int qx = box_q(q.x, inv_s), qy = box_q(q.y, inv_s), qz = box_q(q.z, inv_sz);
-            lx = min(lx, qx);
-            ly = min(ly, qy);
-            lz = min(lz, qz);
-            hx = max(hx, qx + 1);
-            hy = max(hy, qy + 1);
-            hz = max(hz, qz + 1);
+    constexpr int kPad = 4;             // at least K
+    __shared__ float sh[8][kMaxCellsAxis + 2 * kPad];
+    PatchDev* P = pd + blockIdx.y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ncx = P->ncx, nrows = P->ncy * P->ncz;
+    const float s_f = P->s_f;
+    const uint32_t first = (uint32_t)P->begin;
+    for (int r = (int)blockIdx.x * 8 + warp; r < nrows; r += (int)gridDim.x * 8) {
+        const int64_t lin = P->cell_base + (int64_t)r * ncx;
+        // at most kMaxCellsAxis cells: four per lane, 32 apart
+        uint32_t beg[4], off[4], cnt[4], tot = 0;
+        if (lane < kPad) sh[warp][lane] = sh[warp][kPad + ncx + lane] = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int x = k * 32 + lane;
+            beg[k] = cnt[k] = off[k] = 0;
+            if (k * 32 < ncx) {
+                if (x < ncx) {
+                    const uint4 c = g.cell[lin + x];
+                    beg[k] = c.x;
+                    cnt[k] = c.y - c.x;
+                    sh[warp][kPad + x] = __uint_as_float(c.z);
+                }
+                uint32_t inc = cnt[k];
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (lane >= o) inc += t;
+                }
+                off[k] = tot + inc - cnt[k];
+                tot += __shfl_sync(0xffffffffu, inc, 31);
+            }
         }
-        g.cell[lin].w = (uint32_t)lx | ((uint32_t)(kBoxQ - hx) << 5) | ((uint32_t)ly << 10) |
-                        ((uint32_t)(kBoxQ - hy) << 15) | ((uint32_t)lz << 20) | ((uint32_t)(kBoxQ - hz) << 25);
+        uint32_t base = 0;
+        if (lane == 0 && tot) base = first + atomicAdd(&P->row_fill, tot);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int x = k * 32 + lane;
+            if (x >= ncx) continue;
+            const uint32_t b = base + off[k];
+            g.row[lin + x] = make_uint2(b, b + cnt[k]);
+            float m = 0.0f;
+            for (int d = -K; d <= K; d++) m = fmaxf(m, sh[warp][kPad + x + d]);
+            hnb_x[lin + x] = m;
+            for (uint32_t u = 0; u < cnt[k]; u++) {
+                const uint32_t j = beg[k] + u;
+                const float4 q = r4[j];
+                g.row_rec[b + u] = make_float4(fmaf((float)x, s_f, q.x), q.y, q.z, q.w);
+                g.row_id[b + u] = j | ((uint32_t)x << kColBits);
+            }
+        }
+        __syncwarp();
     }
 }
 
-// The largest h within K fine cells of each fine cell along each axis, a
-// separable maximum in three passes: along x and along y (in range), then
-// over 2K+1 z planes (periodic; with fewer z cells than that, every plane).
-// A small particle's search from this cell reaches no farther than
-// 2 max(h_i, hnb).  axis 0 reads the cell table's h_max, the others the
-// previous pass.
-__global__ void __launch_bounds__(256) k_hnb_pass(const PatchDev* pd, Grid g, int K, int axis, const float* in,
-                                                  float* out)
-{
-    const PatchDev* P = pd + blockIdx.y;
-    const int ncx = P->ncx, ncy = P->ncy, ncz = P->ncz;
-    const int64_t nxy = (int64_t)ncx * ncy;
-    const int64_t nfine = nxy * ncz;
-    const int n = axis == 0 ? ncx : (axis == 1 ? ncy : ncz);
-    const int64_t stride = axis == 0 ? 1 : (axis == 1 ? ncx : nxy);
-    // every z plane when they are fewer than 2K+1
-    const int kk = axis == 2 && 2 * K + 1 > ncz ? (ncz - 1) / 2 + 1 : K;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nfine; c += (int64_t)gridDim.x * blockDim.x) {
-        const int pos = (int)((c / stride) % n);
-        const int64_t c0 = c - (int64_t)pos * stride;
-        float m = 0.0f;
-        for (int d = -kk; d <= kk; d++) {
-            int q = pos + d;
-            if (axis == 2) q = ((q % n) + n) % n;
-            else if (q < 0 || q >= n) continue;
-            const int64_t cell = P->cell_base + c0 + (int64_t)q * stride;
-            m = fmaxf(m, axis == 0 ? __uint_as_float(g.cell[cell].z) : in[cell]);
-        }
-        out[P->cell_base + c] = m;
-    }
-}
-
-int launch_cell_hnb(const Launch& L, int npatch, const PatchDev* pd, const Grid& g, int K, float* tmp)
-{
-    if (npatch <= 0) return 0;
-    const dim3 grid(npatch > 8 ? 8 : (L.sms * 4 + npatch - 1) / npatch, npatch);
-    k_hnb_pass<<<grid, 256, 0, L.stream>>>(pd, g, K, 0, nullptr, g.hnb);
-    k_hnb_pass<<<grid, 256, 0, L.stream>>>(pd, g, K, 1, g.hnb, tmp);
-    k_hnb_pass<<<grid, 256, 0, L.stream>>>(pd, g, K, 2, tmp, g.hnb);
-    return 3;
-}
-
-// The vote of the cell grid for the next sort: the fine cells that hold
+// The largest h within K fine cells of each fine cell along each axis, from
+// the maxima along x: over 2K+1 rows in y (in range) and 2K+1 z planes
+// (periodic; with fewer z cells than that, every plane).  A small particle's
+// search from this cell reaches no farther than 2 max(h_i, hnb).
+//
+// And the vote of the cell grid for the next sort: the fine cells that hold
 // particles, and among them, in a patch whose spread of h is wide (h_s >
 // 1.4 h_median), those whose particles' neighbourhoods have no h above 0.8
 // h_s.  Many such cells (h wide but smooth in space, as behind the free
 // surface of a patch) favour a 3-cell stencil over median-sized cells; few
 // (h varying from particle to particle) favour cells of edge h_s.
-__global__ void __launch_bounds__(256) k_cell_vote(const PatchDev* pd, Grid g, unsigned long long* vote)
+__global__ void __launch_bounds__(256) k_cell_hnb(const PatchDev* pd, Grid g, int K, const float* hnb_x, unsigned long long* vote)
 {
     const PatchDev* P = pd + blockIdx.y;
-    const int64_t nfine = (int64_t)P->ncx * P->ncy * P->ncz;
+    const int ncx = P->ncx, ncy = P->ncy, ncz = P->ncz;
+    const int64_t nxy = (int64_t)ncx * ncy;
+    const int64_t nfine = nxy * ncz;
     const bool wide = P->hs > 1.4 * P->hmed;
     const float lim = 0.8f * P->hs_f;
+    // every z plane when they are fewer than 2K+1
+    const int kz = 2 * K + 1 > ncz ? (ncz - 1) / 2 + 1 : K;
     uint32_t ne = 0, nn = 0;
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nfine; c += (int64_t)gridDim.x * blockDim.x) {
+        const int z = (int)(c / nxy), y = (int)(c - z * nxy) / ncx;
+        const int ylo = max(-K, -y), yhi = min(K, ncy - 1 - y);
+        float m = 0.0f;
+        for (int dz = -kz; dz <= kz; dz++) {
+            int q = z + dz;
+            while (q < 0) q += ncz;
+            while (q >= ncz) q -= ncz;
+            const float* p = hnb_x + P->cell_base + c + (int64_t)(q - z) * nxy;
+            for (int dy = ylo; dy <= yhi; dy++) m = fmaxf(m, p[(int64_t)dy * ncx]);
+        }
+        g.hnb[P->cell_base + c] = m;
         const uint4 cr = g.cell[P->cell_base + c];
-        if (cr.x >= cr.y) continue;
-        ne++;
-        nn += (uint32_t)(wide && g.hnb[P->cell_base + c] < lim);
+        if (cr.x < cr.y) {
+            ne++;
+            nn += (uint32_t)(wide && m < lim);
+        }
     }
     for (int o = 16; o > 0; o >>= 1) {
         ne += __shfl_xor_sync(0xffffffffu, ne, o);
@@ -873,21 +884,15 @@ __global__ void __launch_bounds__(256) k_cell_vote(const PatchDev* pd, Grid g, u
     }
 }
 
-int launch_cell_vote(const Launch& L, int npatch, const PatchDev* pd, const Grid& g, unsigned long long* vote)
-{
-    cudaMemsetAsync(vote, 0, 2 * sizeof(unsigned long long), L.stream);
-    if (npatch <= 0) return 0;
-    const dim3 grid(npatch > 8 ? 8 : (L.sms * 4 + npatch - 1) / npatch, npatch);
-    k_cell_vote<<<grid, 256, 0, L.stream>>>(pd, g, vote);
-    return 1;
-}
-
-int launch_cell_boxes(const Launch& L, int npatch, const PatchDev* pd, const Grid& g, const float4* r4)
+int launch_cell_tables(const Launch& L, int npatch, PatchDev* pd, const Grid& g, const float4* r4, int K, float* tmp,
+                       unsigned long long* vote)
 {
     if (npatch <= 0) return 0;
-    const int bx = npatch > 8 ? 8 : (L.sms * 4 + npatch - 1) / npatch;
-    k_cell_boxes<<<dim3((unsigned)bx, (unsigned)npatch), 256, 0, L.stream>>>(pd, g, r4);
-    return 1;
+    const int rows_x = npatch > 8 ? 64 : (L.sms * 8 + npatch - 1) / npatch;
+    const int cells_x = npatch > 8 ? 16 : (L.sms * 8 + npatch - 1) / npatch;
+    k_cell_rows<<<dim3((unsigned)rows_x, (unsigned)npatch), 256, 0, L.stream>>>(pd, g, r4, K, tmp);
+    k_cell_hnb<<<dim3((unsigned)cells_x, (unsigned)npatch), 256, 0, L.stream>>>(pd, g, K, tmp, vote);
+    return 2;
 }
 
 }  // namespace sphg

@@ -6,10 +6,10 @@
 // One thread per particle; a warp serves 32 consecutive sorted particles of
 // one patch.  The search has up to three parts, each visiting every
 // candidate of its kind once:
-//   small i, small j: the (2K+1)^3 fine cells around i's cell (template K),
-//     pruned by distance against 2 max(h_i, hnb) (hnb: the largest h around
-//     i's cell) and then against 2 max(h_i, h_max(cell));
-//   big i, small j:   the fine cells within 2 h_i of i (runtime extent);
+//   small i, small j: the rows of fine cells (all x at one y, z) around i's
+//     cell, at most K away, each clipped to the chord of the radius
+//     2 max(h_i, hnb) (hnb: the largest h around i's cell);
+//   big i, small j:   the same rows as far as 2 max(h_i, h_s) reaches;
 //   any i, big j:     the 3 x 3 x 3 coarse cells around i's coarse cell
 //     (only when the patch has big particles).
 // Small particles never reach farther than 2 h_s, and every big one lies in
@@ -75,6 +75,14 @@ constexpr uint32_t kHintMargin = 8;     // growth a row may have since the hint,
 __device__ __forceinline__ float guard_tol(float s_over_h, int D)
 {
     return kTolBase + kTolCell * s_over_h * fmaxf(1.0f, (float)D * (1.0f / 3.0f));
+}
+
+// The same for candidates of the row copy, whose x is taken from the grid's
+// origin: one rounding of up to 2^-24 of kMaxCellsAxis cells on each side,
+// 2^-16 s together, is at most 2^-16 s/h of T; four times that.
+__device__ __forceinline__ float row_tol(float s_over_h, int D)
+{
+    return guard_tol(s_over_h, D) + (1.0f / 16384.0f) * s_over_h;
 }
 
 enum WalkMode { kWalkRing = 0, kWalkFlat = 1 };
@@ -219,22 +227,21 @@ __device__ __forceinline__ uint32_t stencil_code(const PatchDev* P, int dcx, int
     return (uint32_t)((dcx + 2) + 5 * (dcy + 2) + 25 * zd);
 }
 
-// squared distance from i to the tight box of a fine cell: g*r are the raw
-// distances from i to the cell's near faces (-1e30 along an axis where i is
-// inside the cell's slab), the insets come from the cell record at the given
-// bit offsets, in units qs = s / kBoxQ (qsz = sz / kBoxQ along z)
-__device__ __forceinline__ float tight_gap2(uint32_t box, float gxr, uint32_t xs, float gyr, uint32_t ys, float gzr,
-                                            uint32_t zs, float qs, float qsz)
-{
-    const float tx = fmaxf(fmaf((float)((box >> xs) & 31u), qs, gxr), 0.0f);
-    const float ty = fmaxf(fmaf((float)((box >> ys) & 31u), qs, gyr), 0.0f);
-    const float tz = fmaxf(fmaf((float)((box >> zs) & 31u), qsz, gzr), 0.0f);
-    return fmaf(tx, tx, fmaf(ty, ty, tz * tz));
-}
-
-// ---- small i, small j: the (2K+1)^3 fine cells around i's cell ------------
-template <class S, int K, int ZW>
-__device__ __forceinline__ void walk_small(const NbArgs& a, const PatchDev* P, int64_t i, S& row)
+// ---- any i, small j: the rows of fine cells within reach -------------------
+// (2 kx + 1) x (2 kz + 1) rows around i's cell (every z plane with ZW), each
+// clipped to the chord of the search sphere: one run of the row copy.  Bound
+// by instruction issue (70 % of cycles) and by the L1's gathers (71 %).  A
+// walk over cells, pruned by each cell's tight box, tested about as many
+// candidates but paid ~35 instructions for each of ~82 cells and ended a
+// group of four in every one of them; the rows come to 13-21 runs.  Search of
+// 8 M particles (a 200^3 lattice disturbed by 4 %) 10.24 -> 8.63 ms, of the
+// 64-patch batch 7.66 -> 5.90, of the 80^3 irregular patch 1.41 -> 1.25, of
+// 45^3 176 -> 137 us; 100^3 with h raised by a third behind the surface 1.12
+// (unchanged: its cells are 1.3 times as wide).  Slower: lanes that leave the
+// lockstep of the rows for their own runs (L1 77-90 % busy), hits without
+// branches, ids loaded only for hits, groups of 3 or 5.
+template <class S, int ZW>
+__device__ __forceinline__ void walk_rows(const NbArgs& a, const PatchDev* P, int64_t i, int kx, int kz, float Rg2, S& row)
 {
     const float s_f = P->s_f, sz_f = P->sz_f, lz_f = P->lz_f, inv_lz = 1.0f / P->lz_f;
     const int ncx = P->ncx, ncy = P->ncy, ncz = P->ncz;
@@ -246,223 +253,120 @@ __device__ __forceinline__ void walk_small(const NbArgs& a, const PatchDev* P, i
     const float hf = (float)a.h[i];
     const float Ti = ri.w;
     // every z cell visited (ZW): shifts of up to ncz - 1 cells along z
-    const float tol = guard_tol(s_f / hf, ZW ? max(K, ncz) : K);
+    const float tol = row_tol(s_f / hf, ZW ? max(kx, ncz) : max(kx, kz));
     const float flo = 1.0f - tol, fhi = 1.0f + tol;
-    const float slack = (1.0f / 4096.0f) * s_f;
-    // no small neighbour within the stencil has h above hnb of i's cell
-    const float hn = a.g.hnb[cbase + ((uint32_t)cz * (uint32_t)ncy + (uint32_t)cy) * (uint32_t)ncx + (uint32_t)cx];
-    const float Rg = 2.0f * fmaxf(hf, hn) * (1.0f + 1.0f / 512.0f) + slack;
-    const float Rg2 = Rg * Rg;
-    const float Rc = 2.0f * (1.0f + 1.0f / 512.0f);
-    const float qs = s_f * (1.0f / kBoxQ), qsz = sz_f * (1.0f / kBoxQ);
-    // cells more than kr (kz along z) away are farther than Rg: the gap to
-    // cell +-d is at least (d - 1) s, and (kr - 1) s > Rg is impossible for
-    // kr = floor(Rg / s) + 1 (a relative margin covers the FP32 rounding of
-    // the quotient).  The bound is the same on both sides and depends on i
-    // only through max(h_i, hnb), so that lanes whose particles share a cell
-    // keep walking its stencil in step.
-    // (a stencil of at most 2 cells keeps its compile-time bounds)
-    const int kr = K <= 2 ? K : min(K, (int)(Rg * P->inv_s_f * (1.0f + 1.0f / 1024.0f)) + 1);
-    const int kz = ZW ? 0 : (K <= 2 ? K : min(K, (int)(Rg * P->inv_sz_f * (1.0f + 1.0f / 1024.0f)) + 1));
+    const float xi = fmaf((float)cx, s_f, ri.x);
+    const float xs = xi * P->inv_s_f;
+    const int xlo = max(cx - kx, 0), xhi = min(cx + kx, ncx - 1);
+    const int ylo = max(-kx, -cy), yhi = min(kx, ncy - 1 - cy);
     const int nz = ZW ? ncz : 2 * kz + 1;
+    // every offset has a stencil code (the usual case)
+    const bool coded = kx <= 2 && (ZW ? P->zmode && ncz <= 5 : kz <= 2);
     for (int iz = 0; iz < nz; iz++) {
         int czj, zd;
-        float zsh, gz2;
-        // raw distance from i to the near z face of the plane (-big: the own plane)
-        float gzr = -1e30f;
-        uint32_t zshift = 20;
+        float zsh, gz2 = 0.0f;
         if (!ZW) {
             const int dcz = iz - kz;
             czj = cz + dcz;
             if (czj < 0) czj += ncz;
             else if (czj >= ncz) czj -= ncz;
             zsh = (float)dcz * sz_f;
-            if (dcz != 0) gzr = dcz > 0 ? (float)dcz * sz_f - ri.z : ri.z - (float)(dcz + 1) * sz_f;
-            zshift = dcz > 0 ? 20u : 25u;
-            const float gg = fmaxf(gzr, 0.0f);
-            gz2 = gg * gg;
+            const float gz = fmaxf(dcz > 0 ? zsh - ri.z : (dcz < 0 ? ri.z - (zsh + sz_f) : 0.0f), 0.0f);
+            gz2 = gz * gz;
+            if (gz2 >= Rg2) continue;
             zd = dcz + 2;
         } else {
             czj = cz + iz;
             if (czj >= ncz) czj -= ncz;
             zsh = (float)iz * sz_f;
-            gz2 = 0.0f;
-            zd = iz;
+            zd = P->zmode ? iz : 5;
         }
-        if (gz2 >= Rg2) continue;
         const float zo = ri.z - zsh;
-        for (int dcy = -kr; dcy <= kr; dcy++) {
-            const int cyj = cy + dcy;
-            if ((unsigned)cyj >= (unsigned)ncy) continue;
-            const float gyr = dcy > 0 ? (float)dcy * s_f - ri.y : (dcy < 0 ? ri.y - (float)(dcy + 1) * s_f : -1e30f);
-            const uint32_t yshift = dcy > 0 ? 10u : 15u;
-            const float gy = fmaxf(gyr, 0.0f);
-            const float gzy2 = fmaf(gy, gy, gz2);
-            if (gzy2 >= Rg2) continue;
-            const float yo = ri.y - (float)dcy * s_f;
-            const uint32_t lrow = cbase + ((uint32_t)czj * (uint32_t)ncy + (uint32_t)cyj) * (uint32_t)ncx + (uint32_t)cx;
-            const uint32_t kkrow = (uint32_t)(2 + 5 * (dcy + 2) + 25 * zd);
-            // a K = 3 stencil reaches cells 3 away, which have no stencil code
-            const bool rowcode = K <= 2 || (dcy >= -2 && dcy <= 2 && zd >= 0 && zd <= 4);
-            // one copy of the candidate loop for all x offsets (code size)
+        const uint32_t lplane = cbase + (uint32_t)czj * (uint32_t)ncy * (uint32_t)ncx;
+        for (int dcy = ylo; dcy <= yhi; dcy++) {
+            const float ysh = (float)dcy * s_f;
+            const float gy = fmaxf(dcy > 0 ? ysh - ri.y : (dcy < 0 ? ri.y - (ysh + s_f) : 0.0f), 0.0f);
+            const float rem2 = Rg2 - fmaf(gy, gy, gz2);
+            if (!(rem2 > 0.0f)) continue;
+            // the chord, in cells (Rg's margins cover the rounding and the
+            // FP32 cell assignment)
+            const float half = __fsqrt_rn(rem2) * P->inv_s_f;
+            const int x0 = max((int)floorf(xs - half), xlo), x1 = min((int)floorf(xs + half), xhi);
+            if (x0 > x1) continue;
+            const uint32_t lrow = lplane + (uint32_t)(cy + dcy) * (uint32_t)ncx;
+            const uint32_t kb = a.g.row[lrow + (uint32_t)x0].x, ke = a.g.row[lrow + (uint32_t)x1].y;
+            const float yo = ri.y - ysh;
+            const bool rowcode = (uint32_t)(dcy + 2) <= 4u && (uint32_t)zd <= 4u;
+            // row_id + add: the column word where the code exists
+            const uint32_t add = (uint32_t)(2 + 5 * (dcy + 2) + 25 * zd - cx) << kColBits;
+            // kGroup candidates per iteration: their loads are in flight
+            // together (the row copy is padded past its end, so a group may
+            // read past the run; those slots are masked)
 #pragma unroll 1
-            for (int dcx = -kr; dcx <= kr; dcx++) {
-                if ((unsigned)(cx + dcx) >= (unsigned)ncx) continue;
-                const float gxr = dcx > 0 ? (float)dcx * s_f - ri.x : (dcx < 0 ? ri.x - (float)(dcx + 1) * s_f : -1e30f);
-                const float gx = fmaxf(gxr, 0.0f);
-                const float d2 = fmaf(gx, gx, gzy2);
-                if (d2 >= Rg2) continue;
-                const uint32_t lin = lrow + (uint32_t)dcx;
-                const uint4 cr = a.g.cell[lin];
-                const uint2 se = make_uint2(cr.x, cr.y);
-                if (se.x >= se.y) continue;
-                const float R = fmaxf(hf, __uint_as_float(cr.z)) * Rc + slack;
-                if (tight_gap2(cr.w, gxr, dcx > 0 ? 0u : 5u, gyr, yshift, gzr, zshift, qs, qsz) >= R * R) continue;
-                const float xo = ri.x - (float)dcx * s_f;
-                // offsets of up to 2 cells have a stencil code
-                const uint32_t kk = (rowcode && dcx >= -2 && dcx <= 2 ? kkrow + (uint32_t)dcx : kFarCode) << kColBits;
-                // kGroup candidates per iteration: their gathers are in flight
-                // together (the record array has kGroup padding entries, so a
-                // group may read past the cell; those slots are masked)
-                for (uint32_t jb = se.x; jb < se.y; jb += kGroup) {
-                    const float4* qp = a.r4 + jb;
-                    float4 q[kGroup];
+            for (uint32_t k = kb; k < ke; k += kGroup) {
+                const float4* qp = a.g.row_rec + k;
+                const uint32_t* ip = a.g.row_id + k;
+                float4 q[kGroup];
+                uint32_t id[kGroup];
 #pragma unroll
-                    for (int u = 0; u < kGroup; u++) q[u] = qp[u];
-                    const uint32_t rem = se.y - jb;
-                    float r2[kGroup], T[kGroup];
-                    unsigned near = 0;
+                for (int u = 0; u < kGroup; u++) q[u] = qp[u];
 #pragma unroll
-                    for (int u = 0; u < kGroup; u++) {
-                        const float dx = xo - q[u].x, dy = yo - q[u].y;
-                        float dz = zo - q[u].z;
-                        if (ZW) dz = fmaf(-lz_f, rintf(dz * inv_lz), dz);
-                        r2[u] = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                        T[u] = fmaxf(Ti, q[u].w);
-                        if ((uint32_t)u < rem && r2[u] <= T[u] * fhi) near |= 1u << u;
-                    }
-                    if (!near) continue;
-                    const uint32_t c0 = row.mark();
+                for (int u = 0; u < kGroup; u++) id[u] = ip[u];
+                const uint32_t rem = ke - k;
+                float r2[kGroup], T[kGroup];
+                unsigned near = 0;
 #pragma unroll
-                    for (int u = 0; u < kGroup; u++) {
-                        if (!(near & (1u << u))) continue;
-                        const uint32_t j = jb + (uint32_t)u;
-                        if (j == i32) continue;
-                        row.decide(a, P, i, j, r2[u], Ti, T[u], flo, fhi, j | kk);
-                    }
-                    row.group_end(c0);
+                for (int u = 0; u < kGroup; u++) {
+                    const float dx = xi - q[u].x, dy = yo - q[u].y;
+                    float dz = zo - q[u].z;
+                    if (ZW) dz = fmaf(-lz_f, rintf(dz * inv_lz), dz);
+                    r2[u] = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                    T[u] = fmaxf(Ti, q[u].w);
+                    if ((uint32_t)u < rem && r2[u] <= T[u] * fhi) near |= 1u << u;
                 }
+                if (!near) continue;
+                const uint32_t c0 = row.mark();
+#pragma unroll
+                for (int u = 0; u < kGroup; u++) {
+                    if (!(near & (1u << u))) continue;
+                    const uint32_t j = id[u] & kColMask;
+                    if (j == i32) continue;
+                    uint32_t w = id[u] + add;
+                    if (!coded && !(rowcode && (id[u] >> kColBits) - (uint32_t)(cx - 2) <= 4u)) w = j | (kFarCode << kColBits);
+                    row.decide(a, P, i, j, r2[u], Ti, T[u], flo, fhi, w);
+                }
+                row.group_end(c0);
             }
         }
     }
 }
 
-// ---- big i, small j: the fine cells within 2 h_i of i ---------------------
-// (rows pass by value through the out-of-line walks, so that the caller's
-// row stays in registers).  Cells are pruned as in walk_small, against their
-// tight boxes, and candidates are tested kGroup at a time.
-template <class S>
-__device__ __noinline__ S walk_big_fine(const NbArgs& a, const PatchDev* P, int64_t i, S row)
+// extents and search radius of walk_rows for particles of h or less in cell
+// cc: small ones reach K cells and no farther than 2 max(h, hnb), hnb the
+// largest h around the cell; big ones 2 max(h, h_s)
+struct RowReach {
+    int kx, kz;
+    float Rg2;
+    bool zw;
+};
+
+__device__ __forceinline__ RowReach row_reach(const NbArgs& a, const PatchDev* P, uint32_t cc, float h, bool big)
 {
-    const float s_f = P->s_f, sz_f = P->sz_f, lz_f = P->lz_f, inv_lz = 1.0f / P->lz_f;
-    const int ncx = P->ncx, ncy = P->ncy, ncz = P->ncz;
-    const uint32_t cbase = (uint32_t)P->cell_base;
-    const float4 ri = a.r4[i];
-    const uint32_t cc = a.g.cellxyz[i];
-    const int cx = cc & 255, cy = (cc >> 8) & 255, cz = cc >> 16;
-    const float hf = (float)a.h[i];
-    const float Ti = ri.w;
-    const float slack = (1.0f / 4096.0f) * s_f;
-    const float Rc = 2.0f * (1.0f + 1.0f / 512.0f);
-    const float Rg = fmaxf(hf, P->hs_f) * Rc + slack;
-    const float Rg2 = Rg * Rg;
-    const float qs = s_f * (1.0f / kBoxQ), qsz = sz_f * (1.0f / kBoxQ);
-    const int Kb = min((int)ceilf(Rg / s_f), kMaxCellsAxis);
-    const int Kz = min((int)ceilf(Rg / sz_f), kMaxCellsAxis);
+    const float s_f = P->s_f;
+    float hr = P->hs_f;
+    if (!big) hr = a.g.hnb[(uint32_t)P->cell_base + ((cc >> 16) * (uint32_t)P->ncy + ((cc >> 8) & 255u)) * (uint32_t)P->ncx + (cc & 255u)];
+    const float Rg = 2.0f * fmaxf(h, hr) * (1.0f + 1.0f / 512.0f) + (1.0f / 4096.0f) * s_f;
+    // the gap to cell +-d is at least (d - 1) s, and (k - 1) s > Rg is
+    // impossible for k = floor(Rg / s) + 1 (a relative margin covers the FP32
+    // rounding of the quotient)
+    const int kmax = big ? kMaxCellsAxis : P->K;
+    RowReach R;
+    R.Rg2 = Rg * Rg;
+    R.kx = min((int)(Rg * P->inv_s_f * (1.0f + 1.0f / 1024.0f)) + 1, kmax);
+    R.kz = min((int)(Rg * P->inv_sz_f * (1.0f + 1.0f / 1024.0f)) + 1, kmax);
     // a z block longer than the period: every z cell once, minimum image in FP32
-    const bool zw = P->zmode != 0 || 2 * Kz + 1 > ncz;
-    const float tol = guard_tol(s_f / hf, max(Kb, zw ? ncz : Kz));
-    const float flo = 1.0f - tol, fhi = 1.0f + tol;
-    const int nz = zw ? ncz : 2 * Kz + 1;
-    for (int iz = 0; iz < nz; iz++) {
-        int czj, dcz;
-        float gz2 = 0.0f;
-        // raw distance from i to the near z face of the plane (-big: every z
-        // cell visited, or the own plane)
-        float gzr = -1e30f;
-        uint32_t zshift = 20;
-        if (!zw) {
-            dcz = iz - Kz;
-            czj = ((cz + dcz) % ncz + ncz) % ncz;
-            if (dcz != 0) gzr = dcz > 0 ? (float)dcz * sz_f - ri.z : ri.z - (float)(dcz + 1) * sz_f;
-            zshift = dcz > 0 ? 20u : 25u;
-            const float gg = fmaxf(gzr, 0.0f);
-            gz2 = gg * gg;
-            if (gz2 >= Rg2) continue;
-        } else {
-            dcz = iz;
-            czj = cz + iz;
-            if (czj >= ncz) czj -= ncz;
-        }
-        const float zo = ri.z - (float)dcz * sz_f;
-        for (int dcy = -Kb; dcy <= Kb; dcy++) {
-            const int cyj = cy + dcy;
-            if ((unsigned)cyj >= (unsigned)ncy) continue;
-            const float gyr = dcy > 0 ? (float)dcy * s_f - ri.y : (dcy < 0 ? ri.y - (float)(dcy + 1) * s_f : -1e30f);
-            const uint32_t yshift = dcy > 0 ? 10u : 15u;
-            const float gy = fmaxf(gyr, 0.0f);
-            const float gzy2 = fmaf(gy, gy, gz2);
-            if (gzy2 >= Rg2) continue;
-            const float yo = ri.y - (float)dcy * s_f;
-            const uint32_t lrow = cbase + ((uint32_t)czj * (uint32_t)ncy + (uint32_t)cyj) * (uint32_t)ncx;
-#pragma unroll 1
-            for (int dcx = -Kb; dcx <= Kb; dcx++) {
-                const int cxj = cx + dcx;
-                if ((unsigned)cxj >= (unsigned)ncx) continue;
-                const float gxr = dcx > 0 ? (float)dcx * s_f - ri.x : (dcx < 0 ? ri.x - (float)(dcx + 1) * s_f : -1e30f);
-                const float gx = fmaxf(gxr, 0.0f);
-                const float d2 = fmaf(gx, gx, gzy2);
-                if (d2 >= Rg2) continue;
-                const uint4 cr = a.g.cell[lrow + (uint32_t)cxj];
-                const uint2 se = make_uint2(cr.x, cr.y);
-                if (se.x >= se.y) continue;
-                const float R = fmaxf(hf, __uint_as_float(cr.z)) * Rc + slack;
-                if (tight_gap2(cr.w, gxr, dcx > 0 ? 0u : 5u, gyr, yshift, gzr, zshift, qs, qsz) >= R * R) continue;
-                const float xo = ri.x - (float)dcx * s_f;
-                const uint32_t kk = stencil_code(P, dcx, dcy, dcz, !zw) << kColBits;
-                // kGroup candidates at a time (the record array is padded past
-                // its end; slots past the cell are masked)
-                for (uint32_t jb = se.x; jb < se.y; jb += kGroup) {
-                    const float4* qp = a.r4 + jb;
-                    float4 q[kGroup];
-#pragma unroll
-                    for (int u = 0; u < kGroup; u++) q[u] = qp[u];
-                    const uint32_t rem = se.y - jb;
-                    float r2[kGroup], T[kGroup];
-                    unsigned near = 0;
-#pragma unroll
-                    for (int u = 0; u < kGroup; u++) {
-                        const float dx = xo - q[u].x, dy = yo - q[u].y;
-                        float dz = zo - q[u].z;
-                        if (zw) dz = fmaf(-lz_f, rintf(dz * inv_lz), dz);
-                        r2[u] = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                        T[u] = fmaxf(Ti, q[u].w);
-                        if ((uint32_t)u < rem && r2[u] <= T[u] * fhi) near |= 1u << u;
-                    }
-                    if (!near) continue;
-                    const uint32_t c0 = row.mark();
-#pragma unroll
-                    for (int u = 0; u < kGroup; u++) {
-                        if (!(near & (1u << u))) continue;
-                        const uint32_t j = jb + (uint32_t)u;
-                        row.decide(a, P, i, j, r2[u], Ti, T[u], flo, fhi, j | kk);
-                    }
-                    row.group_end(c0);
-                }
-            }
-        }
-    }
-    return row;
+    R.zw = P->zmode != 0 || 2 * R.kz + 1 > P->ncz;
+    return R;
 }
 
 // ---- any i, big j: the coarse cells around i's coarse cell -----------------
@@ -534,15 +438,12 @@ __device__ __noinline__ S walk_coarse(const NbArgs& a, const PatchDev* P, int64_
 }
 
 // the whole search for particle i
-template <class S, int K>
+template <class S>
 __device__ __forceinline__ void walk_all(const NbArgs& a, const PatchDev* P, int64_t i, bool big, S& row)
 {
-    if (!big) {
-        if (P->zmode) walk_small<S, K, 1>(a, P, i, row);
-        else walk_small<S, K, 0>(a, P, i, row);
-    } else {
-        row = walk_big_fine<S>(a, P, i, row);
-    }
+    const RowReach R = row_reach(a, P, a.g.cellxyz[i], (float)a.h[i], big);
+    if (R.zw) walk_rows<S, 1>(a, P, i, R.kx, R.kz, R.Rg2, row);
+    else walk_rows<S, 0>(a, P, i, R.kx, R.kz, R.Rg2, row);
     if (P->nbig > 0) row = walk_coarse<S>(a, P, i, row);
 }
 

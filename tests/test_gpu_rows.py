@@ -1,0 +1,63 @@
+"""The search over rows of cells where its runs can go wrong: rows of 128
+cells (x far from the grid's origin), particles on cell faces, cells of many
+particles, rows of one cell, and few z cells -- lists and n_i against the
+oracle, bit for bit."""
+import numpy as np
+import pytest
+
+from gpu_common import lists_to_original
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    from paper_1905_03344_gb300 import binding, build
+    build.build()
+    binding.lib()
+    return binding
+
+
+def _cloud(kind):
+    rng = np.random.default_rng(11)
+    n = 6000
+    z = rng.uniform(-0.5, 0.5, n)
+    if kind == "long_x":         # 128 cells along x, few along y
+        x, y, h = rng.uniform(0.0, 12.0, n), rng.uniform(-0.1, 0.1, n), rng.uniform(0.03, 0.045, n)
+    elif kind == "long_y":       # rows of few cells
+        x, y, h = rng.uniform(-0.1, 0.1, n), rng.uniform(0.0, 12.0, n), rng.uniform(0.03, 0.045, n)
+    elif kind == "faces":        # coordinates on a lattice of multiples of the cell edge and of ties at 2 h
+        k = rng.integers(0, 24, (3, n))
+        x, y, z = k[0] / 32.0, k[1] / 32.0, (k[2] % 16) / 16.0 - 0.5
+        h = np.where(rng.random(n) < 0.5, 1.0 / 32.0, 3.0 / 64.0)
+    elif kind == "clump":        # a cell of several hundred particles among sparse ones
+        x, y = rng.uniform(-1.0, 1.0, n), rng.uniform(-1.0, 1.0, n)
+        x[:400], y[:400], z[:400] = (rng.normal(c, 0.004, 400) for c in (0.2, -0.3, 0.1))
+        h = rng.uniform(0.05, 0.07, n)
+    elif kind == "big_reach":    # a few particles whose radius spans many rows and the z period
+        x, y = rng.uniform(-0.5, 0.5, n), rng.uniform(-0.5, 0.5, n)
+        h = rng.uniform(0.03, 0.04, n)
+        h[::97] = rng.uniform(0.15, 0.3, len(h[::97]))
+    else:                        # few_z: h so large that every z cell is visited
+        x, y, h = rng.uniform(-2.0, 2.0, n), rng.uniform(-2.0, 2.0, n), rng.uniform(0.14, 0.17, n)
+    v = np.zeros(n)
+    return {"x": x, "y": y, "z": z, "vx": v, "vy": v, "vz": v, "m": np.full(n, 1.0 / n), "h": h, "u": np.ones(n)}
+
+
+@pytest.mark.parametrize("cf", [0.0, 0.4, 1.0])
+@pytest.mark.parametrize("kind", ["long_x", "long_y", "faces", "clump", "big_reach", "few_z"])
+def test_rows(B, orc, kind, cf):
+    f = _cloud(kind)
+    n = len(f["x"])
+    sim = B.SPH(n, cell_factor=cf, max_pairs=800 * n)
+    sim.set_particles(f)
+    for _ in range(2):           # rows counted first, then reserved from hints
+        sim.find_neighbors()
+        off, col, perm = sim.neighbors()
+        o, c = lists_to_original(off, col, perm, n)
+        nb = orc.neighbors(f["x"], f["y"], f["z"], f["h"], 1.0)
+        assert np.array_equal(o, nb.off) and np.array_equal(c, nb.col)
+        assert np.array_equal(sim.field("nown").astype(np.int64), nb.nown)
+    sim.close()
