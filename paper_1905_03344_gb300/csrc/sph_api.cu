@@ -126,7 +126,7 @@ struct sph_ctx {
     uint16_t* patch_of = nullptr;
     uint32_t *keys = nullptr, *vals = nullptr, *keys_alt = nullptr, *vals_alt = nullptr;
     float* hnb_tmp = nullptr;   // one float per cell: the x-y pass of the grid's hnb
-    uint32_t *hist = nullptr, *scan32 = nullptr;
+    uint32_t* hist = nullptr;      // the radix sort's work words
     Grid grid{};
     Recs rec{};
     Fp64 f64{};
@@ -381,6 +381,9 @@ StepArgs step_args(sph_ctx* ctx)
     return a;
 }
 
+// the radix sort's buffers, with the sorted values in vals
+RadixSort radix_of(sph_ctx* ctx, uint32_t* vals) { return RadixSort{ctx->keys, vals, ctx->keys_alt, ctx->vals_alt, ctx->hist}; }
+
 // ---- the phases (asynchronous, no host synchronisation) -----------------------
 // superset: the sort and cells of a candidate superset (reused lists): the
 // search h of every particle grown by its skin, gathered into skinref.h0;
@@ -397,7 +400,7 @@ void enqueue_sort(sph_ctx* ctx, bool superset = false)
     }
     {
         Phase p(ctx, SPH_PHASE_BBOX);
-        ctx->launches += launch_reset_red(L, ctx->npatch, ctx->red);
+        ctx->launches += launch_reset_red(L, ctx->npatch, ctx->red, ctx->hist, (int64_t)radix_work_words(ctx->n));
         ctx->launches += launch_reduce_bbox(L, s, ctx->items, ctx->nitems, ctx->red);
         ctx->launches += launch_h_hist(L, s, ctx->items, ctx->nitems, ctx->red);
         ctx->launches += launch_grid_params(L, ctx->npatch, ctx->red, ctx->pd, ctx->cell_factor, ctx->status,
@@ -405,12 +408,11 @@ void enqueue_sort(sph_ctx* ctx, bool superset = false)
     }
     {
         Phase p(ctx, SPH_PHASE_KEYS);
-        ctx->launches += launch_keys(L, ctx->n, s, ctx->patch_of, ctx->pd, ctx->keys, ctx->vals);
+        ctx->launches += launch_keys(L, ctx->n, s, ctx->patch_of, ctx->pd, radix_of(ctx, ctx->vals), ctx->radix_passes);
     }
     {
         Phase p(ctx, SPH_PHASE_SORT);
-        ctx->launches += launch_radix_sort(L, ctx->n, ctx->radix_passes, ctx->keys, ctx->vals, ctx->keys_alt,
-                                           ctx->vals_alt, ctx->hist, ctx->scan32);
+        ctx->launches += launch_radix_sort(L, ctx->n, ctx->radix_passes, radix_of(ctx, ctx->vals), ctx->status);
     }
     {
         Phase p(ctx, SPH_PHASE_GATHER);
@@ -421,6 +423,7 @@ void enqueue_sort(sph_ctx* ctx, bool superset = false)
                                        ctx->f64, ctx->mixed,
                                        superset ? RowHint{ctx->cnt_s, ctx->hint_ok_s, ctx->rowcap}
                                                 : RowHint{ctx->cnt, ctx->hint_ok, ctx->rowcap},
+                                       ctx->status,
                                        superset ? ctx->hsearch_pre : nullptr, superset ? ctx->skinref.h0 : nullptr);
         ctx->launches += launch_cell_tables(L, ctx->npatch, ctx->pd, ctx->grid, ctx->rec.r4, stencil_k(ctx->cell_factor),
                                             ctx->hnb_tmp, ctx->cf_vote);
@@ -452,8 +455,7 @@ void enqueue_lists(sph_ctx* ctx)
 void enqueue_bins(sph_ctx* ctx)
 {
     if (ctx->bins_valid) return;
-    ctx->launches += launch_pair_bins(launch_of(ctx), ctx->n, ctx->cnt, ctx->keys, ctx->bin_order, ctx->keys_alt,
-                                      ctx->vals_alt, ctx->hist, ctx->scan32, ctx->bin_bounds);
+    ctx->launches += launch_pair_bins(launch_of(ctx), ctx->n, ctx->cnt, radix_of(ctx, ctx->bin_order), ctx->bin_bounds, ctx->status);
     ctx->bins_valid = true;
 }
 
@@ -880,8 +882,7 @@ sph_status sph_create(const sph_config* cfg_in, sph_ctx** out)
     ok = ok && dalloc(ctx, ctx->patch_of, N);
     ok = ok && dalloc(ctx, ctx->keys, N) && dalloc(ctx, ctx->vals, N) && dalloc(ctx, ctx->keys_alt, N) &&
          dalloc(ctx, ctx->vals_alt, N);
-    const size_t hw = radix_hist_words(ctx->cap_n);
-    ok = ok && dalloc(ctx, ctx->hist, hw) && dalloc(ctx, ctx->scan32, (size_t)scan_tmp_words((int64_t)hw));
+    ok = ok && dalloc(ctx, ctx->hist, radix_work_capacity(ctx->cap_n));
     uint4* cellrec = nullptr;
     uint32_t* cellxyz = nullptr;
     ok = ok && dalloc(ctx, cellrec, (size_t)ctx->cap_cells) && dalloc(ctx, cellxyz, N) &&

@@ -190,12 +190,24 @@ int launch_reduce_bbox(const Launch& L, const State& s, const WorkItem* items, i
 int launch_h_hist(const Launch& L, const State& s, const WorkItem* items, int nitems, PatchRed* red);
 int launch_grid_params(const Launch& L, int npatch, const PatchRed* red, PatchDev* pd,
                        double cell_factor, int* status, unsigned long long* vote);
-int launch_keys(const Launch& L, int64_t n, const State& s, const uint16_t* patch_of,
-                PatchDev* pd, uint32_t* keys, uint32_t* vals);
-// LSD radix sort of (keys, vals); result in (keys, vals); uses alternates.
-int launch_radix_sort(const Launch& L, int64_t n, int passes, uint32_t* keys, uint32_t* vals,
-                      uint32_t* keys_alt, uint32_t* vals_alt, uint32_t* hist, uint32_t* scan_tmp);
-size_t radix_hist_words(int64_t n);
+// the buffers of the radix sort: the sorted pairs end up in (keys, vals); work
+// holds the digit counts of every pass, the passes' tickets and the tiles'
+// look-back words, all cleared before the keys are made
+constexpr int kRsMaxPasses = 4;
+struct RadixSort {
+    uint32_t *keys, *vals, *keys_alt, *vals_alt, *work;
+    // where the unsorted pairs go, for an odd or even number of passes
+    void input(int passes, uint32_t*& k, uint32_t*& v) const
+    {
+        k = passes & 1 ? keys_alt : keys;
+        v = passes & 1 ? vals_alt : vals;
+    }
+};
+size_t radix_work_words(int64_t n);       // words of work a sort of n uses
+size_t radix_work_capacity(int64_t cap);  // ... of at most cap
+int launch_keys(const Launch& L, int64_t n, const State& s, const uint16_t* patch_of, PatchDev* pd, const RadixSort& rs, int passes);
+// LSD radix sort of 8 * passes key bits
+int launch_radix_sort(const Launch& L, int64_t n, int passes, const RadixSort& rs, int* status);
 // Row-length hints for the list pool: the previous lists' row lengths,
 // carried into the new sorted order by the gather.  Only a hint: the list
 // kernel reserves from it and repairs rows that outgrow their reservation.
@@ -211,7 +223,7 @@ struct RowHint {
 int launch_gather(const Launch& L, int64_t n, const uint32_t* skeys, const uint32_t* svals,
                   const State& src, const State& dst, const uint32_t* perm_src,
                   uint32_t* perm_dst, const PatchDev* pd, const Grid& g, const Recs& r,
-                  const Fp64& f, int mixed, const RowHint& hint, const double* hsearch = nullptr,
+                  const Fp64& f, int mixed, const RowHint& hint, const int* status, const double* hsearch = nullptr,
                   double* hsearch_out = nullptr);
 // the FP32 records of the current state in the current sorted order, on the
 // grid of the last sort (what the gather writes, with the unscaled h)
@@ -295,8 +307,8 @@ __host__ __device__ __forceinline__ int octave_tpp(int o, int w)
 }
 // order = the particles stably sorted by octave (sorted order kept inside
 // each octave), bounds[o] = first position of octave o, bounds[kPairOctaves] = n
-int launch_pair_bins(const Launch& L, int64_t n, const uint32_t* cnt, uint32_t* keys, uint32_t* order,
-                     uint32_t* keys_alt, uint32_t* vals_alt, uint32_t* hist, uint32_t* scan_tmp, uint32_t* bounds);
+// (rs.vals is the order)
+int launch_pair_bins(const Launch& L, int64_t n, const uint32_t* cnt, const RadixSort& rs, uint32_t* bounds, int* status);
 // the sums over row-length bins with 2^w words per lane (one launch per
 // distinct lanes-per-particle value)
 int launch_density_binned(const Launch& L, PairArgs a, int w, int mixed);
@@ -352,6 +364,6 @@ int launch_unpermute_f32(const Launch& L, int64_t n, const float* src, int strid
 int launch_unpermute_u32(const Launch& L, int64_t n, const uint32_t* src, const uint32_t* perm,
                          double* dst);
 int launch_validate(const Launch& L, int64_t n, const State& s, int* status);
-int launch_reset_red(const Launch& L, int npatch, PatchRed* red);
+int launch_reset_red(const Launch& L, int npatch, PatchRed* red, uint32_t* zero, int64_t words);
 
 }  // namespace sphg

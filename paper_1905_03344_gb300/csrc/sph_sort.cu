@@ -4,7 +4,7 @@
 // atomics), grid parameters, Morton cell keys, a stable LSD radix sort of
 // (key, slot), and the gather of every particle field into the sorted order,
 // which also writes the cell table and the FP32 cell-relative records.
-// Also the device-wide exclusive scan used by the radix sort and the CSR.
+// Also the device-wide exclusive scan used by the CSR.
 #include "sph_internal.cuh"
 
 namespace sphg {
@@ -87,9 +87,11 @@ int launch_reduce_bbox(const Launch& L, const State& s, const WorkItem* items, i
     return 1;
 }
 
-__global__ void k_reset_red(int npatch, PatchRed* red)
+// (and clears the radix sort's counters)
+__global__ void k_reset_red(int npatch, PatchRed* red, uint32_t* zero, int64_t words)
 {
     int p = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int64_t k = p; k < words; k += (int64_t)gridDim.x * blockDim.x) zero[k] = 0u;
     if (p < npatch) {
         red[p].xmin = ~0ull;
         red[p].ymin = ~0ull;
@@ -143,9 +145,9 @@ int launch_h_hist(const Launch& L, const State& s, const WorkItem* items, int ni
     return 1;
 }
 
-int launch_reset_red(const Launch& L, int npatch, PatchRed* red)
+int launch_reset_red(const Launch& L, int npatch, PatchRed* red, uint32_t* zero, int64_t words)
 {
-    k_reset_red<<<(npatch + 255) / 256, 256, 0, L.stream>>>(npatch, red);
+    k_reset_red<<<blocks_for(words > npatch ? words : npatch, 256, L.sms, 8), 256, 0, L.stream>>>(npatch, red, zero, words);
     return 1;
 }
 
@@ -296,9 +298,27 @@ int launch_grid_params(const Launch& L, int npatch, const PatchRed* red, PatchDe
 // cell coordinates in FP32 from the FP64 offset to the grid origin (error <
 // 1e-4 cell, inside the margin).  Counts the big particles of each patch.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_keys(int64_t n, State s, const uint16_t* patch_of,
-                                              PatchDev* pd, uint32_t* keys, uint32_t* vals)
+// Also counts the digits of every pass of the radix sort (hist, kRsMaxPasses
+// x 256).
+__device__ __forceinline__ void count_digits(uint32_t key, int passes, uint32_t (*sh)[256])
 {
+    for (int p = 0; p < passes; p++) atomicAdd(&sh[p][(key >> (8 * p)) & 255u], 1u);
+}
+
+__device__ __forceinline__ void add_digits(int passes, const uint32_t (*sh)[256], uint32_t* hist)
+{
+    for (int k = threadIdx.x; k < passes * 256; k += blockDim.x) {
+        const uint32_t c = (&sh[0][0])[k];
+        if (c) atomicAdd(&hist[k], c);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_keys(int64_t n, State s, const uint16_t* patch_of,
+                                              PatchDev* pd, uint32_t* keys, uint32_t* vals, int passes, uint32_t* hist)
+{
+    __shared__ uint32_t sh[kRsMaxPasses][256];
+    for (int k = threadIdx.x; k < kRsMaxPasses * 256; k += blockDim.x) (&sh[0][0])[k] = 0u;
+    __syncthreads();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int p = patch_of[i];
@@ -317,17 +337,23 @@ __global__ void __launch_bounds__(256) k_keys(int64_t n, State s, const uint16_t
         cx = min(max(cx, 0), P->ncx - 1);
         cy = min(max(cy, 0), P->ncy - 1);
         cz = min(max(cz, 0), P->ncz - 1);
-        keys[i] = ((uint32_t)p << kPatchShift) | ((uint32_t)big << kClassShift) | part1by2((uint32_t)cx) |
-                  (part1by2((uint32_t)cy) << 1) | (part1by2((uint32_t)cz) << 2);
+        const uint32_t key = ((uint32_t)p << kPatchShift) | ((uint32_t)big << kClassShift) | part1by2((uint32_t)cx) |
+                             (part1by2((uint32_t)cy) << 1) | (part1by2((uint32_t)cz) << 2);
+        keys[i] = key;
         vals[i] = (uint32_t)i;
+        count_digits(key, passes, sh);
     }
+    __syncthreads();
+    add_digits(passes, sh, hist);
 }
 
 int launch_keys(const Launch& L, int64_t n, const State& s, const uint16_t* patch_of,
-                PatchDev* pd, uint32_t* keys, uint32_t* vals)
+                PatchDev* pd, const RadixSort& rs, int passes)
 {
     if (n <= 0) return 0;
-    k_keys<<<blocks_for(n, 256, L.sms, 16), 256, 0, L.stream>>>(n, s, patch_of, pd, keys, vals);
+    uint32_t *k, *v;
+    rs.input(passes, k, v);
+    k_keys<<<blocks_for(n, 256, L.sms, 8), 256, 0, L.stream>>>(n, s, patch_of, pd, k, v, passes, rs.work);
     return 1;
 }
 
@@ -441,151 +467,168 @@ int launch_scan_u32_to_u64(const Launch& L, int64_t n, const uint32_t* in, uint6
     return 3;
 }
 
-static int scan_u32(const Launch& L, int64_t n, const uint32_t* in, uint32_t* out, uint32_t* tmp)
-{
-    const int64_t nb = (n + kScanTile - 1) / kScanTile;
-    k_scan_reduce<uint32_t, uint32_t><<<(unsigned)nb, kScanThreads, 0, L.stream>>>(in, n, tmp);
-    k_scan_spine<uint32_t><<<1, 1024, 0, L.stream>>>(tmp, nb);
-    k_scan_down<uint32_t, uint32_t><<<(unsigned)nb, kScanThreads, 0, L.stream>>>(in, n, tmp, out, 0);
-    return 3;
-}
-
 // ---------------------------------------------------------------------------
-// Stable LSD radix sort, 8-bit digits.  Per pass: a digit histogram per
-// tile of 4096 keys (digit-major), an exclusive scan of the histograms, and a
-// scatter that ranks keys stably inside the tile (warp match + per-warp
-// counters, warps in tile order), stages the tile in shared memory in digit
-// order and writes each digit run contiguously.
+// Stable LSD radix sort, 8-bit digits, one kernel per pass.  The digits of
+// all passes are counted while the keys are made.  A block takes the next
+// tile (in the order of a ticket), ranks its keys stably (warp match +
+// per-warp counters, warps in tile order), publishes the tile's digit counts
+// and looks back over the tiles before it for their sum, each of which is
+// published as its own counts first and as the sum up to it once that is
+// known; then it stages the tile in shared memory in digit order and writes
+// each digit run contiguously.  A tile only waits for tiles with earlier
+// tickets, which never wait for it.  The wait is bounded all the same; a
+// block whose wait runs out flags it and writes nothing out of range.
+//
+// A pass is bound by the latency of a tile's chain (load, rank, look back,
+// stage, write), so by how many tiles are resident: five blocks on an SM with
+// 12 keys a thread, 48 registers and 35 KB; 16 keys at 128 registers, two
+// blocks, took 100 us a pass at 8 M where this takes 72, votes per digit bit
+// in place of the match 75, 8 keys 73.  Up to 622,592 keys (four tiles an SM)
+// the tiles have 1024 keys, which keeps more SMs busy.  The pass per digit of
+// a histogram, a three-kernel scan and a scatter (with a copy back after an
+// odd number of passes) that this replaces took 15 launches where this takes
+// 3: 460 -> 216 us at 8 M, 126 -> 51 us at 1 M, 102 -> 21 us at 8000.
 // ---------------------------------------------------------------------------
 constexpr int kRsThreads = 256;
 constexpr int kRsWarps = kRsThreads / 32;
-constexpr int kRsStrips = 16;
-constexpr int kRsTile = kRsWarps * 32 * kRsStrips;  // 4096
+constexpr uint32_t kRsAggregate = 1u << 30, kRsPrefix = 2u << 30, kRsValue = kRsAggregate - 1u;
+constexpr int kRsSpins = 1 << 22;
+constexpr int kRsItems = 12;            // keys a thread takes in the larger tiles
 
-__global__ void __launch_bounds__(kRsThreads) k_rs_hist(const uint32_t* keys, int64_t n, int shift,
-                                                       uint32_t* hist, int ntiles)
+template <int ITEMS>
+__global__ void __launch_bounds__(kRsThreads, ITEMS == 4 ? 6 : 5) k_rs_pass(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
+                                                       int64_t n, int shift, const uint32_t* __restrict__ ghist, uint32_t* ticket,
+                                                       volatile uint32_t* state, uint32_t* kout, uint32_t* vout, int* status)
 {
-    __shared__ uint32_t sh[256];
-    const int lane = threadIdx.x & 31;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        sh[threadIdx.x] = 0;
-        __syncthreads();
-        const int64_t base = (int64_t)tile * kRsTile;
-        for (int k = threadIdx.x; k < kRsTile; k += blockDim.x) {
-            const int64_t i = base + k;
-            const uint32_t d = i < n ? ((keys[i] >> shift) & 255u) : 256u;
-            const unsigned peers = __match_any_sync(0xffffffffu, d);
-            if (d < 256u && lane == __ffs(peers) - 1) atomicAdd(&sh[d], (uint32_t)__popc(peers));
-        }
-        __syncthreads();
-        hist[(int64_t)threadIdx.x * ntiles + tile] = sh[threadIdx.x];
-        __syncthreads();
-    }
-}
-
-__global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const uint32_t* kin, const uint32_t* vin,
-                                                          int64_t n, int shift, const uint32_t* hoff,
-                                                          int ntiles, uint32_t* kout, uint32_t* vout)
-{
-    __shared__ uint32_t s_keys[kRsTile];
-    __shared__ uint32_t s_vals[kRsTile];
+    constexpr int kTile = kRsThreads * ITEMS;
+    __shared__ uint32_t s_keys[kTile];
+    __shared__ uint32_t s_vals[kTile];
     __shared__ uint32_t s_wcnt[kRsWarps][256];
     __shared__ uint32_t s_dstart[256];
     __shared__ uint32_t s_goff[256];
     __shared__ uint32_t s_scan[33];
+    __shared__ uint32_t s_tile;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        for (int k = threadIdx.x; k < kRsWarps * 256; k += blockDim.x) (&s_wcnt[0][0])[k] = 0;
-        __syncthreads();
-        uint32_t kr[kRsStrips], vr[kRsStrips];
-        uint16_t pr[kRsStrips];
-        const int64_t wbase = (int64_t)tile * kRsTile + (int64_t)warp * 32 * kRsStrips;
+    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+    for (int k = threadIdx.x; k < kRsWarps * 256; k += kRsThreads) (&s_wcnt[0][0])[k] = 0;
+    __syncthreads();
+    const int64_t tile = s_tile;
+    const int64_t wbase = tile * kTile + (int64_t)warp * 32 * ITEMS;
+    uint32_t kr[ITEMS], vr[ITEMS];
+    uint16_t pr[ITEMS];
 #pragma unroll
-        for (int t = 0; t < kRsStrips; t++) {
-            const int64_t i = wbase + t * 32 + lane;
-            const bool valid = i < n;
-            const uint32_t key = valid ? kin[i] : 0xffffffffu;
-            const uint32_t val = valid ? vin[i] : 0u;
-            const uint32_t d = valid ? ((key >> shift) & 255u) : 256u;
-            const unsigned peers = __match_any_sync(0xffffffffu, d);
-            const int rank = __popc(peers & ((1u << lane) - 1u));
-            uint32_t before = 0;
-            if (valid) before = s_wcnt[warp][d];
-            __syncwarp();
-            if (valid && lane == __ffs(peers) - 1) s_wcnt[warp][d] = before + (uint32_t)__popc(peers);
-            __syncwarp();
-            kr[t] = key;
-            vr[t] = val;
-            pr[t] = (uint16_t)(before + rank);
-        }
-        __syncthreads();
-        {   // per digit: exclusive offsets of the warps, then digit starts in the tile
-            const int d = threadIdx.x;
-            uint32_t run = 0;
-            for (int w = 0; w < kRsWarps; w++) {
-                uint32_t c = s_wcnt[w][d];
-                s_wcnt[w][d] = run;
-                run += c;
-            }
-            uint32_t tot;
-            s_dstart[d] = block_excl_scan<uint32_t>(run, &tot, s_scan);
-            s_goff[d] = hoff[(int64_t)d * ntiles + tile];
-        }
-        __syncthreads();
+    for (int t = 0; t < ITEMS; t++) {
+        const int64_t i = wbase + t * 32 + lane;
+        kr[t] = i < n ? kin[i] : 0xffffffffu;
+        vr[t] = i < n ? vin[i] : 0u;
+    }
 #pragma unroll
-        for (int t = 0; t < kRsStrips; t++) {
-            const int64_t i = wbase + t * 32 + lane;
-            if (i < n) {
-                const uint32_t d = (kr[t] >> shift) & 255u;
-                const uint32_t lp = s_dstart[d] + s_wcnt[warp][d] + pr[t];
-                s_keys[lp] = kr[t];
-                s_vals[lp] = vr[t];
+    for (int t = 0; t < ITEMS; t++) {
+        const bool valid = wbase + t * 32 + lane < n;
+        const uint32_t d = valid ? ((kr[t] >> shift) & 255u) : 256u;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const int rank = __popc(peers & ((1u << lane) - 1u));
+        uint32_t before = 0;
+        if (valid) before = s_wcnt[warp][d];
+        __syncwarp();
+        if (valid && rank == 0) s_wcnt[warp][d] = before + (uint32_t)__popc(peers);
+        __syncwarp();
+        pr[t] = (uint16_t)(before + rank);
+    }
+    __syncthreads();
+    {   // per digit: exclusive offsets of the warps, digit starts in the tile and in the output
+        const int d = threadIdx.x;
+        uint32_t cnt = 0;
+        for (int w = 0; w < kRsWarps; w++) {
+            const uint32_t c = s_wcnt[w][d];
+            s_wcnt[w][d] = cnt;
+            cnt += c;
+        }
+        volatile uint32_t* mine = state + tile * 256 + d;
+        *mine = cnt | (tile == 0 ? kRsPrefix : kRsAggregate);
+        uint32_t tot;
+        const uint32_t start = block_excl_scan<uint32_t>(cnt, &tot, s_scan);
+        const uint32_t first = block_excl_scan<uint32_t>(ghist[d], &tot, s_scan);
+        // eight tiles back at a time (their loads are in flight together)
+        uint32_t before = 0;
+        int spins = 0;
+        for (int64_t q = tile - 1; q >= 0;) {
+            uint32_t v[8];
+#pragma unroll
+            for (int e = 0; e < 8; e++) v[e] = q - e >= 0 ? state[(q - e) * 256 + d] : 0u + kRsPrefix;
+            int used = 0;
+#pragma unroll
+            for (int e = 0; e < 8; e++)
+                if (used == e && v[e] >= kRsAggregate) {
+                    before += v[e] & kRsValue;
+                    used = v[e] >= kRsPrefix ? 64 : e + 1;
+                }
+            if (used >= 64) break;
+            q -= used;
+            if (used == 0 && ++spins > kRsSpins) {
+                atomicOr(status, kStTimeout);
+                break;
             }
         }
-        __syncthreads();
-        const int64_t rem = n - (int64_t)tile * kRsTile;
-        const int tn = rem < kRsTile ? (int)rem : kRsTile;
-        for (int k = threadIdx.x; k < tn; k += blockDim.x) {
-            const uint32_t key = s_keys[k];
-            const uint32_t d = (key >> shift) & 255u;
-            const uint32_t g = s_goff[d] + ((uint32_t)k - s_dstart[d]);
+        if (tile > 0) *mine = (before + cnt) | kRsPrefix;
+        s_dstart[d] = start;
+        s_goff[d] = first + before - start;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < ITEMS; t++) {
+        if (wbase + t * 32 + lane < n) {
+            const uint32_t d = (kr[t] >> shift) & 255u;
+            const uint32_t lp = s_dstart[d] + s_wcnt[warp][d] + pr[t];
+            s_keys[lp] = kr[t];
+            s_vals[lp] = vr[t];
+        }
+    }
+    __syncthreads();
+    const int64_t rem = n - tile * kTile;
+    const int tn = rem < kTile ? (int)rem : kTile;
+    for (int k = threadIdx.x; k < tn; k += kRsThreads) {
+        const uint32_t key = s_keys[k];
+        const uint32_t g = s_goff[(key >> shift) & 255u] + (uint32_t)k;
+        if (g < (uint32_t)n) {
             kout[g] = key;
             vout[g] = s_vals[k];
         }
-        __syncthreads();
     }
 }
 
-size_t radix_hist_words(int64_t n)
+static int rs_items(int64_t n) { return n <= 608 * 1024 ? 4 : kRsItems; }
+static int64_t rs_tiles(int64_t n) { return (n + rs_items(n) * kRsThreads - 1) / (rs_items(n) * kRsThreads); }
+
+size_t radix_work_words(int64_t n) { return (size_t)kRsMaxPasses * (256 + 16 + 256 * (size_t)rs_tiles(n < 1 ? 1 : n)); }
+
+size_t radix_work_capacity(int64_t cap)
 {
-    int64_t ntiles = (n + kRsTile - 1) / kRsTile;
-    if (ntiles < 1) ntiles = 1;
-    return (size_t)(256 * ntiles);
+    const size_t a = radix_work_words(cap), b = radix_work_words(cap < 608 * 1024 ? cap : 608 * 1024);
+    return a > b ? a : b;
 }
 
-int launch_radix_sort(const Launch& L, int64_t n, int passes, uint32_t* keys, uint32_t* vals,
-                      uint32_t* keys_alt, uint32_t* vals_alt, uint32_t* hist, uint32_t* scan_tmp)
+int launch_radix_sort(const Launch& L, int64_t n, int passes, const RadixSort& rs, int* status)
 {
-    if (n <= 1) return 0;
-    const int ntiles = (int)((n + kRsTile - 1) / kRsTile);
-    const int grid = ntiles < L.sms * 4 ? ntiles : L.sms * 4;
-    const int64_t nh = (int64_t)256 * ntiles;
-    int launches = 0;
-    uint32_t *ki = keys, *vi = vals, *ko = keys_alt, *vo = vals_alt;
+    if (n <= 0) return 0;
+    uint32_t *ki, *vi;
+    rs.input(passes, ki, vi);
+    const int64_t tiles = rs_tiles(n);
+    // the default split of the L1 would keep fewer blocks on an SM
+    cudaFuncSetAttribute(k_rs_pass<4>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    cudaFuncSetAttribute(k_rs_pass<kRsItems>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     for (int ps = 0; ps < passes; ps++) {
-        const int shift = 8 * ps;
-        k_rs_hist<<<grid, kRsThreads, 0, L.stream>>>(ki, n, shift, hist, ntiles);
-        launches += 1 + scan_u32(L, nh, hist, hist, scan_tmp);
-        k_rs_scatter<<<grid, kRsThreads, 0, L.stream>>>(ki, vi, n, shift, hist, ntiles, ko, vo);
-        launches++;
-        uint32_t* t = ki; ki = ko; ko = t;
-        t = vi; vi = vo; vo = t;
+        uint32_t* ko = ki == rs.keys ? rs.keys_alt : rs.keys;
+        uint32_t* vo = vi == rs.vals ? rs.vals_alt : rs.vals;
+        uint32_t* tickets = rs.work + kRsMaxPasses * 256;
+        uint32_t* state = tickets + kRsMaxPasses * 16 + (int64_t)ps * 256 * tiles;
+        const auto kern = rs_items(n) == 4 ? k_rs_pass<4> : k_rs_pass<kRsItems>;
+        kern<<<(unsigned)tiles, kRsThreads, 0, L.stream>>>(ki, vi, n, 8 * ps, rs.work + 256 * ps, tickets + 16 * ps, state, ko, vo,
+                                                           status);
+        ki = ko;
+        vi = vo;
     }
-    if (ki != keys) {   // odd number of passes: copy back
-        cudaMemcpyAsync(keys, ki, (size_t)n * 4, cudaMemcpyDeviceToDevice, L.stream);
-        cudaMemcpyAsync(vals, vi, (size_t)n * 4, cudaMemcpyDeviceToDevice, L.stream);
-    }
-    return launches;
+    return passes;
 }
 
 // ---------------------------------------------------------------------------
@@ -593,42 +636,41 @@ int launch_radix_sort(const Launch& L, int64_t n, int passes, uint32_t* keys, ui
 // one radix pass; the bin starts are the scanned digit offsets of the first
 // tile.
 // ---------------------------------------------------------------------------
-__global__ void k_octave_keys(int64_t n, const uint32_t* cnt, uint32_t* keys, uint32_t* vals)
+__global__ void __launch_bounds__(256) k_octave_keys(int64_t n, const uint32_t* cnt, uint32_t* keys, uint32_t* vals, uint32_t* hist)
 {
+    __shared__ uint32_t sh[1][256];
+    sh[0][threadIdx.x] = 0u;
+    __syncthreads();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t c = cnt[i];
         // 0 for an empty row, else 1 + ceil(log2 c) (32 - clz(c - 1) = ceil(log2 c))
         const int o = c == 0u ? 0 : 33 - __clz(c - 1u);
-        keys[i] = (uint32_t)min(o, kPairOctaves - 1);
+        const uint32_t key = (uint32_t)min(o, kPairOctaves - 1);
+        keys[i] = key;
         vals[i] = (uint32_t)i;
+        count_digits(key, 1, sh);
     }
+    __syncthreads();
+    add_digits(1, sh, hist);
 }
 
-__global__ void k_octave_bounds(const uint32_t* hist, int ntiles, int64_t n, uint32_t* bounds)
+__global__ void k_octave_bounds(const uint32_t* hist, int64_t n, uint32_t* bounds)
 {
     const int o = threadIdx.x;
-    if (o < kPairOctaves) bounds[o] = hist[(int64_t)o * ntiles];
-    if (o == kPairOctaves) bounds[o] = (uint32_t)n;
+    const uint32_t c = o < kPairOctaves ? hist[o] : 0u;
+    const uint32_t inc = warp_incl_scan(c);
+    if (o <= kPairOctaves) bounds[o] = o < kPairOctaves ? inc - c : (uint32_t)n;
 }
 
-int launch_pair_bins(const Launch& L, int64_t n, const uint32_t* cnt, uint32_t* keys, uint32_t* order,
-                     uint32_t* keys_alt, uint32_t* vals_alt, uint32_t* hist, uint32_t* scan_tmp, uint32_t* bounds)
+int launch_pair_bins(const Launch& L, int64_t n, const uint32_t* cnt, const RadixSort& rs, uint32_t* bounds, int* status)
 {
     if (n <= 0) return 0;
-    int64_t blocks = (n + 255) / 256;
-    if (blocks > (int64_t)L.sms * 16) blocks = (int64_t)L.sms * 16;
-    k_octave_keys<<<(unsigned)blocks, 256, 0, L.stream>>>(n, cnt, keys, order);
-    int launches = 1;
-    const int ntiles = (int)((n + kRsTile - 1) / kRsTile);
-    if (n > 1) {
-        launches += launch_radix_sort(L, n, 1, keys, order, keys_alt, vals_alt, hist, scan_tmp);
-    } else {
-        // one particle, no sort: every bound but the last is 0, so it is
-        // summed by the last octave's launch (any lanes-per-particle count
-        // gives a correct sum)
-        cudaMemsetAsync(hist, 0, sizeof(uint32_t) * 256, L.stream);
-    }
-    k_octave_bounds<<<1, 32, 0, L.stream>>>(hist, ntiles, n, bounds);
+    cudaMemsetAsync(rs.work, 0, radix_work_words(n) * sizeof(uint32_t), L.stream);
+    uint32_t *k, *v;
+    rs.input(1, k, v);
+    k_octave_keys<<<blocks_for(n, 256, L.sms, 8), 256, 0, L.stream>>>(n, cnt, k, v, rs.work);
+    const int launches = 1 + launch_radix_sort(L, n, 1, rs, status);
+    k_octave_bounds<<<1, 32, 0, L.stream>>>(rs.work, n, bounds);
     return launches + 1;
 }
 
@@ -682,9 +724,20 @@ __global__ void __launch_bounds__(256) k_gather(int64_t n, const uint32_t* skeys
                                                 State src, State dst, const uint32_t* perm_src,
                                                 uint32_t* perm_dst, const PatchDev* pd, Grid g,
                                                 Recs r, Fp64 f, int mixed, RowHint hint,
-                                                const double* hsearch, double* hsearch_out)
+                                                const double* hsearch, double* hsearch_out, const int* status)
 {
     const bool have_hint = *hint.valid != 0;
+    // a sort whose wait ran out: the particles keep their order, and the step
+    // ends with its status
+    if (*status & kStTimeout) {
+        const double* from[13] = {src.x, src.y, src.z, src.vx, src.vy, src.vz, src.m, src.h, src.u, src.du_prev, src.axp, src.ayp, src.azp};
+        double* to[13] = {dst.x, dst.y, dst.z, dst.vx, dst.vy, dst.vz, dst.m, dst.h, dst.u, dst.du_prev, dst.axp, dst.ayp, dst.azp};
+        for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+            for (int q = 0; q < 13; q++) to[q][k] = from[q][k];
+            perm_dst[k] = perm_src[k];
+        }
+        return;
+    }
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
          k += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t key = skeys[k];
@@ -734,12 +787,12 @@ __global__ void __launch_bounds__(256) k_gather(int64_t n, const uint32_t* skeys
 int launch_gather(const Launch& L, int64_t n, const uint32_t* skeys, const uint32_t* svals,
                   const State& src, const State& dst, const uint32_t* perm_src, uint32_t* perm_dst,
                   const PatchDev* pd, const Grid& g, const Recs& r, const Fp64& f, int mixed,
-                  const RowHint& hint, const double* hsearch, double* hsearch_out)
+                  const RowHint& hint, const int* status, const double* hsearch, double* hsearch_out)
 {
     if (n <= 0) return 0;
     k_gather<<<blocks_for(n, 256, L.sms, 16), 256, 0, L.stream>>>(n, skeys, svals, src, dst, perm_src,
                                                                  perm_dst, pd, g, r, f, mixed, hint, hsearch,
-                                                                 hsearch_out);
+                                                                 hsearch_out, status);
     return 1;
 }
 
