@@ -62,11 +62,6 @@ __global__ void k_gather_u32(int64_t n, const uint32_t* src, const uint32_t* per
     }
 }
 
-__global__ void k_accum_pairs(const unsigned long long* total, unsigned long long* acc, const int* status)
-{
-    if (!(*status & kStBad)) *acc += *total;
-}
-
 __global__ void k_fill_patch_of(const WorkItem* items, int nitems, uint16_t* patch_of)
 {
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
@@ -348,6 +343,7 @@ PairArgs pair_args(sph_ctx* ctx)
     a.kernel_n = ctx->cfg.kernel_n;
     a.grad_h = ctx->cfg.grad_h;
     a.kb = ctx->kernel_b;
+    a.red = ctx->red;
     a.status = ctx->status;
     a.order = nullptr;
     a.bounds = nullptr;
@@ -378,6 +374,8 @@ StepArgs step_args(sph_ctx* ctx)
     a.partials = ctx->partials;
     a.cons = ctx->cons;
     a.status = ctx->status;
+    a.listed = ctx->pool_used + 1;
+    a.pair_acc = ctx->pair_acc;
     return a;
 }
 
@@ -553,15 +551,15 @@ bool reuse_lists(const sph_ctx* ctx) { return ctx->skin > 0.0 && !ctx->fused; }
 // density, dt, momentum, update (the step after its neighbour phase)
 void enqueue_pair_phases(sph_ctx* ctx)
 {
-    enqueue_density(ctx);
     const Launch L = launch_of(ctx);
+    if (reuse_lists(ctx)) {
+        Phase p(ctx, SPH_PHASE_UPDATE);
+        ctx->launches += launch_hc_reset(L, step_args(ctx));
+    }
+    enqueue_density(ctx);
     {
         Phase p(ctx, SPH_PHASE_UPDATE);
-        const StepArgs a = step_args(ctx);
-        k_accum_pairs<<<1, 1, 0, ctx->stream>>>(ctx->pool_used + 1, ctx->pair_acc, ctx->status);
-        ctx->launches += 1;
-        ctx->launches += launch_hc_min(L, a);
-        ctx->launches += launch_dt(L, a);
+        ctx->launches += launch_dt(L, step_args(ctx));
     }
     enqueue_momentum(ctx);
     {
@@ -627,6 +625,7 @@ sph_status setup_patches(sph_ctx* ctx, int np, const int64_t* offsets)
 {
     std::vector<PatchDev> pd(np);
     std::vector<WorkItem> items;
+    const int chunk = item_chunk(offsets[np], ctx->sms);
     int64_t cbase = 0;
     for (int p = 0; p < np; p++) {
         PatchDev P;
@@ -642,10 +641,10 @@ sph_status setup_patches(sph_ctx* ctx, int np, const int64_t* offsets)
         cbase += cap;
         P.lz = ctx->cfg.lz;
         P.item_begin = (int)items.size();
-        for (int64_t b = P.begin; b < P.end; b += kItemChunk) {
+        for (int64_t b = P.begin; b < P.end; b += chunk) {
             WorkItem w;
             w.begin = b;
-            w.end = b + kItemChunk < P.end ? b + kItemChunk : P.end;
+            w.end = b + chunk < P.end ? b + chunk : P.end;
             w.patch = p;
             w.pad = 0;
             items.push_back(w);
@@ -868,7 +867,11 @@ sph_status sph_create(const sph_config* cfg_in, sph_ctx** out)
         ctx->max_pairs_s = (int64_t)((double)ctx->max_pairs * g * g * g * 1.1) + 64;
         ctx->pool_cap = ctx->max_pairs_s * 5 / 2 + 24 * cfg.max_particles + 64;
     }
-    ctx->cap_items = (int)(ctx->cap_n / kItemChunk + ctx->cap_patch + 1);
+    {
+        // item_chunk() gives at most this many full items
+        const int64_t slots = (int64_t)ctx->sms * 8;
+        ctx->cap_items = (int)((ctx->cap_n / (slots * 4096) + 1) * slots + ctx->cap_patch + 1);
+    }
     ctx->cap_cells = 2 * ctx->cap_n + (int64_t)4096 * ctx->cap_patch;
     const size_t N = (size_t)ctx->cap_n;
 
@@ -894,12 +897,12 @@ sph_status sph_create(const sph_config* cfg_in, sph_ctx** out)
     ok = ok && dalloc(ctx, ctx->rec.r4, N + 16);
     if (ctx->mixed) {
         ok = ok && dalloc(ctx, ctx->rec.r5, N) && dalloc(ctx, ctx->rec.rv, N) && dalloc(ctx, ctx->rec.rt, N) &&
-             dalloc(ctx, ctx->rec.hc, N) && dalloc(ctx, ctx->rec.pf, N) && dalloc(ctx, ctx->rec.uf, N) &&
+             dalloc(ctx, ctx->rec.pf, N) && dalloc(ctx, ctx->rec.uf, N) &&
              dalloc(ctx, ctx->rec.acc, N);
     } else {
         Fp64& f = ctx->f64;
-        double** g[14] = {&f.vhx, &f.vhy, &f.vhz, &f.rho, &f.P, &f.c, &f.A, &f.hc, &f.w, &f.w5, &f.ax, &f.ay, &f.az, &f.du};
-        for (int k = 0; k < 14 && ok; k++) ok = dalloc(ctx, *g[k], N);
+        double** g[13] = {&f.vhx, &f.vhy, &f.vhz, &f.rho, &f.P, &f.c, &f.A, &f.w, &f.w5, &f.ax, &f.ay, &f.az, &f.du};
+        for (int k = 0; k < 13 && ok; k++) ok = dalloc(ctx, *g[k], N);
     }
     ok = ok && dalloc(ctx, ctx->bin_order, N) && dalloc(ctx, ctx->bin_bounds, (size_t)kPairOctaves + 1);
     ok = ok && dalloc(ctx, ctx->cnt, N) && dalloc(ctx, ctx->cnt_orig, N) && dalloc(ctx, ctx->nown, N) &&

@@ -31,7 +31,19 @@ constexpr int kColBits = 25;                   // packed column: j | stencil << 
 constexpr uint32_t kColMask = (1u << kColBits) - 1u;
 constexpr int64_t kMaxParticles = int64_t(1) << kColBits;
 constexpr int kMaxPatches = 256;
-constexpr int kItemChunk = 4096;               // particles per work item
+// Particles per work item (a chunk of one patch that one block of 256 threads
+// takes): eight items for every SM where there are few particles (two blocks
+// for all of 8000 left the step's passes at 40 us each), else rounds of eight
+// of at most 4096 particles each (a shorter item spends the FP64 pipe on its
+// block sum: 1024 took 0.74 ms in k_update at 8 M, 4096 0.63).
+inline int item_chunk(int64_t n, int sms)
+{
+    const int64_t slots = (int64_t)sms * 8;
+    const int64_t rounds = (n + slots * 4096 - 1) / (slots * 4096);
+    const int64_t per = slots * (rounds < 1 ? 1 : rounds);
+    const int64_t c = ((n + per - 1) / per + 255) / 256 * 256;
+    return (int)(c < 256 ? 256 : c);
+}
 constexpr uint32_t kFarCode = 127;             // column stencil code: offset from the cell coordinates
 #ifndef SPH_BIG_SHARE
 #define SPH_BIG_SHARE 64
@@ -130,7 +142,6 @@ struct Recs {             // FP32 records (written by gather / density)
     float4* r5;          // {ox, oy, oz, m}      pair sums (mixed)
     float4* rv;          // {vhx, vhy, vhz, 1/(2h)} time-centred velocity (mixed)
     float4* rt;          // {rho, P/rho^2, c, h} thermodynamics (mixed)
-    float* hc;           // h/c (mixed)
     float* pf;           // P (mixed)
     float* uf;           // u, staged by the gather (mixed)
     float4* acc;         // {ax, ay, az, du} (mixed)
@@ -138,7 +149,7 @@ struct Recs {             // FP32 records (written by gather / density)
 
 struct Fp64 {             // FP64-path fields
     double *vhx, *vhy, *vhz;   // time-centred velocity
-    double *rho, *P, *c, *A, *hc;
+    double *rho, *P, *c, *A;
     double *w, *w5;            // w = 1/(2h) and w^5 of the kernel gradient
     double *ax, *ay, *az, *du;
 };
@@ -283,6 +294,7 @@ struct PairArgs {
     int kernel, kernel_n;                // SPH_KERNEL_*; n of the Sinc kernel
     int grad_h;                          // 1: grad-h form (density stores A/Omega)
     double kb;                           // sigma_W (Wendland) or B_n (Sinc)
+    PatchRed* red;                       // hcmin: the density sum's minimum of h/c per patch
     int* status;
     // row-length bins (nullptr order: every particle, in sorted order): the
     // launch takes positions bounds[bin_lo] .. bounds[bin_hi + 1] of order,
@@ -336,8 +348,12 @@ struct StepArgs {
     double* partials;    // [nitems][7]
     double* cons;        // [npatch][7]
     int* status;
+    const unsigned long long* listed;  // entries of this step's lists
+    unsigned long long* pair_acc;      // ... summed over the steps
 };
-int launch_hc_min(const Launch& L, const StepArgs& a);
+// the minima of h/c afresh, for a density sum with no sort before it
+int launch_hc_reset(const Launch& L, const StepArgs& a);
+// the time-step of every patch, and the step's pairs added to pair_acc
 int launch_dt(const Launch& L, const StepArgs& a);
 int launch_update(const Launch& L, const StepArgs& a);
 // reused candidate supersets: the state the superset was built on (sorted

@@ -53,48 +53,17 @@ __device__ __forceinline__ void cons_accum(double x, double y, double vx, double
     acc[6] = fma(m, u, acc[6]);
 }
 
-// ---- min over particles of h/c, per patch ---------------------------------
-__global__ void __launch_bounds__(256) k_hc_min(StepArgs a)
-{
-    __shared__ unsigned long long sh[8];
-    if (*a.status & kStBad) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
-        const WorkItem w = a.items[it];
-        unsigned long long mn = ~0ull;
-        for (int64_t i = w.begin + threadIdx.x; i < w.end; i += blockDim.x) {
-            const double v = a.mixed ? (double)a.r.hc[i] : a.f.hc[i];
-            const unsigned long long o = ord_f64(v);
-            mn = o < mn ? o : mn;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long t = __shfl_xor_sync(0xffffffffu, mn, o);
-            mn = t < mn ? t : mn;
-        }
-        if (lane == 0) sh[warp] = mn;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int ww = 1; ww < (int)(blockDim.x >> 5); ww++) mn = sh[ww] < mn ? sh[ww] : mn;
-            atomicMin(&a.red[w.patch].hcmin, mn);
-        }
-        __syncthreads();
-    }
-}
-
-// every step starts its minima afresh (a step that reuses its lists runs no
-// sort, whose reset would otherwise clear them)
+// a step that reuses its lists runs no sort, whose reset would clear the
+// minima of h/c
 __global__ void k_hc_reset(PatchRed* red, int npatch)
 {
     for (int p = threadIdx.x; p < npatch; p += blockDim.x) red[p].hcmin = ~0ull;
 }
 
-int launch_hc_min(const Launch& L, const StepArgs& a)
+int launch_hc_reset(const Launch& L, const StepArgs& a)
 {
-    if (a.nitems <= 0) return 0;
     k_hc_reset<<<1, 256, 0, L.stream>>>(a.red, a.npatch);
-    const int grid = a.nitems < L.sms * 8 ? a.nitems : L.sms * 8;
-    k_hc_min<<<grid, 256, 0, L.stream>>>(a);
-    return 2;
+    return 1;
 }
 
 // ---- Courant time-step per patch ------------------------------------------
@@ -102,6 +71,7 @@ __global__ void k_dt(StepArgs a)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.npatch || (*a.status & kStBad)) return;
+    if (p == 0) *a.pair_acc += *a.listed;
     PatchDev* P = a.pd + p;
     if (P->end <= P->begin) {
         P->dt = 0.0;
@@ -219,22 +189,30 @@ __device__ __forceinline__ void neumaier_add(double& s, double& c, double v)
     s = t;
 }
 
-// one warp per (patch, quantity): lane l takes the item partials l, l + 32,
-// ... in order with a compensated sum; lane 0 then adds the 32 lane sums in
-// lane order.  The order is fixed, so the result is reproducible.  With
-// advance != 0 (after an update) it also closes the step.
-__global__ void __launch_bounds__(32) k_conserved_finalize(StepArgs a, int advance)
+// One block per (patch, quantity): thread t takes the item partials t, t + 256,
+// ... in order with a compensated sum; lane l of the first warp adds the sums
+// of threads l, l + 32, ..., and lane 0 the 32 lane sums in lane order.  The
+// order is fixed, so the result is reproducible.  Bound by the chain of
+// dependent additions: with one warp for all partials it took 32 us at 8 M
+// particles.  With advance != 0 (after an update) it also closes the step.
+__global__ void __launch_bounds__(256) k_conserved_finalize(StepArgs a, int advance)
 {
+    __shared__ double sh_s[256], sh_c[256];
     const int t = blockIdx.x;
     if (t >= a.npatch * 7) return;
-    const int lane = threadIdx.x;
     const int p = t / 7, q = t % 7;
     PatchDev* P = a.pd + p;
-    const bool ok = !(*a.status & kStBad);
-    if (advance && !ok) return;
+    if (advance && (*a.status & kStBad)) return;
     double s = 0.0, c = 0.0;
-    for (int it = P->item_begin + lane; it < P->item_end; it += 32)
-        neumaier_add(s, c, a.partials[(int64_t)it * 7 + q]);
+    for (int it = P->item_begin + threadIdx.x; it < P->item_end; it += 256) neumaier_add(s, c, a.partials[(int64_t)it * 7 + q]);
+    sh_s[threadIdx.x] = s;
+    sh_c[threadIdx.x] = c;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    for (int k = threadIdx.x + 32; k < 256; k += 32) {
+        neumaier_add(s, c, sh_s[k]);
+        c += sh_c[k];
+    }
     double S = 0.0, C = 0.0;
     for (int l = 0; l < 32; l++) {
         const double sl = __shfl_sync(0xffffffffu, s, l);
@@ -242,7 +220,7 @@ __global__ void __launch_bounds__(32) k_conserved_finalize(StepArgs a, int advan
         neumaier_add(S, C, sl);
         C += cl;
     }
-    if (lane == 0) {
+    if (threadIdx.x == 0) {
         a.cons[p * 7 + q] = S + C;
         if (advance && q == 0) {
             P->dt_prev = P->dt;
@@ -253,13 +231,13 @@ __global__ void __launch_bounds__(32) k_conserved_finalize(StepArgs a, int advan
 
 int launch_conserved_finalize(const Launch& L, const StepArgs& a)
 {
-    k_conserved_finalize<<<a.npatch * 7, 32, 0, L.stream>>>(a, 0);
+    k_conserved_finalize<<<a.npatch * 7, 256, 0, L.stream>>>(a, 0);
     return 1;
 }
 
 int launch_step_finalize(const Launch& L, const StepArgs& a)
 {
-    k_conserved_finalize<<<a.npatch * 7, 32, 0, L.stream>>>(a, 1);
+    k_conserved_finalize<<<a.npatch * 7, 256, 0, L.stream>>>(a, 1);
     return 1;
 }
 
