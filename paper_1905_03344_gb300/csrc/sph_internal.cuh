@@ -87,6 +87,7 @@ struct PatchDev {
     int32_t nbig;                // big particles (h > hs), counted by the key kernel
     uint32_t row_fill;           // slots of the row copy handed out so far
     double hs;                   // class threshold: small iff h <= hs
+    double hlz, hsz;             // lz / 2, sz / 2
     float hs_f;
     double hmed;                 // median of h (histogram bin centre)
     int32_t kc;                  // coarse cell = 2^kc fine cells per axis
@@ -171,6 +172,43 @@ __host__ __device__ __forceinline__ double unord_f64(unsigned long long u)
     return d;
 #endif
 }
+// FP64 conversions, sign tests and comparisons in integer arithmetic.  An SM
+// retires two FP64 operations a clock, and a conversion or a comparison takes
+// as much of that pipe as a multiply-add: with them the passes over the
+// particles (keys, gather, update) were bound by it, not by memory.
+//
+// the nearest float, ties to even, as (float)d
+__device__ __forceinline__ float f64_to_f32(double d)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+    const uint32_t e = (hi >> 20) & 0x7ffu;
+    if (e - 897u > 253u) return (hi << 1 | lo) == 0u ? __uint_as_float(hi) : (float)d;   // 0; outside the normal floats
+    const uint32_t m = __funnelshift_l(lo, hi & 0x000fffffu, 3);      // 23 bits
+    const uint32_t rest = lo << 3;
+    const uint32_t up = rest > 0x80000000u || (rest == 0x80000000u && (m & 1u)) ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | (((e - 896u) << 23) + m + up));
+}
+// (double)f
+__device__ __forceinline__ double f32_to_f64(float f)
+{
+    const uint32_t u = __float_as_uint(f), t = u & 0x7fffffffu;
+    if (t - 0x00800000u >= 0x7f000000u) return t == 0u ? __hiloint2double((int)u, 0) : (double)f;   // 0; subnormal, infinite, NaN
+    return __hiloint2double((int)((u & 0x80000000u) | ((t >> 3) + 0x38000000u)), (int)(u << 29));
+}
+// (double)v for 0 <= v < 2^20
+__device__ __forceinline__ double small_to_f64(uint32_t v)
+{
+    if (v == 0u) return 0.0;
+    const int k = 31 - __clz(v);
+    return __hiloint2double((int)(((1023u + (uint32_t)k) << 20) | ((v << (20 - k)) & 0x000fffffu)), 0);
+}
+// a > b and a < -b for b > 0 and a no NaN
+__device__ __forceinline__ bool above(double a, double b) { return __double_as_longlong(a) > __double_as_longlong(b); }
+__device__ __forceinline__ bool below_neg(double a, double b)
+{
+    return (unsigned long long)__double_as_longlong(a) > ((unsigned long long)__double_as_longlong(b) | 0x8000000000000000ull);
+}
+
 __host__ __device__ __forceinline__ uint32_t part1by2(uint32_t v)
 {
     v &= 0x3ffu;

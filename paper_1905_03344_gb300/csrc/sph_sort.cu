@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(256) k_reduce_bbox(State s, const WorkItem* it
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const WorkItem w = items[it];
         unsigned long long v[5] = {~0ull, ~0ull, 0ull, 0ull, 0ull};
+#pragma unroll 4
         for (int64_t i = w.begin + threadIdx.x; i < w.end; i += blockDim.x) {
             unsigned long long a = ord_f64(s.x[i]), b = ord_f64(s.y[i]), c = ord_f64(s.h[i]);
             v[0] = umin64(v[0], a);
@@ -112,23 +113,33 @@ __global__ void k_reset_red(int npatch, PatchRed* red, uint32_t* zero, int64_t w
 __global__ void __launch_bounds__(256) k_h_hist(State s, const WorkItem* items, int nitems, PatchRed* red)
 {
     __shared__ uint32_t hist[kHBins];
-    const int lane = threadIdx.x & 31;
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const WorkItem w = items[it];
         for (int b = threadIdx.x; b < kHBins; b += blockDim.x) hist[b] = 0u;
         __syncthreads();
         const double hmax = unord_f64(red[w.patch].hmax);
         const double scale = hmax > 0.0 ? (double)kHBins / hmax : 0.0;
-        // warp-uniform trip count (blockDim is a multiple of 32)
+        const float scale_f = (float)scale;
         for (int64_t i0 = w.begin; i0 < w.end; i0 += blockDim.x) {
             const int64_t i = i0 + threadIdx.x;
-            int b = -1;
+            int b;
             if (i < w.end) {
-                const double t = s.h[i] * scale;
-                b = t >= 0.0 && t < (double)kHBins ? (int)t : kHBins - 1;
+                // the bin in FP32 where it is clear of the bins' edges (h is
+                // at most h_max, so past the last edge it is the last bin)
+                const double h = s.h[i];
+                const float tf = f64_to_f32(h) * scale_f;
+                b = (int)tf;
+                const float fr = tf - (float)b;
+                if (b >= kHBins - 1 && fr > 1e-4f) {
+                    b = kHBins - 1;
+                } else if (b > kHBins - 1) {
+                    b = kHBins - 1;
+                } else if (!(fr > 1e-4f && fr < 1.0f - 1e-4f)) {
+                    const double t = h * scale;
+                    b = t >= 0.0 && t < (double)kHBins ? (int)t : kHBins - 1;
+                }
+                atomicAdd(&hist[b], 1u);
             }
-            const unsigned peers = __match_any_sync(0xffffffffu, b);
-            if (b >= 0 && lane == __ffs(peers) - 1) atomicAdd(&hist[b], (uint32_t)__popc(peers));
         }
         __syncthreads();
         for (int b = threadIdx.x; b < kHBins; b += blockDim.x)
@@ -272,6 +283,8 @@ __global__ void k_grid_params(int npatch, const PatchRed* red, PatchDev* pd, dou
     P.inv_s_f = (float)(1.0 / s);
     P.inv_sz_f = (float)(1.0 / P.sz);
     P.hmax_f = (float)hmax;
+    P.hlz = 0.5 * P.lz;
+    P.hsz = 0.5 * P.sz;
     P.hs = hs;
     P.hs_f = (float)hs;
     P.hmed = hmed;
@@ -323,16 +336,16 @@ __global__ void __launch_bounds__(256) k_keys(int64_t n, State s, const uint16_t
          i += (int64_t)gridDim.x * blockDim.x) {
         const int p = patch_of[i];
         PatchDev* P = pd + p;
-        const bool big = s.h[i] > P->hs;
+        const bool big = above(s.h[i], P->hs);
         // one atomic per warp and patch: the lanes of a warp that share the
         // patch add their big particles together
         const unsigned act = __activemask();
         const unsigned peers = __match_any_sync(act, p);
         const unsigned bigs = __ballot_sync(act, big) & peers;
         if (bigs && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&P->nbig, __popc(bigs));
-        const float tx = (float)(s.x[i] - P->xmin) * P->inv_s_f;
-        const float ty = (float)(s.y[i] - P->ymin) * P->inv_s_f;
-        const float tz = (float)(s.z[i] + 0.5 * P->lz) * P->inv_sz_f;
+        const float tx = f64_to_f32(s.x[i] - P->xmin) * P->inv_s_f;
+        const float ty = f64_to_f32(s.y[i] - P->ymin) * P->inv_s_f;
+        const float tz = f64_to_f32(s.z[i] + P->hlz) * P->inv_sz_f;
         int cx = (int)floorf(tx), cy = (int)floorf(ty), cz = (int)floorf(tz);
         cx = min(max(cx, 0), P->ncx - 1);
         cy = min(max(cy, 0), P->ncy - 1);
@@ -695,21 +708,21 @@ __device__ __forceinline__ void write_records(int64_t k, const PatchDev* P, uint
                                               double m, double h, double u, double axp, double ayp, double azp,
                                               float hq, Recs& r, Fp64& f, int mixed)
 {
-    const float ox = (float)(x - (P->xmin + (double)cx * P->s));
-    const float oy = (float)(y - (P->ymin + (double)cy * P->s));
-    double ozd = z - (-0.5 * P->lz + (double)cz * P->sz);
-    const double oc = ozd - 0.5 * P->sz;
-    if (oc > 0.5 * P->lz) ozd -= P->lz;
-    else if (oc < -0.5 * P->lz) ozd += P->lz;
-    const float oz = (float)ozd;
-    const float hf = (float)h;
+    const float ox = f64_to_f32(x - fma(small_to_f64(cx), P->s, P->xmin));
+    const float oy = f64_to_f32(y - fma(small_to_f64(cy), P->s, P->ymin));
+    double ozd = z - fma(small_to_f64(cz), P->sz, -P->hlz);
+    const double oc = ozd - P->hsz;
+    if (above(oc, P->hlz)) ozd -= P->lz;
+    else if (below_neg(oc, P->hlz)) ozd += P->lz;
+    const float oz = f64_to_f32(ozd);
+    const float hf = f64_to_f32(h);
     r.r4[k] = make_float4(ox, oy, oz, 4.0f * hq * hq);
     const double half = P->step > 0 ? 0.5 * P->dt_prev : 0.0;
     const double vhx = vx + axp * half, vhy = vy + ayp * half, vhz = vz + azp * half;
     if (mixed) {
-        r.r5[k] = make_float4(ox, oy, oz, (float)m);
-        r.rv[k] = make_float4((float)vhx, (float)vhy, (float)vhz, 0.5f / hf);
-        r.uf[k] = (float)u;
+        r.r5[k] = make_float4(ox, oy, oz, f64_to_f32(m));
+        r.rv[k] = make_float4(f64_to_f32(vhx), f64_to_f32(vhy), f64_to_f32(vhz), 0.5f / hf);
+        r.uf[k] = f64_to_f32(u);
     } else {
         f.vhx[k] = vhx;
         f.vhy[k] = vhy;
@@ -761,7 +774,7 @@ __global__ void __launch_bounds__(256) k_gather(int64_t n, const uint32_t* skeys
         const uint32_t cx = compact1by2(mort), cy = compact1by2(mort >> 1), cz = compact1by2(mort >> 2);
         g.cellxyz[k] = cx | (cy << 8) | (cz << 16);
         // h of the search
-        const float hf = (float)(hsearch ? hsearch[si] : h);
+        const float hf = f64_to_f32(hsearch ? hsearch[si] : h);
         if (hsearch_out) hsearch_out[k] = hsearch[si];
         write_records(k, P, cx, cy, cz, x, y, z, vx, vy, vz, m, h, dst.u[k], axp, ayp, azp, hf, r, f, mixed);
         if (!big) {

@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(256) k_update(StepArgs a)
     for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
         const WorkItem w = a.items[it];
         const PatchDev* P = a.pd + w.patch;
-        const double dt = P->dt, lz = P->lz;
+        const double dt = P->dt, lz = P->lz, hlz = 0.5 * lz;
         const bool first = P->step == 0;
         const double kick = 0.5 * (dt + (first ? 0.0 : P->dt_prev));
         const double r = first ? 0.0 : dt / P->dt_prev;
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(256) k_update(StepArgs a)
             double ax, ay, az, du;
             if (a.mixed) {
                 const float4 q = a.r.acc[i];
-                ax = q.x; ay = q.y; az = q.z; du = q.w;
+                ax = f32_to_f64(q.x); ay = f32_to_f64(q.y); az = f32_to_f64(q.z); du = f32_to_f64(q.w);
             } else {
                 ax = a.f.ax[i]; ay = a.f.ay[i]; az = a.f.az[i]; du = a.f.du[i];
             }
@@ -122,8 +122,8 @@ __global__ void __launch_bounds__(256) k_update(StepArgs a)
             const double x = a.s.x[i] + vx * dt;
             const double y = a.s.y[i] + vy * dt;
             double z = a.s.z[i] + vz * dt;
-            if (z >= 0.5 * lz) z -= lz;
-            else if (z < -0.5 * lz) z += lz;
+            if (!above(hlz, z)) z -= lz;
+            else if (below_neg(z, hlz)) z += lz;
             const double u0 = a.s.u[i];
             const double u = first ? u0 + dt * du : u0 + dt * (c1 * du - c0 * a.s.du_prev[i]);
             a.s.vx[i] = vx; a.s.vy[i] = vy; a.s.vz[i] = vz;
