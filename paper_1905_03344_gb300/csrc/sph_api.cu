@@ -339,6 +339,9 @@ PairArgs pair_args(sph_ctx* ctx)
     a.alpha = ctx->cfg.av_alpha;
     a.beta = ctx->cfg.av_beta;
     a.eps = ctx->cfg.av_eps;
+    a.vh = 0.5 * std::sqrt(a.eps);
+    a.vc = a.alpha / std::sqrt(a.eps);
+    a.vb = 2.0 * a.beta / a.eps;
     a.kernel = ctx->cfg.kernel;
     a.kernel_n = ctx->cfg.kernel_n;
     a.grad_h = ctx->cfg.grad_h;
@@ -418,7 +421,7 @@ void enqueue_sort(sph_ctx* ctx, bool superset = false)
         const int nxt = 1 - ctx->cur;
         ctx->launches += launch_gather(L, ctx->n, ctx->keys, ctx->vals, ctx->st[ctx->cur], ctx->st[nxt],
                                        ctx->perm[ctx->cur], ctx->perm[nxt], ctx->pd, ctx->grid, ctx->rec,
-                                       ctx->f64, ctx->mixed,
+                                       ctx->f64, ctx->mixed, ctx->cfg.kernel,
                                        superset ? RowHint{ctx->cnt_s, ctx->hint_ok_s, ctx->rowcap}
                                                 : RowHint{ctx->cnt, ctx->hint_ok, ctx->rowcap},
                                        ctx->status,
@@ -531,7 +534,8 @@ void enqueue_filter(sph_ctx* ctx)
     {
         Phase p(ctx, SPH_PHASE_GATHER);
         ctx->launches += launch_refresh_records(L, ctx->n, ctx->st[ctx->cur], ctx->patch_of, ctx->pd,
-                                                ctx->grid.cellxyz, ctx->rec, ctx->f64, ctx->mixed);
+                                                ctx->grid.cellxyz, ctx->rec, ctx->f64, ctx->mixed,
+                                                ctx->cfg.kernel);
     }
     {
         Phase p(ctx, SPH_PHASE_NB_RESET);
@@ -901,8 +905,8 @@ sph_status sph_create(const sph_config* cfg_in, sph_ctx** out)
              dalloc(ctx, ctx->rec.acc, N);
     } else {
         Fp64& f = ctx->f64;
-        double** g[13] = {&f.vhx, &f.vhy, &f.vhz, &f.rho, &f.P, &f.c, &f.A, &f.w, &f.w5, &f.ax, &f.ay, &f.az, &f.du};
-        for (int k = 0; k < 13 && ok; k++) ok = dalloc(ctx, *g[k], N);
+        double** g[16] = {&f.vhx, &f.vhy, &f.vhz, &f.rho, &f.P, &f.c, &f.A, &f.w, &f.g0, &f.g1, &f.ha, &f.ca, &f.ax, &f.ay, &f.az, &f.du};
+        for (int k = 0; k < 16 && ok; k++) ok = dalloc(ctx, *g[k], N);
     }
     ok = ok && dalloc(ctx, ctx->bin_order, N) && dalloc(ctx, ctx->bin_bounds, (size_t)kPairOctaves + 1);
     ok = ok && dalloc(ctx, ctx->cnt, N) && dalloc(ctx, ctx->cnt_orig, N) && dalloc(ctx, ctx->nown, N) &&

@@ -146,7 +146,7 @@ struct MomSinkD {
     int kn;
     uint32_t* q;
     uint32_t head, tail;
-    double ax, ay, az, du;
+    MomAccD A;
 
     __device__ __forceinline__ uint32_t mark() const { return 0u; }
     __device__ __forceinline__ void decide(const NbArgs& a, const PatchDev* P, int64_t i, uint32_t j, float r2,
@@ -159,13 +159,7 @@ struct MomSinkD {
     // every queued pair, in order
     __device__ __forceinline__ void group_end(uint32_t)
     {
-        for (; head != tail; head++) {
-            const PairTermsD t = momentum_pair_fp64<KERN, GH>(*pa, I, q[32 * (head & (kQueue - 1))], kn);
-            ax += t.ax;
-            ay += t.ay;
-            az += t.az;
-            du += t.du;
-        }
+        for (; head != tail; head++) momentum_pair_fp64<KERN, GH>(*pa, I, q[32 * (head & (kQueue - 1))], kn, A);
     }
     __device__ __forceinline__ void finish() { group_end(0u); }
 };
@@ -284,10 +278,10 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_MOM_MINB)
         const int64_t i = U.begin + lane;
         if (i < U.end) {
             const bool big = i >= P->end - (int64_t)P->nbig;
-            MomSinkD<KERN, GH> s = {&pa, side_fp64(pa, P, i), pa.kernel_n, qlane, 0u, 0u, 0.0, 0.0, 0.0, 0.0};
+            MomSinkD<KERN, GH> s = {&pa, side_fp64(pa, P, i), pa.kernel_n, qlane, 0u, 0u, {0.0, 0.0, 0.0, 0.0}};
             walk_all<MomSinkD<KERN, GH>>(a, P, i, big, s);
             s.finish();
-            momentum_finish_fp64(pa, i, S80, s.ax, s.ay, s.az, s.du);
+            momentum_finish_fp64(pa, i, S80, s.A);
         }
     }
 }

@@ -151,7 +151,11 @@ struct Recs {             // FP32 records (written by gather / density)
 struct Fp64 {             // FP64-path fields
     double *vhx, *vhy, *vhz;   // time-centred velocity
     double *rho, *P, *c, *A;
-    double *w, *w5;            // w = 1/(2h) and w^5 of the kernel gradient
+    double *w;                 // 1/(2h)
+    double *g0, *g1;           // of the kernel gradient's factor: w^(5/3) and
+                               // w^(8/3) (Wendland), w^5 and w (Sinc)
+    double *ha, *ca;           // of the viscosity, from the density sum:
+                               // h sqrt(eps) / 2 and c alpha / sqrt(eps)
     double *ax, *ay, *az, *du;
 };
 
@@ -272,12 +276,12 @@ struct RowHint {
 int launch_gather(const Launch& L, int64_t n, const uint32_t* skeys, const uint32_t* svals,
                   const State& src, const State& dst, const uint32_t* perm_src,
                   uint32_t* perm_dst, const PatchDev* pd, const Grid& g, const Recs& r,
-                  const Fp64& f, int mixed, const RowHint& hint, const int* status, const double* hsearch = nullptr,
+                  const Fp64& f, int mixed, int kernel, const RowHint& hint, const int* status, const double* hsearch = nullptr,
                   double* hsearch_out = nullptr);
 // the FP32 records of the current state in the current sorted order, on the
 // grid of the last sort (what the gather writes, with the unscaled h)
 int launch_refresh_records(const Launch& L, int64_t n, const State& s, const uint16_t* patch_of,
-                           const PatchDev* pd, const uint32_t* cellxyz, const Recs& r, const Fp64& f, int mixed);
+                           const PatchDev* pd, const uint32_t* cellxyz, const Recs& r, const Fp64& f, int mixed, int kernel);
 // after the gather: the row copy of the small particles' search records,
 // g.hnb for stencil half-extent K (tmp: one float per cell) and the state's
 // vote for the grid of the next sort (vote[0]: non-empty fine cells, vote[1]:
@@ -329,6 +333,7 @@ struct PairArgs {
     Recs r;
     Fp64 f;
     double gamma, alpha, beta, eps;
+    double vh, vc, vb;                   // sqrt(eps) / 2, alpha / sqrt(eps), 2 beta / eps
     int kernel, kernel_n;                // SPH_KERNEL_*; n of the Sinc kernel
     int grad_h;                          // 1: grad-h form (density stores A/Omega)
     double kb;                           // sigma_W (Wendland) or B_n (Sinc)

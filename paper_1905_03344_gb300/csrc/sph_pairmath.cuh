@@ -178,6 +178,57 @@ __device__ __forceinline__ double sinc_g(double x, double sn, double cs)
     return fma(-x, cs, sn) / (x * x * x);
 }
 
+// FP64 helpers of the pair loops.  The FP64 pipe, two lanes a clock and SM,
+// bounds both FP64 sums, and library square roots and divisions, comparisons
+// and max each put several operations on it that integer and FP32 units can
+// do or start.
+// max(q, 0) for a q that is no NaN
+__device__ __forceinline__ double pos0(double q)
+{
+    const int hi = __double2hiint(q);
+    return __hiloint2double(hi < 0 ? 0 : hi, hi < 0 ? 0 : __double2loint(q));
+}
+// the bits of a positive double in the normal float range as a float (not
+// rounded), and back
+__device__ __forceinline__ float seed_f32(double x)
+{
+    return __uint_as_float(__funnelshift_l((uint32_t)__double2loint(x), (uint32_t)__double2hiint(x) - 0x38000000u, 3));
+}
+__device__ __forceinline__ double seed_f64(float f)
+{
+    const uint32_t u = __float_as_uint(f);
+    return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
+}
+// x is positive with an exponent within 2^+-120
+__device__ __forceinline__ bool seedable(double x)
+{
+    return (uint32_t)__double2hiint(x) - (903u << 20) < (240u << 20);
+}
+// sqrt(x) by Goldschmidt's iteration from an FP32 reciprocal square root (22
+// bits; one step makes 44), then the residual's correction (Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000
+// processor", 1990): six FP64 operations
+__device__ __forceinline__ double sqrt_fp64(double x)
+{
+    if (!seedable(x)) return sqrt(x);
+    const double y = seed_f64(rsqrtf(seed_f32(x)));
+    const double g = x * y;
+    const double h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));   // y / 2
+    const double e = fma(-g, h, 0.5);
+    const double g1 = fma(g, e, g), h1 = fma(h, e, h);
+    return fma(fma(-g1, g1, x), h1, g1);
+}
+// n / x for a positive x, to about an ulp: the FP32 reciprocal's error
+// e = 1 - x y (23 bits), y (1 + e + e^2) leaves e^3 (Newton's iteration of
+// the third order)
+__device__ __forceinline__ double div_fp64(double n, double x)
+{
+    if (!seedable(x)) return n / x;
+    const double y = seed_f64(__fdividef(1.0f, seed_f32(x)));
+    const double e = fma(-x, y, 1.0);
+    return n * fma(y, fma(e, e, e), y);
+}
+
 template <int KERN>
 struct KernF;
 
@@ -192,7 +243,7 @@ struct KernF<SPH_KERNEL_WENDLAND> {
     }
     static __device__ __forceinline__ double dens(double r, double w, int)
     {
-        const double q = fmax(fma(-r, w, 1.0), 0.0);
+        const double q = pos0(fma(-r, w, 1.0));
         const double q2 = q * q;
         return q2 * q2 * fma(-4.0, q, 5.0);
     }
@@ -202,10 +253,11 @@ struct KernF<SPH_KERNEL_WENDLAND> {
         const float q = fmaxf(fmaf(-r, w, 1.0f), 0.0f);
         return w5 * (q * q * q);
     }
-    static __device__ __forceinline__ double grad(double r, double w, double w5, int)
+    // (in FP64 from g0 = w^(5/3) and g1 = g0 w, as (g0 q)^3)
+    static __device__ __forceinline__ double grad(double r, double g0, double g1, int)
     {
-        const double q = fmax(fma(-r, w, 1.0), 0.0);
-        return w5 * q * q * q;
+        const double t = pos0(fma(-r, g1, g0));
+        return t * t * t;
     }
     static __host__ __device__ double grad_scale(double kb, int) { return 80.0 * kb; }
     // grad-h weight -v S'(v) of the shape S = q^4 (5 - 4q), q = 1 - v/2:
@@ -218,7 +270,7 @@ struct KernF<SPH_KERNEL_WENDLAND> {
     }
     static __device__ __forceinline__ double omega_w(double r, double w, int)
     {
-        const double q = fmax(fma(-r, w, 1.0), 0.0);
+        const double q = pos0(fma(-r, w, 1.0));
         const double p = 1.0 - q;
         return 20.0 * (p * p) * (q * q * q);
     }
@@ -256,7 +308,7 @@ struct KernF<SPH_KERNEL_SINC> {
         const float S = x > 0.0f ? __fdividef(sn, x) : 1.0f;
         return w5 * ipowf(S, n - 1) * sinc_g(x, sn, cs);
     }
-    static __device__ __forceinline__ double grad(double r, double w, double w5, int n)
+    static __device__ __forceinline__ double grad(double r, double w5, double w, int n)
     {
         const double x = kPi * r * w;
         if (!(x < kPi)) return 0.0;
@@ -693,8 +745,8 @@ __device__ __forceinline__ void pair_dx_fp64(const State& s, double xi, double y
     dx = xi - s.x[j];
     dy = yi - s.y[j];
     dz = zi - s.z[j];
-    if (dz > 0.5 * lz) dz -= lz;
-    else if (dz < -0.5 * lz) dz += lz;
+    // |dz| > lz / 2: only particles near the period's ends
+    if (above(fabs(dz), 0.5 * lz)) dz = __double2hiint(dz) < 0 ? dz + lz : dz - lz;
 }
 
 template <int KERN, bool GH>
@@ -703,7 +755,7 @@ __device__ __forceinline__ void density_pair_fp64(const PairArgs& a, double xi, 
 {
     double dx, dy, dz;
     pair_dx_fp64(a.s, xi, yi, zi, j, lz, dx, dy, dz);
-    const double r = sqrt(fma(dx, dx, fma(dy, dy, dz * dz)));
+    const double r = sqrt_fp64(fma(dx, dx, fma(dy, dy, dz * dz)));
     const double m = a.s.m[j];
     if (GH) {
         double d, g;
@@ -725,6 +777,8 @@ __device__ __forceinline__ double density_finish_fp64(const PairArgs& a, int64_t
     a.f.rho[i] = rho;
     a.f.P[i] = Pr;
     a.f.c[i] = c;
+    a.f.ha[i] = a.vh * hi;
+    a.f.ca[i] = a.vc * c;
     double A = Pr / (rho * rho);
     if (GH) {
         const double om = sumd / (3.0 * (a.s.m[i] + sum));
@@ -738,7 +792,7 @@ __device__ __forceinline__ double density_finish_fp64(const PairArgs& a, int64_t
 
 // particle i's values for the FP64 momentum sum
 struct SideD {
-    double x, y, z, vx, vy, vz, h, w, w5, rho, A, c, lz;
+    double x, y, z, vx, vy, vz, ha, g0, g1, rho, A, ca, lz;
 };
 
 __device__ __forceinline__ SideD side_fp64(const PairArgs& a, const PatchDev* P, int64_t i)
@@ -750,69 +804,72 @@ __device__ __forceinline__ SideD side_fp64(const PairArgs& a, const PatchDev* P,
     I.vx = a.f.vhx[i];
     I.vy = a.f.vhy[i];
     I.vz = a.f.vhz[i];
-    I.h = a.s.h[i];
-    I.w = a.f.w[i];
-    I.w5 = a.f.w5[i];
+    I.ha = a.f.ha[i];
+    I.g0 = a.f.g0[i];
+    I.g1 = a.f.g1[i];
     I.rho = a.f.rho[i];
     I.A = a.f.A[i];
-    I.c = a.f.c[i];
+    I.ca = a.f.ca[i];
     I.lz = P->lz;
     return I;
 }
 
-struct PairTermsD {
+struct MomAccD {
     double ax, ay, az, du;
 };
 
-// one pair of the momentum and energy sums (R4-R6; R20 with GH, A holding A/Omega)
+// one pair of the momentum and energy sums (R4-R6; R20 with GH, A holding
+// A/Omega), added to S with multiply-adds.  49 FP64 operations in the
+// symmetrised Wendland form (35 and 14 for the viscosity of an approaching
+// pair), where the library's square root and division, comparisons on the
+// FP64 pipe, separate products and sums and a factor w^5 came to about 68.
 template <int KERN, bool GH>
-__device__ __forceinline__ PairTermsD momentum_pair_fp64(const PairArgs& a, const SideD& I, uint32_t j, int kn)
+__device__ __forceinline__ void momentum_pair_fp64(const PairArgs& a, const SideD& I, uint32_t j, int kn, MomAccD& S)
 {
     double dx, dy, dz;
     pair_dx_fp64(a.s, I.x, I.y, I.z, j, I.lz, dx, dy, dz);
     const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-    const double r = sqrt(r2);
-    const double fi = KernF<KERN>::grad(r, I.w, I.w5, kn), fj = KernF<KERN>::grad(r, a.f.w[j], a.f.w5[j], kn);
+    const double r = sqrt_fp64(r2);
+    const double fi = KernF<KERN>::grad(r, I.g0, I.g1, kn), fj = KernF<KERN>::grad(r, a.f.g0[j], a.f.g1[j], kn);
     const double F = __dadd_rn(fi, fj);   // not contracted with either product
     const double vx = I.vx - a.f.vhx[j], vy = I.vy - a.f.vhy[j], vz = I.vz - a.f.vhz[j];
     const double vdot = fma(vx, dx, fma(vy, dy, vz * dz));
     double pi_ = 0.0;
-    if (vdot < 0.0) {
-        // Pi = mu (beta mu - alpha cbar) / rhobar with mu = N / D, N = hbar v.x,
-        // D = r^2 + eps hbar^2, as one division: N (beta N - alpha cbar D) / (D^2 rhobar)
-        const double hbar = 0.5 * (I.h + a.s.h[j]);
-        const double N = hbar * vdot, D = fma(a.eps * hbar, hbar, r2);
-        const double cbar = 0.5 * (I.c + a.f.c[j]), rhobar = 0.5 * (I.rho + a.f.rho[j]);
-        pi_ = N * fma(a.beta, N, -a.alpha * cbar * D) / (D * D * rhobar);
+    if (__double2hiint(vdot) < 0) {
+        // Pi = mu (beta mu - alpha cbar) / rhobar, mu = hbar v.x / D, D = r^2 +
+        // eps hbar^2, as one division: with H = sqrt(eps) hbar (the sum of the
+        // two ha), M = H v.x and C the sum of the two ca,
+        // Pi = M (2 beta/eps M - C D) / (D^2 (rho_i + rho_j))
+        const double H = I.ha + a.f.ha[j];
+        const double M = H * vdot, D = fma(H, H, r2);
+        const double C = I.ca + a.f.ca[j], rs = I.rho + a.f.rho[j];
+        pi_ = div_fp64(M * fma(a.vb, M, -(C * D)), D * D * rs);
     }
     const double mj = a.s.m[j];
-    PairTermsD t;
     if (GH) {
         // each side's pressure term with its own kernel
         const double fa = mj * fma(2.0 * I.A, fi, fma(2.0 * a.f.A[j], fj, pi_ * F));
-        t.ax = fa * dx;
-        t.ay = fa * dy;
-        t.az = fa * dz;
-        t.du = -mj * fma(2.0 * I.A, fi, 0.5 * pi_ * F) * vdot;
+        S.ax = fma(fa, dx, S.ax);
+        S.ay = fma(fa, dy, S.ay);
+        S.az = fma(fa, dz, S.az);
+        S.du = fma(-mj * vdot, fma(2.0 * I.A, fi, 0.5 * pi_ * F), S.du);
     } else {
         const double g = mj * F;
         const double fa = g * (I.A + a.f.A[j] + pi_);
-        t.ax = fa * dx;
-        t.ay = fa * dy;
-        t.az = fa * dz;
-        t.du = -g * fma(0.5, pi_, I.A) * vdot;
+        S.ax = fma(fa, dx, S.ax);
+        S.ay = fma(fa, dy, S.ay);
+        S.az = fma(fa, dz, S.az);
+        S.du = fma(-g * vdot, fma(0.5, pi_, I.A), S.du);
     }
-    return t;
 }
 
-__device__ __forceinline__ void momentum_finish_fp64(const PairArgs& a, int64_t i, double S, double ax, double ay,
-                                                     double az, double du)
+__device__ __forceinline__ void momentum_finish_fp64(const PairArgs& a, int64_t i, double s, const MomAccD& S)
 {
-    a.f.ax[i] = S * ax;
-    a.f.ay[i] = S * ay;
-    a.f.az[i] = S * az;
-    a.f.du[i] = S * du;
-    if (!isfinite(ax) || !isfinite(ay) || !isfinite(az) || !isfinite(du)) atomicOr(a.status, kStNonFinite);
+    a.f.ax[i] = s * S.ax;
+    a.f.ay[i] = s * S.ay;
+    a.f.az[i] = s * S.az;
+    a.f.du[i] = s * S.du;
+    if (!isfinite(S.ax) || !isfinite(S.ay) || !isfinite(S.az) || !isfinite(S.du)) atomicOr(a.status, kStNonFinite);
 }
 
 }  // namespace sphg

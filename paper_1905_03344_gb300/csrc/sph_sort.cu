@@ -706,7 +706,7 @@ int launch_pair_bins(const Launch& L, int64_t n, const uint32_t* cnt, const Radi
 __device__ __forceinline__ void write_records(int64_t k, const PatchDev* P, uint32_t cx, uint32_t cy, uint32_t cz,
                                               double x, double y, double z, double vx, double vy, double vz,
                                               double m, double h, double u, double axp, double ayp, double azp,
-                                              float hq, Recs& r, Fp64& f, int mixed)
+                                              float hq, Recs& r, Fp64& f, int mixed, int kernel)
 {
     const float ox = f64_to_f32(x - fma(small_to_f64(cx), P->s, P->xmin));
     const float oy = f64_to_f32(y - fma(small_to_f64(cy), P->s, P->ymin));
@@ -728,15 +728,23 @@ __device__ __forceinline__ void write_records(int64_t k, const PatchDev* P, uint
         f.vhy[k] = vhy;
         f.vhz[k] = vhz;
         const double w = 0.5 / h;
+        const double w5 = w * w * w * w * w;
         f.w[k] = w;
-        f.w5[k] = w * w * w * w * w;
+        if (kernel == SPH_KERNEL_WENDLAND) {
+            const double g0 = cbrt(w5);
+            f.g0[k] = g0;
+            f.g1[k] = g0 * w;
+        } else {
+            f.g0[k] = w5;
+            f.g1[k] = w;
+        }
     }
 }
 
 __global__ void __launch_bounds__(256) k_gather(int64_t n, const uint32_t* skeys, const uint32_t* svals,
                                                 State src, State dst, const uint32_t* perm_src,
                                                 uint32_t* perm_dst, const PatchDev* pd, Grid g,
-                                                Recs r, Fp64 f, int mixed, RowHint hint,
+                                                Recs r, Fp64 f, int mixed, int kernel, RowHint hint,
                                                 const double* hsearch, double* hsearch_out, const int* status)
 {
     const bool have_hint = *hint.valid != 0;
@@ -776,7 +784,7 @@ __global__ void __launch_bounds__(256) k_gather(int64_t n, const uint32_t* skeys
         // h of the search
         const float hf = f64_to_f32(hsearch ? hsearch[si] : h);
         if (hsearch_out) hsearch_out[k] = hsearch[si];
-        write_records(k, P, cx, cy, cz, x, y, z, vx, vy, vz, m, h, dst.u[k], axp, ayp, azp, hf, r, f, mixed);
+        write_records(k, P, cx, cy, cz, x, y, z, vx, vy, vz, m, h, dst.u[k], axp, ayp, azp, hf, r, f, mixed, kernel);
         if (!big) {
             // fine cell of small particles: bounded by a change of key
             const int64_t lin = P->cell_base + ((int64_t)cz * P->ncy + cy) * P->ncx + cx;
@@ -799,12 +807,12 @@ __global__ void __launch_bounds__(256) k_gather(int64_t n, const uint32_t* skeys
 
 int launch_gather(const Launch& L, int64_t n, const uint32_t* skeys, const uint32_t* svals,
                   const State& src, const State& dst, const uint32_t* perm_src, uint32_t* perm_dst,
-                  const PatchDev* pd, const Grid& g, const Recs& r, const Fp64& f, int mixed,
+                  const PatchDev* pd, const Grid& g, const Recs& r, const Fp64& f, int mixed, int kernel,
                   const RowHint& hint, const int* status, const double* hsearch, double* hsearch_out)
 {
     if (n <= 0) return 0;
     k_gather<<<blocks_for(n, 256, L.sms, 16), 256, 0, L.stream>>>(n, skeys, svals, src, dst, perm_src,
-                                                                 perm_dst, pd, g, r, f, mixed, hint, hsearch,
+                                                                 perm_dst, pd, g, r, f, mixed, kernel, hint, hsearch,
                                                                  hsearch_out, status);
     return 1;
 }
@@ -814,23 +822,23 @@ int launch_gather(const Launch& L, int64_t n, const uint32_t* skeys, const uint3
 // positions, h and time state
 __global__ void __launch_bounds__(256) k_refresh_records(int64_t n, State s, const uint16_t* patch_of,
                                                          const PatchDev* pd, const uint32_t* cellxyz, Recs r,
-                                                         Fp64 f, int mixed)
+                                                         Fp64 f, int mixed, int kernel)
 {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const PatchDev* P = pd + patch_of[k];
         const uint32_t c = cellxyz[k];
         const double h = s.h[k];
         write_records(k, P, c & 255u, (c >> 8) & 255u, c >> 16, s.x[k], s.y[k], s.z[k], s.vx[k], s.vy[k], s.vz[k],
-                      s.m[k], h, s.u[k], s.axp[k], s.ayp[k], s.azp[k], (float)h, r, f, mixed);
+                      s.m[k], h, s.u[k], s.axp[k], s.ayp[k], s.azp[k], (float)h, r, f, mixed, kernel);
     }
 }
 
 int launch_refresh_records(const Launch& L, int64_t n, const State& s, const uint16_t* patch_of,
-                           const PatchDev* pd, const uint32_t* cellxyz, const Recs& r, const Fp64& f, int mixed)
+                           const PatchDev* pd, const uint32_t* cellxyz, const Recs& r, const Fp64& f, int mixed, int kernel)
 {
     if (n <= 0) return 0;
     k_refresh_records<<<blocks_for(n, 256, L.sms, 16), 256, 0, L.stream>>>(n, s, patch_of, pd, cellxyz, r, f,
-                                                                          mixed);
+                                                                          mixed, kernel);
     return 1;
 }
 
