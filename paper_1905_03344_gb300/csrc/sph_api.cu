@@ -87,6 +87,7 @@ struct sph_ctx {
     int npatch = 0, nitems = 0, radix_passes = 3;
     int tpp_pair = 8;              // lanes per particle of the momentum sum
     int tpp_den = 8;               // ... and of the density sum
+    bool tpp_auto = true;          // neither configured nor tuned: by default_tpp()
     // row-length bins of the pair sums: log2 of the list words per lane
     // (0: every particle with the uniform tpp above)
     int bins_pair = 0, bins_den = 0;
@@ -624,6 +625,23 @@ sph_status after_launches(sph_ctx* ctx, const char* where)
     return SPH_OK;
 }
 
+// Lanes per particle of the pair sums before any tuning.  A lane takes four
+// list words at a time and a row has about a hundred, so more lanes idle in
+// its last round and spend longer on the group's reduction; fewer leave SMs
+// without warps where there are few particles.  Mixed sums, density +
+// momentum in us for 2 / 4 / 8 / 16 / 32 lanes: 1728 particles 30 / 22 / 19 /
+// 17 / 17, 8000 31 / 23 / 22 / 25 / 30, 36k 41 / 41 / 47 / 56 / 73, 1 M 672 /
+// 698 / 837 / 1236 / 1780, 1 M of the irregular patch (rows of 50 to 400) 1538
+// / 1384 / 1380 / 1559 / 2029; so four, or enough for 50,000 lanes.  The FP64
+// sums keep eight, whose shorter chains round less.
+int default_tpp(int64_t n, int mixed)
+{
+    if (!mixed) return 8;
+    int t = 4;
+    while (t < 32 && n * t < 50000) t *= 2;
+    return t;
+}
+
 // patch table for the given original-order offsets (slots == original order)
 sph_status setup_patches(sph_ctx* ctx, int np, const int64_t* offsets)
 {
@@ -694,6 +712,7 @@ sph_status setup_patches(sph_ctx* ctx, int np, const int64_t* offsets)
     int bits = 0;
     while ((1 << bits) < np) bits++;
     ctx->radix_passes = (kPatchShift + bits + 7) / 8;
+    if (ctx->tpp_auto) ctx->tpp_pair = ctx->tpp_den = default_tpp(offsets[np], ctx->mixed);
     ctx->patch_off.assign(offsets, offsets + np + 1);
     ctx->nb_valid = ctx->rho_valid = ctx->acc_valid = ctx->sup_valid = false;
     ctx->cnt_valid = false;
@@ -848,6 +867,7 @@ sph_status sph_create(const sph_config* cfg_in, sph_ctx** out)
     ctx->cell_factor = cfg.cell_factor;
     ctx->cf_auto = cf_default;
     if (t) ctx->tpp_pair = ctx->tpp_den = t;
+    ctx->tpp_auto = t == 0;
     if (pb > 0) {
         int w = 0;
         while ((1 << w) < pb) w++;
@@ -1545,6 +1565,7 @@ sph_status sph_autotune(sph_ctx* ctx)
     cudaEventDestroy(e1);
     ctx->cell_factor = best_f;
     ctx->cf_auto = true;
+    ctx->tpp_auto = false;
     ctx->tpp_pair = best_pair;
     ctx->tpp_den = best_den;
     ctx->bins_pair = best_bpair;
