@@ -147,6 +147,7 @@ struct sph_ctx {
     int* status = nullptr;
     int* h_status = nullptr;     // pinned
     unsigned long long* pair_acc = nullptr;  // sum of |N| over the steps taken
+    unsigned* dt_ticket = nullptr; // blocks of the time-step kernel that are done
     std::vector<int64_t> patch_off;
 
     bool nb_valid = false, rho_valid = false, acc_valid = false;
@@ -347,7 +348,6 @@ PairArgs pair_args(sph_ctx* ctx)
     a.kernel_n = ctx->cfg.kernel_n;
     a.grad_h = ctx->cfg.grad_h;
     a.kb = ctx->kernel_b;
-    a.red = ctx->red;
     a.status = ctx->status;
     a.order = nullptr;
     a.bounds = nullptr;
@@ -380,6 +380,7 @@ StepArgs step_args(sph_ctx* ctx)
     a.status = ctx->status;
     a.listed = ctx->pool_used + 1;
     a.pair_acc = ctx->pair_acc;
+    a.dt_ticket = ctx->dt_ticket;
     return a;
 }
 
@@ -557,10 +558,6 @@ bool reuse_lists(const sph_ctx* ctx) { return ctx->skin > 0.0 && !ctx->fused; }
 void enqueue_pair_phases(sph_ctx* ctx)
 {
     const Launch L = launch_of(ctx);
-    if (reuse_lists(ctx)) {
-        Phase p(ctx, SPH_PHASE_UPDATE);
-        ctx->launches += launch_hc_reset(L, step_args(ctx));
-    }
     enqueue_density(ctx);
     {
         Phase p(ctx, SPH_PHASE_UPDATE);
@@ -921,12 +918,12 @@ sph_status sph_create(const sph_config* cfg_in, sph_ctx** out)
     ok = ok && dalloc(ctx, ctx->rec.r4, N + 16);
     if (ctx->mixed) {
         ok = ok && dalloc(ctx, ctx->rec.r5, N) && dalloc(ctx, ctx->rec.rv, N) && dalloc(ctx, ctx->rec.rt, N) &&
-             dalloc(ctx, ctx->rec.pf, N) && dalloc(ctx, ctx->rec.uf, N) &&
+             dalloc(ctx, ctx->rec.hc, N) && dalloc(ctx, ctx->rec.pf, N) && dalloc(ctx, ctx->rec.uf, N) &&
              dalloc(ctx, ctx->rec.acc, N);
     } else {
         Fp64& f = ctx->f64;
-        double** g[16] = {&f.vhx, &f.vhy, &f.vhz, &f.rho, &f.P, &f.c, &f.A, &f.w, &f.g0, &f.g1, &f.ha, &f.ca, &f.ax, &f.ay, &f.az, &f.du};
-        for (int k = 0; k < 16 && ok; k++) ok = dalloc(ctx, *g[k], N);
+        double** g[17] = {&f.vhx, &f.vhy, &f.vhz, &f.rho, &f.P, &f.c, &f.A, &f.hc, &f.w, &f.g0, &f.g1, &f.ha, &f.ca, &f.ax, &f.ay, &f.az, &f.du};
+        for (int k = 0; k < 17 && ok; k++) ok = dalloc(ctx, *g[k], N);
     }
     ok = ok && dalloc(ctx, ctx->bin_order, N) && dalloc(ctx, ctx->bin_bounds, (size_t)kPairOctaves + 1);
     ok = ok && dalloc(ctx, ctx->cnt, N) && dalloc(ctx, ctx->cnt_orig, N) && dalloc(ctx, ctx->nown, N) &&
@@ -949,7 +946,7 @@ sph_status sph_create(const sph_config* cfg_in, sph_ctx** out)
         if (ok && cudaMallocHost(&ctx->h_skin_flag, sizeof(int)) != cudaSuccess) ok = false;
     }
     ctx->grid.patch_of = ctx->patch_of;
-    ok = ok && dalloc(ctx, ctx->cf_vote, 2);
+    ok = ok && dalloc(ctx, ctx->cf_vote, 2) && dalloc(ctx, ctx->dt_ticket, 1);
     if (ok && cudaMallocHost(&ctx->h_cf_vote, 2 * sizeof(unsigned long long)) != cudaSuccess) ok = false;
     if (ok && cudaMallocHost(&ctx->h_status, sizeof(int)) != cudaSuccess) ok = false;
     if (!ok) {
@@ -958,6 +955,7 @@ sph_status sph_create(const sph_config* cfg_in, sph_ctx** out)
     }
     cudaMemsetAsync(ctx->status, 0, sizeof(int), ctx->stream);
     cudaMemsetAsync(ctx->pair_acc, 0, sizeof(unsigned long long), ctx->stream);
+    cudaMemsetAsync(ctx->dt_ticket, 0, sizeof(unsigned), ctx->stream);
     {
         // R10: h <- h (1 + (n_target / n)^(1/3)) / 2, the factor for each count
         // below kHFacN in FP64 on the host

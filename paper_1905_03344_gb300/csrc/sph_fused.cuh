@@ -187,7 +187,6 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_DEN_MINB)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float kb8 = (float)(8.0 * pa.kb), gam = (float)pa.gamma;
     const PairSrc src = pair_src(pa);
-    HcMin<float> hc;
     for (int64_t q = (int64_t)blockIdx.x * kNbtWarps + warp; q < a.nunits; q += (int64_t)gridDim.x * kNbtWarps) {
         const WorkItem U = a.units[q];
         const PatchDev* P = a.pd + U.patch;
@@ -198,14 +197,13 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_DEN_MINB)
             DensSink<KERN, GH> s = {src, pair_side(pa, P, i), pa.r.rv[i].w, pa.kernel_n, P->zmode,
                                     0.0f, 0.0f, 0.0f, 0.0f, 0u, 0u};
             walk_all<DensSink<KERN, GH>>(a, P, i, big, s);
-            hc.add(pa.red, U.patch, density_finish<GH>(pa, i, s.I.ri.w, s.inv2h, kb8, gam, s.sum, s.comp, s.sumd, s.compd));
+            density_finish<GH>(pa, i, s.I.ri.w, s.inv2h, kb8, gam, s.sum, s.comp, s.sumd, s.compd);
             a.cnt[i] = s.cnt;
             a.nown[i] = s.own;
             cnt = s.cnt;
         }
         count_pairs(a, cnt);
     }
-    hc.flush(pa.red);
 }
 
 template <int KERN, bool GH>
@@ -242,7 +240,6 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_DEN_MINB)
 {
     if (*a.status & kStBad) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    HcMin<double> hc;
     for (int64_t q = (int64_t)blockIdx.x * kNbtWarps + warp; q < a.nunits; q += (int64_t)gridDim.x * kNbtWarps) {
         const WorkItem U = a.units[q];
         const PatchDev* P = a.pd + U.patch;
@@ -253,14 +250,13 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_DEN_MINB)
             DensSinkD<KERN, GH> s = {&pa, pa.s.x[i], pa.s.y[i], pa.s.z[i], pa.f.w[i], P->lz,
                                      pa.kernel_n, 0.0, 0.0, 0u, 0u};
             walk_all<DensSinkD<KERN, GH>>(a, P, i, big, s);
-            hc.add(pa.red, U.patch, density_finish_fp64<GH>(pa, i, s.sum, s.sumd));
+            density_finish_fp64<GH>(pa, i, s.sum, s.sumd);
             a.cnt[i] = s.cnt;
             a.nown[i] = s.own;
             cnt = s.cnt;
         }
         count_pairs(a, cnt);
     }
-    hc.flush(pa.red);
 }
 
 template <int KERN, bool GH>

@@ -143,6 +143,7 @@ struct Recs {             // FP32 records (written by gather / density)
     float4* r5;          // {ox, oy, oz, m}      pair sums (mixed)
     float4* rv;          // {vhx, vhy, vhz, 1/(2h)} time-centred velocity (mixed)
     float4* rt;          // {rho, P/rho^2, c, h} thermodynamics (mixed)
+    float* hc;           // h/c (mixed)
     float* pf;           // P (mixed)
     float* uf;           // u, staged by the gather (mixed)
     float4* acc;         // {ax, ay, az, du} (mixed)
@@ -150,7 +151,7 @@ struct Recs {             // FP32 records (written by gather / density)
 
 struct Fp64 {             // FP64-path fields
     double *vhx, *vhy, *vhz;   // time-centred velocity
-    double *rho, *P, *c, *A;
+    double *rho, *P, *c, *A, *hc;
     double *w;                 // 1/(2h)
     double *g0, *g1;           // of the kernel gradient's factor: w^(5/3) and
                                // w^(8/3) (Wendland), w^5 and w (Sinc)
@@ -231,6 +232,90 @@ __host__ __device__ __forceinline__ uint32_t compact1by2(uint32_t v)
     v = (v | (v >> 16)) & 0x000003FFu;
     return v;
 }
+
+#ifdef __CUDACC__
+// Sums of 7 per-thread values over a block of 256 threads, in a fixed order;
+// thread q < 7 returns sum q.  The lanes of a warp halve the values they hold
+// while they add (four, two and one of eight, then two plain steps): 9
+// additions on the FP64 pipe where a butterfly per value takes 35.
+__device__ __forceinline__ double block_sum7(const double (&v)[7], double (*sh)[8])
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+    double a[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const double hi = k < 3 ? v[k + 4] : 0.0;
+        a[k] = (h16 ? hi : v[k]) + __shfl_xor_sync(0xffffffffu, h16 ? v[k] : hi, 16);
+    }
+    double b[2];
+#pragma unroll
+    for (int k = 0; k < 2; k++) b[k] = (h8 ? a[k + 2] : a[k]) + __shfl_xor_sync(0xffffffffu, h8 ? a[k] : a[k + 2], 8);
+    double c = (h4 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h4 ? b[0] : b[1], 4);
+    c += __shfl_xor_sync(0xffffffffu, c, 2);
+    c += __shfl_xor_sync(0xffffffffu, c, 1);
+    const int q = (h16 ? 4 : 0) + (h8 ? 2 : 0) + (h4 ? 1 : 0);
+    if ((lane & 3) == 0 && q < 7) sh[q][warp] = c;
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x < 7)
+        for (int w = 0; w < 8; w++) s += sh[threadIdx.x][w];
+    __syncthreads();
+    return s;
+}
+
+// one particle's share of the conserved sums, accumulated with FMAs: M, P,
+// L_z = m (x v_y - y v_x), twice E_kin (to be halved), E_int
+__device__ __forceinline__ void cons_accum(double x, double y, double vx, double vy, double vz, double m,
+                                           double u, double (&acc)[7])
+{
+    acc[0] += m;
+    acc[1] = fma(m, vx, acc[1]);
+    acc[2] = fma(m, vy, acc[2]);
+    acc[3] = fma(m, vz, acc[3]);
+    acc[4] = fma(m, fma(x, vy, -y * vx), acc[4]);
+    acc[5] = fma(m, fma(vx, vx, fma(vy, vy, vz * vz)), acc[5]);
+    acc[6] = fma(m, u, acc[6]);
+}
+
+// s + c: a compensated sum (Neumaier)
+__device__ __forceinline__ void neumaier_add(double& s, double& c, double v)
+{
+    const double t = s + v;
+    if (fabs(s) >= fabs(v)) c += (s - t) + v;
+    else c += (v - t) + s;
+    s = t;
+}
+
+// Compensated sum of part[0], part[stride], ... part[(n - 1) stride] by a
+// block of 256 threads: thread t takes the terms t, t + 256, ... in order,
+// lane l of the first warp adds the sums of threads l, l + 32, ..., and lane 0
+// the 32 lane sums in lane order.  The order is fixed, so the result is
+// reproducible; thread 0 returns it.  Bound by the chain of dependent
+// additions and loads: one warp for the partials of 8 M particles took 32 us,
+// one thread for those of 2 M 150.
+__device__ __forceinline__ double block_neumaier(const double* part, int n, int stride, double* sh_s, double* sh_c)
+{
+    double s = 0.0, c = 0.0;
+    for (int k = threadIdx.x; k < n; k += 256) neumaier_add(s, c, part[(int64_t)k * stride]);
+    sh_s[threadIdx.x] = s;
+    sh_c[threadIdx.x] = c;
+    __syncthreads();
+    if (threadIdx.x >= 32) return 0.0;
+    for (int k = threadIdx.x + 32; k < 256; k += 32) {
+        neumaier_add(s, c, sh_s[k]);
+        c += sh_c[k];
+    }
+    double S = 0.0, C = 0.0;
+    for (int l = 0; l < 32; l++) {
+        const double sl = __shfl_sync(0xffffffffu, s, l);
+        const double cl = __shfl_sync(0xffffffffu, c, l);
+        neumaier_add(S, C, sl);
+        C += cl;
+    }
+    return S + C;
+}
+#endif
 
 // ---- launch wrappers (each returns the number of kernels launched) --------
 struct Launch {
@@ -337,7 +422,6 @@ struct PairArgs {
     int kernel, kernel_n;                // SPH_KERNEL_*; n of the Sinc kernel
     int grad_h;                          // 1: grad-h form (density stores A/Omega)
     double kb;                           // sigma_W (Wendland) or B_n (Sinc)
-    PatchRed* red;                       // hcmin: the density sum's minimum of h/c per patch
     int* status;
     // row-length bins (nullptr order: every particle, in sorted order): the
     // launch takes positions bounds[bin_lo] .. bounds[bin_hi + 1] of order,
@@ -393,10 +477,10 @@ struct StepArgs {
     int* status;
     const unsigned long long* listed;  // entries of this step's lists
     unsigned long long* pair_acc;      // ... summed over the steps
+    unsigned* dt_ticket;               // blocks of k_dt that are done (0 between steps)
 };
-// the minima of h/c afresh, for a density sum with no sort before it
-int launch_hc_reset(const Launch& L, const StepArgs& a);
-// the time-step of every patch, and the step's pairs added to pair_acc
+// the time-step of every patch from its smallest h/c, and the step's pairs
+// added to pair_acc
 int launch_dt(const Launch& L, const StepArgs& a);
 int launch_update(const Launch& L, const StepArgs& a);
 // reused candidate supersets: the state the superset was built on (sorted

@@ -579,51 +579,10 @@ __device__ __forceinline__ void density_pair(const PairSrc& src, const PairSide&
     density_term<KERN, GH>(dx, dy, dz, inv2h, kn, m, sum, comp, sumd, compd);
 }
 
-// The Courant condition's minimum of h/c per patch, kept by a thread over the
-// particles it finishes (whose patches come in runs) and added to the
-// patch's minimum by its warp when the thread is done.  A pass of its own
-// over the stored ratios took 38 us at 8 M particles.
-template <typename T>
-struct HcMin {
-    T v;
-    int patch = -1;
-    // (the minimum only falls: a value that is not below it needs no atomic)
-    static __device__ __forceinline__ void put(PatchRed* red, int p, unsigned long long o)
-    {
-        if (o < *(volatile unsigned long long*)&red[p].hcmin) atomicMin(&red[p].hcmin, o);
-    }
-    __device__ __forceinline__ void add(PatchRed* red, int p, T hc)
-    {
-        if (p != patch) {
-            if (patch >= 0) put(red, patch, ord_f64((double)v));
-            patch = p;
-            v = hc;
-        } else if (hc < v) {
-            v = hc;
-        }
-    }
-    // every lane of the warp
-    __device__ __forceinline__ void flush(PatchRed* red)
-    {
-        __syncwarp();
-        unsigned long long o = patch >= 0 ? ord_f64((double)v) : ~0ull;
-        const int p = __reduce_max_sync(0xffffffffu, patch);
-        if (__all_sync(0xffffffffu, patch == p || patch < 0)) {
-            for (int k = 16; k > 0; k >>= 1) {
-                const unsigned long long t = __shfl_xor_sync(0xffffffffu, o, k);
-                o = t < o ? t : o;
-            }
-            if ((threadIdx.x & 31) == 0 && p >= 0) put(red, p, o);
-        } else if (patch >= 0) {
-            put(red, patch, o);
-        }
-    }
-};
-
 // density epilogue of particle i: rho from the shape sum (self term m_i),
-// EOS, and the records the momentum sum reads; returns h/c
+// EOS, and the records the momentum sum reads
 template <bool GH>
-__device__ __forceinline__ float density_finish(const PairArgs& a, int64_t i, float mi, float inv2h, float kb8,
+__device__ __forceinline__ void density_finish(const PairArgs& a, int64_t i, float mi, float inv2h, float kb8,
                                                float gam, float sum, float comp, float sumd, float compd)
 {
     const float tot = mi + (sum - comp);                 // self term m_i W(0) ~ m_i
@@ -643,8 +602,8 @@ __device__ __forceinline__ float density_finish(const PairArgs& a, int64_t i, fl
     const float hf = 0.5f / inv2h;
     a.r.rt[i] = make_float4(rho, A, c, hf);
     a.r.pf[i] = Pr;
+    a.r.hc[i] = hf / c;
     if (!(rho > 0.0f) || !isfinite(rho) || !isfinite(Pr) || !isfinite(c)) atomicOr(a.status, kStNonFinite);
-    return hf / c;
 }
 
 #ifndef SPH_MOM_PACK
@@ -768,7 +727,7 @@ __device__ __forceinline__ void density_pair_fp64(const PairArgs& a, double xi, 
 }
 
 template <bool GH>
-__device__ __forceinline__ double density_finish_fp64(const PairArgs& a, int64_t i, double sum, double sumd)
+__device__ __forceinline__ void density_finish_fp64(const PairArgs& a, int64_t i, double sum, double sumd)
 {
     const double hi = a.s.h[i];
     const double rho = a.kb * (a.s.m[i] + sum) / (hi * hi * hi);
@@ -786,8 +745,8 @@ __device__ __forceinline__ double density_finish_fp64(const PairArgs& a, int64_t
         if (!(om > 0.0)) atomicOr(a.status, kStNonFinite);
     }
     a.f.A[i] = A;
+    a.f.hc[i] = hi / c;
     if (!(rho > 0.0) || !isfinite(rho) || !isfinite(Pr) || !isfinite(c)) atomicOr(a.status, kStNonFinite);
-    return hi / c;
 }
 
 // particle i's values for the FP64 momentum sum

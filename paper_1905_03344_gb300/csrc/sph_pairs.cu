@@ -142,13 +142,11 @@ __global__ void __launch_bounds__(256, SPH_DEN_MINB) k_density_mixed(PairArgs a)
     pair_range(a, kb, ke);
     const int64_t k0 = kb + ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / TPP;
     RowAhead ahead = row_ahead_read(a, pair_at(a, k0 + gs, ke));
-    HcMin<float> hc;
     for (int64_t k = k0; k < ke; k += gs) {
         const int64_t i = pair_at(a, k, ke);
         row_ahead_prefetch<TPP>(a, ahead, G.gl);
         ahead = row_ahead_read(a, pair_at(a, k + 2 * gs, ke));
-        const int patch = a.patch_of[i];
-        const PatchDev* P = a.pd + patch;
+        const PatchDev* P = a.pd + a.patch_of[i];
         const PairSide I = pair_side(a, P, i);
         const float inv2h = a.r.rv[i].w;                   // 1 / (2 h_i)
         const uint32_t* row = a.col + a.rowstart[i];
@@ -158,10 +156,8 @@ __global__ void __launch_bounds__(256, SPH_DEN_MINB) k_density_mixed(PairArgs a)
         else density_row<TPP, 0, KERN, GH>(a, row, len, G.gl, I, inv2h, sum, comp, sumd, compd);
         group_kahan_reduce<TPP>(sum, comp, G.gmask);
         if (GH) group_kahan_reduce<TPP>(sumd, compd, G.gmask);
-        if (G.gl == 0)
-            hc.add(a.red, patch, density_finish<GH>(a, i, I.ri.w, inv2h, kb8, gam, sum, comp, sumd, compd));
+        if (G.gl == 0) density_finish<GH>(a, i, I.ri.w, inv2h, kb8, gam, sum, comp, sumd, compd);
     }
-    hc.flush(a.red);
 }
 
 // ---------------------------------------------------------------------------
@@ -176,7 +172,6 @@ __global__ void __launch_bounds__(256) k_density_fp64(PairArgs a)
     const int64_t gs = ((int64_t)gridDim.x * blockDim.x) / TPP;
     int64_t kb, ke;
     pair_range(a, kb, ke);
-    HcMin<double> hc;
     // A group sums TPP particles, one after the other, before its lanes finish
     // one each: the epilogue's divisions and square root, some 60 operations on
     // the FP64 pipe, cost a warp the same for one lane as for all (125,000
@@ -203,9 +198,8 @@ __global__ void __launch_bounds__(256) k_density_fp64(PairArgs a)
                 sumd_i = sumd;
             }
         }
-        if (mine >= 0) hc.add(a.red, a.patch_of[mine], density_finish_fp64<GH>(a, mine, sum_i, sumd_i));
+        if (mine >= 0) density_finish_fp64<GH>(a, mine, sum_i, sumd_i);
     }
-    hc.flush(a.red);
 }
 
 // ---------------------------------------------------------------------------

@@ -15,82 +15,79 @@
 
 namespace sphg {
 
-__device__ __forceinline__ double warp_sum_d(double v)
-{
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// sum of 7 per-thread values over a block of 256 threads; result valid in thread 0
-__device__ __forceinline__ void block_sum7(double v[7], double (*sh)[8])
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int q = 0; q < 7; q++) v[q] = warp_sum_d(v[q]);
-    if (lane == 0)
-        for (int q = 0; q < 7; q++) sh[q][warp] = v[q];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int q = 0; q < 7; q++) {
-            double s = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); w++) s += sh[q][w];
-            v[q] = s;
-        }
-    }
-    __syncthreads();
-}
-
-// one particle's share of the conserved sums, accumulated with FMAs: M, P,
-// L_z = m (x v_y - y v_x), twice E_kin (halved once per work item), E_int
-__device__ __forceinline__ void cons_accum(double x, double y, double vx, double vy, double vz, double m,
-                                           double u, double acc[7])
-{
-    acc[0] += m;
-    acc[1] = fma(m, vx, acc[1]);
-    acc[2] = fma(m, vy, acc[2]);
-    acc[3] = fma(m, vz, acc[3]);
-    acc[4] = fma(m, fma(x, vy, -y * vx), acc[4]);
-    acc[5] = fma(m, fma(vx, vx, fma(vy, vy, vz * vz)), acc[5]);
-    acc[6] = fma(m, u, acc[6]);
-}
-
-// a step that reuses its lists runs no sort, whose reset would clear the
-// minima of h/c
-__global__ void k_hc_reset(PatchRed* red, int npatch)
-{
-    for (int p = threadIdx.x; p < npatch; p += blockDim.x) red[p].hcmin = ~0ull;
-}
-
-int launch_hc_reset(const Launch& L, const StepArgs& a)
-{
-    k_hc_reset<<<1, 256, 0, L.stream>>>(a.red, a.npatch);
-    return 1;
-}
-
 // ---- Courant time-step per patch ------------------------------------------
-__global__ void k_dt(StepArgs a)
+// The smallest h/c of every patch (one block per work item), and in the last
+// block to finish the time-steps; it leaves the minima cleared for the next
+// step, whether that one sorts or reuses its lists.  (The same minimum kept
+// in registers by the density sums, which run at their register limit, took
+// 2 to 4 % of their time.)
+__global__ void __launch_bounds__(256) k_dt(StepArgs a)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= a.npatch || (*a.status & kStBad)) return;
-    if (p == 0) *a.pair_acc += *a.listed;
-    PatchDev* P = a.pd + p;
-    if (P->end <= P->begin) {
-        P->dt = 0.0;
-        return;
+    __shared__ unsigned long long sh[8];
+    __shared__ bool last;
+    if (*a.status & kStBad) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
+        const WorkItem w = a.items[it];
+        unsigned long long mn = ~0ull;
+        if (a.mixed) {
+            // (as floats first: two conversions a thread on the FP64 pipe)
+            float v = __int_as_float(0x7f800000);
+#pragma unroll 4
+            for (int64_t i = w.begin + threadIdx.x; i < w.end; i += blockDim.x) v = fminf(v, a.r.hc[i]);
+            mn = ord_f64((double)v);
+        } else {
+            for (int64_t i = w.begin + threadIdx.x; i < w.end; i += blockDim.x) {
+                const unsigned long long o = ord_f64(a.f.hc[i]);
+                mn = o < mn ? o : mn;
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long t = __shfl_xor_sync(0xffffffffu, mn, o);
+            mn = t < mn ? t : mn;
+        }
+        if (lane == 0) sh[warp] = mn;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int ww = 1; ww < (int)(blockDim.x >> 5); ww++) mn = sh[ww] < mn ? sh[ww] : mn;
+            atomicMin(&a.red[w.patch].hcmin, mn);
+        }
+        __syncthreads();
     }
-    double dt;
-    if (a.dt_fixed > 0.0) {
-        dt = a.dt_fixed;
-    } else {
-        dt = a.courant * unord_f64(a.red[p].hcmin);
-        if (P->step > 0 && a.dt_growth * P->dt_prev < dt) dt = a.dt_growth * P->dt_prev;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(a.dt_ticket, 1u) == gridDim.x - 1u;
     }
-    if (!(dt > 0.0) || !isfinite(dt)) atomicOr(a.status, kStNonFinite);
-    P->dt = dt;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (threadIdx.x == 0) {
+        *a.dt_ticket = 0u;
+        *a.pair_acc += *a.listed;
+    }
+    for (int p = threadIdx.x; p < a.npatch; p += blockDim.x) {
+        PatchDev* P = a.pd + p;
+        const unsigned long long hcmin = atomicExch(&a.red[p].hcmin, ~0ull);
+        if (P->end <= P->begin) {
+            P->dt = 0.0;
+            continue;
+        }
+        double dt;
+        if (a.dt_fixed > 0.0) {
+            dt = a.dt_fixed;
+        } else {
+            dt = a.courant * unord_f64(hcmin);
+            if (P->step > 0 && a.dt_growth * P->dt_prev < dt) dt = a.dt_growth * P->dt_prev;
+        }
+        if (!(dt > 0.0) || !isfinite(dt)) atomicOr(a.status, kStNonFinite);
+        P->dt = dt;
+    }
 }
 
 int launch_dt(const Launch& L, const StepArgs& a)
 {
-    k_dt<<<(a.npatch + 127) / 128, 128, 0, L.stream>>>(a);
+    const int cap = L.sms * 8;
+    k_dt<<<a.nitems < 1 ? 1 : (a.nitems < cap ? a.nitems : cap), 256, 0, L.stream>>>(a);
     return 1;
 }
 
@@ -144,9 +141,8 @@ __global__ void __launch_bounds__(256) k_update(StepArgs a)
             cons_accum(x, y, vx, vy, vz, a.s.m[i], u, acc);
         }
         acc[5] *= 0.5;
-        block_sum7(acc, sh);
-        if (threadIdx.x == 0)
-            for (int q = 0; q < 7; q++) a.partials[(int64_t)it * 7 + q] = acc[q];
+        const double sum = block_sum7(acc, sh);
+        if (threadIdx.x < 7) a.partials[(int64_t)it * 7 + threadIdx.x] = sum;
     }
 }
 
@@ -167,9 +163,8 @@ __global__ void __launch_bounds__(256) k_conserved_items(StepArgs a)
         for (int64_t i = w.begin + threadIdx.x; i < w.end; i += blockDim.x)
             cons_accum(a.s.x[i], a.s.y[i], a.s.vx[i], a.s.vy[i], a.s.vz[i], a.s.m[i], a.s.u[i], acc);
         acc[5] *= 0.5;
-        block_sum7(acc, sh);
-        if (threadIdx.x == 0)
-            for (int q = 0; q < 7; q++) a.partials[(int64_t)it * 7 + q] = acc[q];
+        const double sum = block_sum7(acc, sh);
+        if (threadIdx.x < 7) a.partials[(int64_t)it * 7 + threadIdx.x] = sum;
     }
 }
 
@@ -181,20 +176,8 @@ int launch_conserved_items(const Launch& L, const StepArgs& a)
     return 1;
 }
 
-__device__ __forceinline__ void neumaier_add(double& s, double& c, double v)
-{
-    const double t = s + v;
-    if (fabs(s) >= fabs(v)) c += (s - t) + v;
-    else c += (v - t) + s;
-    s = t;
-}
-
-// One block per (patch, quantity): thread t takes the item partials t, t + 256,
-// ... in order with a compensated sum; lane l of the first warp adds the sums
-// of threads l, l + 32, ..., and lane 0 the 32 lane sums in lane order.  The
-// order is fixed, so the result is reproducible.  Bound by the chain of
-// dependent additions: with one warp for all partials it took 32 us at 8 M
-// particles.  With advance != 0 (after an update) it also closes the step.
+// One block per (patch, quantity).  With advance != 0 (after an update) it
+// also closes the step.
 __global__ void __launch_bounds__(256) k_conserved_finalize(StepArgs a, int advance)
 {
     __shared__ double sh_s[256], sh_c[256];
@@ -203,25 +186,9 @@ __global__ void __launch_bounds__(256) k_conserved_finalize(StepArgs a, int adva
     const int p = t / 7, q = t % 7;
     PatchDev* P = a.pd + p;
     if (advance && (*a.status & kStBad)) return;
-    double s = 0.0, c = 0.0;
-    for (int it = P->item_begin + threadIdx.x; it < P->item_end; it += 256) neumaier_add(s, c, a.partials[(int64_t)it * 7 + q]);
-    sh_s[threadIdx.x] = s;
-    sh_c[threadIdx.x] = c;
-    __syncthreads();
-    if (threadIdx.x >= 32) return;
-    for (int k = threadIdx.x + 32; k < 256; k += 32) {
-        neumaier_add(s, c, sh_s[k]);
-        c += sh_c[k];
-    }
-    double S = 0.0, C = 0.0;
-    for (int l = 0; l < 32; l++) {
-        const double sl = __shfl_sync(0xffffffffu, s, l);
-        const double cl = __shfl_sync(0xffffffffu, c, l);
-        neumaier_add(S, C, sl);
-        C += cl;
-    }
+    const double sum = block_neumaier(a.partials + (int64_t)P->item_begin * 7 + q, P->item_end - P->item_begin, 7, sh_s, sh_c);
     if (threadIdx.x == 0) {
-        a.cons[p * 7 + q] = S + C;
+        a.cons[p * 7 + q] = sum;
         if (advance && q == 0) {
             P->dt_prev = P->dt;
             P->step += 1;
