@@ -240,104 +240,156 @@ __device__ __forceinline__ uint32_t stencil_code(const PatchDev* P, int dcx, int
 // (unchanged: its cells are 1.3 times as wide).  Slower: lanes that leave the
 // lockstep of the rows for their own runs (L1 77-90 % busy), hits without
 // branches, ids loaded only for hits, groups of 3 or 5.
+//
+// what the rows of one particle's walk share
+struct RowCtx {
+    float s_f, sz_f, lz_f, inv_lz, inv_s;
+    int ncx, ncy, ncz, cx, cy, cz, zmode;
+    uint32_t cbase, i32;
+    float xi, xs, yi, zi, Ti, flo, fhi, Rg2;
+    int xlo, xhi, ylo, yhi, kz, nz;
+    bool coded;                         // every offset has a stencil code (the usual case)
+};
+
+template <int ZW>
+__device__ __forceinline__ RowCtx row_ctx(const NbArgs& a, const PatchDev* P, int64_t i, int kx, int kz, float Rg2)
+{
+    RowCtx c;
+    const float4 ri = a.r4[i];
+    const uint32_t cc = a.g.cellxyz[i];
+    c.s_f = P->s_f;
+    c.sz_f = P->sz_f;
+    c.lz_f = P->lz_f;
+    c.inv_lz = 1.0f / P->lz_f;
+    c.inv_s = P->inv_s_f;
+    c.ncx = P->ncx;
+    c.ncy = P->ncy;
+    c.ncz = P->ncz;
+    c.zmode = P->zmode;
+    c.cbase = (uint32_t)P->cell_base;
+    c.i32 = (uint32_t)i;
+    c.cx = cc & 255;
+    c.cy = (cc >> 8) & 255;
+    c.cz = cc >> 16;
+    c.Ti = ri.w;
+    // every z cell visited (ZW): shifts of up to ncz - 1 cells along z
+    const float tol = row_tol(c.s_f / (float)a.h[i], ZW ? max(kx, c.ncz) : max(kx, kz));
+    c.flo = 1.0f - tol;
+    c.fhi = 1.0f + tol;
+    c.Rg2 = Rg2;
+    c.xi = fmaf((float)c.cx, c.s_f, ri.x);
+    c.xs = c.xi * c.inv_s;
+    c.yi = ri.y;
+    c.zi = ri.z;
+    c.xlo = max(c.cx - kx, 0);
+    c.xhi = min(c.cx + kx, c.ncx - 1);
+    c.ylo = max(-kx, -c.cy);
+    c.yhi = min(kx, c.ncy - 1 - c.cy);
+    c.kz = kz;
+    c.nz = ZW ? c.ncz : 2 * kz + 1;
+    c.coded = kx <= 2 && (ZW ? c.zmode && c.ncz <= 5 : kz <= 2);
+    return c;
+}
+
+// the z plane iz of the walk
+struct RowPlane {
+    int czj, zd;
+    float zo, gz2;
+};
+
+template <int ZW>
+__device__ __forceinline__ RowPlane row_plane(const RowCtx& c, int iz)
+{
+    RowPlane p;
+    float zsh;
+    p.gz2 = 0.0f;
+    if (!ZW) {
+        const int dcz = iz - c.kz;
+        p.czj = c.cz + dcz;
+        if (p.czj < 0) p.czj += c.ncz;
+        else if (p.czj >= c.ncz) p.czj -= c.ncz;
+        zsh = (float)dcz * c.sz_f;
+        const float gz = fmaxf(dcz > 0 ? zsh - c.zi : (dcz < 0 ? c.zi - (zsh + c.sz_f) : 0.0f), 0.0f);
+        p.gz2 = gz * gz;
+        p.zd = dcz + 2;
+    } else {
+        p.czj = c.cz + iz;
+        if (p.czj >= c.ncz) p.czj -= c.ncz;
+        zsh = (float)iz * c.sz_f;
+        p.zd = c.zmode ? iz : 5;
+    }
+    p.zo = c.zi - zsh;
+    return p;
+}
+
+// the row dcy of plane p: its run of the row copy, tested
+template <class S, int ZW>
+__device__ __forceinline__ void walk_row(const NbArgs& a, const PatchDev* P, int64_t i, const RowCtx& c, const RowPlane& p,
+                                         int dcy, S& row)
+{
+    const float ysh = (float)dcy * c.s_f;
+    const float gy = fmaxf(dcy > 0 ? ysh - c.yi : (dcy < 0 ? c.yi - (ysh + c.s_f) : 0.0f), 0.0f);
+    const float rem2 = c.Rg2 - fmaf(gy, gy, p.gz2);
+    if (!(rem2 > 0.0f)) return;
+    // the chord, in cells (Rg's margins cover the rounding and the FP32 cell
+    // assignment)
+    const float half = __fsqrt_rn(rem2) * c.inv_s;
+    const int x0 = max((int)floorf(c.xs - half), c.xlo), x1 = min((int)floorf(c.xs + half), c.xhi);
+    if (x0 > x1) return;
+    const uint32_t lrow = c.cbase + ((uint32_t)p.czj * (uint32_t)c.ncy + (uint32_t)(c.cy + dcy)) * (uint32_t)c.ncx;
+    const uint32_t kb = a.g.row[lrow + (uint32_t)x0].x, ke = a.g.row[lrow + (uint32_t)x1].y;
+    const float yo = c.yi - ysh;
+    const bool rowcode = (uint32_t)(dcy + 2) <= 4u && (uint32_t)p.zd <= 4u;
+    // row_id + add: the column word where the code exists
+    const uint32_t add = (uint32_t)(2 + 5 * (dcy + 2) + 25 * p.zd - c.cx) << kColBits;
+    // kGroup candidates per iteration: their loads are in flight together (the
+    // row copy is padded past its end, so a group may read past the run; those
+    // slots are masked)
+#pragma unroll 1
+    for (uint32_t k = kb; k < ke; k += kGroup) {
+        const float4* qp = a.g.row_rec + k;
+        const uint32_t* ip = a.g.row_id + k;
+        float4 q[kGroup];
+        uint32_t id[kGroup];
+#pragma unroll
+        for (int u = 0; u < kGroup; u++) q[u] = qp[u];
+#pragma unroll
+        for (int u = 0; u < kGroup; u++) id[u] = ip[u];
+        const uint32_t rem = ke - k;
+        float r2[kGroup], T[kGroup];
+        unsigned near = 0;
+#pragma unroll
+        for (int u = 0; u < kGroup; u++) {
+            const float dx = c.xi - q[u].x, dy = yo - q[u].y;
+            float dz = p.zo - q[u].z;
+            if (ZW) dz = fmaf(-c.lz_f, rintf(dz * c.inv_lz), dz);
+            r2[u] = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+            T[u] = fmaxf(c.Ti, q[u].w);
+            if ((uint32_t)u < rem && r2[u] <= T[u] * c.fhi) near |= 1u << u;
+        }
+        if (!near) continue;
+        const uint32_t c0 = row.mark();
+#pragma unroll
+        for (int u = 0; u < kGroup; u++) {
+            if (!(near & (1u << u))) continue;
+            const uint32_t j = id[u] & kColMask;
+            if (j == c.i32) continue;
+            uint32_t w = id[u] + add;
+            if (!c.coded && !(rowcode && (id[u] >> kColBits) - (uint32_t)(c.cx - 2) <= 4u)) w = j | (kFarCode << kColBits);
+            row.decide(a, P, i, j, r2[u], c.Ti, T[u], c.flo, c.fhi, w);
+        }
+        row.group_end(c0);
+    }
+}
+
 template <class S, int ZW>
 __device__ __forceinline__ void walk_rows(const NbArgs& a, const PatchDev* P, int64_t i, int kx, int kz, float Rg2, S& row)
 {
-    const float s_f = P->s_f, sz_f = P->sz_f, lz_f = P->lz_f, inv_lz = 1.0f / P->lz_f;
-    const int ncx = P->ncx, ncy = P->ncy, ncz = P->ncz;
-    const uint32_t cbase = (uint32_t)P->cell_base;
-    const uint32_t i32 = (uint32_t)i;
-    const float4 ri = a.r4[i];
-    const uint32_t cc = a.g.cellxyz[i];
-    const int cx = cc & 255, cy = (cc >> 8) & 255, cz = cc >> 16;
-    const float hf = (float)a.h[i];
-    const float Ti = ri.w;
-    // every z cell visited (ZW): shifts of up to ncz - 1 cells along z
-    const float tol = row_tol(s_f / hf, ZW ? max(kx, ncz) : max(kx, kz));
-    const float flo = 1.0f - tol, fhi = 1.0f + tol;
-    const float xi = fmaf((float)cx, s_f, ri.x);
-    const float xs = xi * P->inv_s_f;
-    const int xlo = max(cx - kx, 0), xhi = min(cx + kx, ncx - 1);
-    const int ylo = max(-kx, -cy), yhi = min(kx, ncy - 1 - cy);
-    const int nz = ZW ? ncz : 2 * kz + 1;
-    // every offset has a stencil code (the usual case)
-    const bool coded = kx <= 2 && (ZW ? P->zmode && ncz <= 5 : kz <= 2);
-    for (int iz = 0; iz < nz; iz++) {
-        int czj, zd;
-        float zsh, gz2 = 0.0f;
-        if (!ZW) {
-            const int dcz = iz - kz;
-            czj = cz + dcz;
-            if (czj < 0) czj += ncz;
-            else if (czj >= ncz) czj -= ncz;
-            zsh = (float)dcz * sz_f;
-            const float gz = fmaxf(dcz > 0 ? zsh - ri.z : (dcz < 0 ? ri.z - (zsh + sz_f) : 0.0f), 0.0f);
-            gz2 = gz * gz;
-            if (gz2 >= Rg2) continue;
-            zd = dcz + 2;
-        } else {
-            czj = cz + iz;
-            if (czj >= ncz) czj -= ncz;
-            zsh = (float)iz * sz_f;
-            zd = P->zmode ? iz : 5;
-        }
-        const float zo = ri.z - zsh;
-        const uint32_t lplane = cbase + (uint32_t)czj * (uint32_t)ncy * (uint32_t)ncx;
-        for (int dcy = ylo; dcy <= yhi; dcy++) {
-            const float ysh = (float)dcy * s_f;
-            const float gy = fmaxf(dcy > 0 ? ysh - ri.y : (dcy < 0 ? ri.y - (ysh + s_f) : 0.0f), 0.0f);
-            const float rem2 = Rg2 - fmaf(gy, gy, gz2);
-            if (!(rem2 > 0.0f)) continue;
-            // the chord, in cells (Rg's margins cover the rounding and the
-            // FP32 cell assignment)
-            const float half = __fsqrt_rn(rem2) * P->inv_s_f;
-            const int x0 = max((int)floorf(xs - half), xlo), x1 = min((int)floorf(xs + half), xhi);
-            if (x0 > x1) continue;
-            const uint32_t lrow = lplane + (uint32_t)(cy + dcy) * (uint32_t)ncx;
-            const uint32_t kb = a.g.row[lrow + (uint32_t)x0].x, ke = a.g.row[lrow + (uint32_t)x1].y;
-            const float yo = ri.y - ysh;
-            const bool rowcode = (uint32_t)(dcy + 2) <= 4u && (uint32_t)zd <= 4u;
-            // row_id + add: the column word where the code exists
-            const uint32_t add = (uint32_t)(2 + 5 * (dcy + 2) + 25 * zd - cx) << kColBits;
-            // kGroup candidates per iteration: their loads are in flight
-            // together (the row copy is padded past its end, so a group may
-            // read past the run; those slots are masked)
-#pragma unroll 1
-            for (uint32_t k = kb; k < ke; k += kGroup) {
-                const float4* qp = a.g.row_rec + k;
-                const uint32_t* ip = a.g.row_id + k;
-                float4 q[kGroup];
-                uint32_t id[kGroup];
-#pragma unroll
-                for (int u = 0; u < kGroup; u++) q[u] = qp[u];
-#pragma unroll
-                for (int u = 0; u < kGroup; u++) id[u] = ip[u];
-                const uint32_t rem = ke - k;
-                float r2[kGroup], T[kGroup];
-                unsigned near = 0;
-#pragma unroll
-                for (int u = 0; u < kGroup; u++) {
-                    const float dx = xi - q[u].x, dy = yo - q[u].y;
-                    float dz = zo - q[u].z;
-                    if (ZW) dz = fmaf(-lz_f, rintf(dz * inv_lz), dz);
-                    r2[u] = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                    T[u] = fmaxf(Ti, q[u].w);
-                    if ((uint32_t)u < rem && r2[u] <= T[u] * fhi) near |= 1u << u;
-                }
-                if (!near) continue;
-                const uint32_t c0 = row.mark();
-#pragma unroll
-                for (int u = 0; u < kGroup; u++) {
-                    if (!(near & (1u << u))) continue;
-                    const uint32_t j = id[u] & kColMask;
-                    if (j == i32) continue;
-                    uint32_t w = id[u] + add;
-                    if (!coded && !(rowcode && (id[u] >> kColBits) - (uint32_t)(cx - 2) <= 4u)) w = j | (kFarCode << kColBits);
-                    row.decide(a, P, i, j, r2[u], Ti, T[u], flo, fhi, w);
-                }
-                row.group_end(c0);
-            }
-        }
+    const RowCtx c = row_ctx<ZW>(a, P, i, kx, kz, Rg2);
+    for (int iz = 0; iz < c.nz; iz++) {
+        const RowPlane p = row_plane<ZW>(c, iz);
+        if (p.gz2 >= Rg2) continue;
+        for (int dcy = c.ylo; dcy <= c.yhi; dcy++) walk_row<S, ZW>(a, P, i, c, p, dcy, row);
     }
 }
 

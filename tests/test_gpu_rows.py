@@ -2,6 +2,8 @@
 cells (x far from the grid's origin), particles on cell faces, cells of many
 particles, rows of one cell, and few z cells -- lists and n_i against the
 oracle, bit for bit."""
+import os
+
 import numpy as np
 import pytest
 
@@ -20,9 +22,8 @@ def B():
     return binding
 
 
-def _cloud(kind):
+def _cloud(kind, n):
     rng = np.random.default_rng(11)
-    n = 6000
     z = rng.uniform(-0.5, 0.5, n)
     if kind == "long_x":         # 128 cells along x, few along y
         x, y, h = rng.uniform(0.0, 12.0, n), rng.uniform(-0.1, 0.1, n), rng.uniform(0.03, 0.045, n)
@@ -42,22 +43,25 @@ def _cloud(kind):
         h[::97] = rng.uniform(0.15, 0.3, len(h[::97]))
     else:                        # few_z: h so large that every z cell is visited
         x, y, h = rng.uniform(-2.0, 2.0, n), rng.uniform(-2.0, 2.0, n), rng.uniform(0.14, 0.17, n)
+    if kind not in ("faces", "few_z"):
+        h = h * (6000.0 / n) ** (1.0 / 3.0)
     v = np.zeros(n)
     return {"x": x, "y": y, "z": z, "vx": v, "vy": v, "vz": v, "m": np.full(n, 1.0 / n), "h": h, "u": np.ones(n)}
 
 
-@pytest.mark.parametrize("cf", [0.0, 0.4, 1.0])
+# 6000 particles are searched by teams of lanes, 56000 by a thread each
+@pytest.mark.parametrize("n,cf", [(6000, 0.0), (6000, 0.4), (6000, 1.0), (56000, 0.0), (56000, 0.4)])
 @pytest.mark.parametrize("kind", ["long_x", "long_y", "faces", "clump", "big_reach", "few_z"])
-def test_rows(B, orc, kind, cf):
-    f = _cloud(kind)
-    n = len(f["x"])
+def test_rows(B, orc, kind, n, cf):
+    f = _cloud(kind, n)
     sim = B.SPH(n, cell_factor=cf, max_pairs=800 * n)
     sim.set_particles(f)
+    nb = None
     for _ in range(2):           # rows counted first, then reserved from hints
         sim.find_neighbors()
         off, col, perm = sim.neighbors()
         o, c = lists_to_original(off, col, perm, n)
-        nb = orc.neighbors(f["x"], f["y"], f["z"], f["h"], 1.0)
+        nb = nb or orc.neighbors(f["x"], f["y"], f["z"], f["h"], 1.0, nthreads=os.cpu_count() or 1)
         assert np.array_equal(o, nb.off) and np.array_equal(c, nb.col)
         assert np.array_equal(sim.field("nown").astype(np.int64), nb.nown)
     sim.close()
