@@ -298,16 +298,18 @@ __device__ __forceinline__ double block_neumaier(const double* part, int n, int 
 {
     double s = 0.0, c = 0.0;
     for (int k = threadIdx.x; k < n; k += 256) neumaier_add(s, c, part[(int64_t)k * stride]);
-    sh_s[threadIdx.x] = s;
-    sh_c[threadIdx.x] = c;
-    __syncthreads();
+    if (n > 32) {                       // (no term beyond the first warp otherwise)
+        sh_s[threadIdx.x] = s;
+        sh_c[threadIdx.x] = c;
+        __syncthreads();
+    }
     if (threadIdx.x >= 32) return 0.0;
-    for (int k = threadIdx.x + 32; k < 256; k += 32) {
+    for (int k = threadIdx.x + 32; k < 256 && k < n; k += 32) {
         neumaier_add(s, c, sh_s[k]);
         c += sh_c[k];
     }
     double S = 0.0, C = 0.0;
-    for (int l = 0; l < 32; l++) {
+    for (int l = 0; l < 32 && l < n; l++) {
         const double sl = __shfl_sync(0xffffffffu, s, l);
         const double cl = __shfl_sync(0xffffffffu, c, l);
         neumaier_add(S, C, sl);
