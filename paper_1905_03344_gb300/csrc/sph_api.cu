@@ -39,12 +39,6 @@ bool is_sticky(cudaError_t e)
     }
 }
 
-__global__ void k_iota(int64_t n, uint32_t* p)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = (uint32_t)i;
-}
-
 // dst[perm[k]] = src[k]: a sorted-order array back to the caller's order
 __global__ void k_scatter_u32(int64_t n, const uint32_t* src, const uint32_t* perm, uint32_t* dst)
 {
@@ -606,10 +600,12 @@ sph_status check_status(sph_ctx* ctx, const char* where)
     return SPH_OK;
 }
 
-sph_status begin_call(sph_ctx* ctx)
+// clear: whether the call's kernels report through the status word
+sph_status begin_call(sph_ctx* ctx, bool clear = true)
 {
     if (!ctx) return fail(nullptr, SPH_EINVAL, "null context");
     if (ctx->poisoned) return fail(ctx, SPH_ESTATE, "context poisoned by an earlier CUDA error");
+    if (!clear) return SPH_OK;
     cudaError_t e = cudaMemsetAsync(ctx->status, 0, sizeof(int), ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "status reset");
     return SPH_OK;
@@ -1000,15 +996,19 @@ sph_status sph_set_particles(sph_ctx* ctx, int64_t n, const double* x, const dou
     }
     ctx->cur = 0;
     State& s = ctx->st[0];
-    const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    for (int k = 0; k < 9; k++)
-        if (n > 0) CK(cudaMemcpyAsync(state_field(s, k), src[k], (size_t)n * 8, kind, ctx->stream));
-    for (int k = 9; k < 13; k++) CK(cudaMemsetAsync(state_field(s, k), 0, (size_t)(n > 0 ? n : 1) * 8, ctx->stream));
+    // device arrays (of aligned doubles) are copied and checked in one pass;
+    // others are copied first and checked where they land
+    bool direct = on_device && n > 0;
+    for (int k = 0; k < 9; k++) direct = direct && (uintptr_t)src[k] % sizeof(double) == 0;
     ctx->n = n;
-    if (n > 0) {
-        const int grid = (int)((n + 255) / 256 < ctx->sms * 16 ? (n + 255) / 256 : ctx->sms * 16);
-        k_iota<<<grid, 256, 0, ctx->stream>>>(n, ctx->perm[0]);
-        launch_validate(launch_of(ctx), n, s, ctx->status);
+    if (direct) {
+        launch_load(launch_of(ctx), n, src, s, ctx->perm[0], ctx->status);
+    } else {
+        const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+        for (int k = 0; k < 9; k++)
+            if (n > 0) CK(cudaMemcpyAsync(state_field(s, k), src[k], (size_t)n * 8, kind, ctx->stream));
+        const double* own[9] = {s.x, s.y, s.z, s.vx, s.vy, s.vz, s.m, s.h, s.u};
+        if (n > 0) launch_load(launch_of(ctx), n, own, s, ctx->perm[0], ctx->status);
     }
     int64_t offs[2] = {0, n};
     st = setup_patches(ctx, 1, offs);
@@ -1115,6 +1115,19 @@ sph_status sph_get_neighbors(sph_ctx* ctx, const uint64_t** off, const uint32_t*
 
 sph_status sph_copy_neighbors(sph_ctx* ctx, uint64_t* off, uint32_t* col, uint32_t* perm, int on_device)
 {
+    if (on_device && ctx && !ctx->poisoned && ctx->nb_valid && !ctx->canon_valid && off && col && perm &&
+        (uintptr_t)off % sizeof(uint64_t) == 0 && (uintptr_t)col % sizeof(uint32_t) == 0) {
+        // the rows straight into the caller's buffers
+        sph_status st = begin_call(ctx);
+        if (st != SPH_OK) return st;
+        const Launch L = launch_of(ctx);
+        ctx->launches += launch_scan_u32_to_u64(L, ctx->n, ctx->cnt, off, ctx->scan64);
+        ctx->launches += launch_canonical_rows(L, ctx->n, ctx->rowstart, ctx->cnt, off, ctx->col, col);
+        if (ctx->n > 0)
+            CK(cudaMemcpyAsync(perm, ctx->perm[ctx->cur], sizeof(uint32_t) * ctx->n, cudaMemcpyDeviceToDevice, ctx->stream));
+        CK(cudaStreamSynchronize(ctx->stream));
+        return after_launches(ctx, "sph_copy_neighbors");
+    }
     const uint64_t* o = nullptr;
     const uint32_t *c = nullptr, *pm = nullptr;
     int64_t nnz = 0;
@@ -1275,7 +1288,7 @@ sph_status sph_conserved(sph_ctx* ctx, int32_t patch, double out[7])
 
 sph_status sph_get_field(sph_ctx* ctx, int32_t field, double* dst, int on_device)
 {
-    sph_status st = begin_call(ctx);
+    sph_status st = begin_call(ctx, false);
     if (st != SPH_OK) return st;
     if (field < 0 || field >= SPH_FIELD_COUNT) return fail(ctx, SPH_EINVAL, "unknown field");
     if (!dst && ctx->n > 0) return fail(ctx, SPH_EINVAL, "dst is NULL");

@@ -508,7 +508,9 @@ int launch_unpermute_f32(const Launch& L, int64_t n, const float* src, int strid
                          const uint32_t* perm, double* dst);
 int launch_unpermute_u32(const Launch& L, int64_t n, const uint32_t* src, const uint32_t* perm,
                          double* dst);
-int launch_validate(const Launch& L, int64_t n, const State& s, int* status);
+// new particles: src (x y z vx vy vz m h u; may be s's own arrays) into s, the
+// time fields cleared, perm the identity; status: kStNonFinite for bad values
+int launch_load(const Launch& L, int64_t n, const double* const src[9], const State& s, uint32_t* perm, int* status);
 int launch_reset_red(const Launch& L, int npatch, PatchRed* red, uint32_t* zero, int64_t words);
 
 }  // namespace sphg
