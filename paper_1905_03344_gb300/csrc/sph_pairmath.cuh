@@ -137,16 +137,23 @@ __device__ __forceinline__ void rel_dx(const float4& e, float s_f, float sz_f, f
 constexpr float kPif = 3.14159265358979323846f;
 constexpr double kPi = 3.14159265358979323846;
 
-__device__ __forceinline__ float ipowf(float b, int e)
+// b^e for 1 <= e <= 16 by squaring (e is the same for all threads): a loop of
+// e multiplications took the Sinc sums a seventh of their instructions
+template <typename T>
+__device__ __forceinline__ T ipow(T b, int e)
 {
-    float r = 1.0f;
-    for (int k = 0; k < e; k++) r *= b;
-    return r;
-}
-__device__ __forceinline__ double ipowd(double b, int e)
-{
-    double r = 1.0;
-    for (int k = 0; k < e; k++) r *= b;
+    T r = e & 1 ? b : T(1);
+    T p = b * b;
+    if (e & 2) r *= p;
+    if (e >= 4) {
+        p *= p;
+        if (e & 4) r *= p;
+        if (e >= 8) {
+            p *= p;
+            if (e & 8) r *= p;
+            if (e & 16) r *= p * p;
+        }
+    }
     return r;
 }
 
@@ -291,13 +298,13 @@ struct KernF<SPH_KERNEL_SINC> {
         if (!(x < kPif)) return 0.0f;
         float sn, cs;
         __sincosf(x, &sn, &cs);
-        return ipowf(x > 0.0f ? __fdividef(sn, x) : 1.0f, n);
+        return ipow(x > 0.0f ? __fdividef(sn, x) : 1.0f, n);
     }
     static __device__ __forceinline__ double dens(double r, double w, int n)
     {
         const double x = kPi * r * w;
         if (!(x < kPi)) return 0.0;
-        return ipowd(x > 0.0 ? sin(x) / x : 1.0, n);
+        return ipow(x > 0.0 ? sin(x) / x : 1.0, n);
     }
     static __device__ __forceinline__ float grad(float r, float w, float w5, int n)
     {
@@ -306,7 +313,7 @@ struct KernF<SPH_KERNEL_SINC> {
         float sn, cs;
         __sincosf(x, &sn, &cs);
         const float S = x > 0.0f ? __fdividef(sn, x) : 1.0f;
-        return w5 * ipowf(S, n - 1) * sinc_g(x, sn, cs);
+        return w5 * ipow(S, n - 1) * sinc_g(x, sn, cs);
     }
     static __device__ __forceinline__ double grad(double r, double w5, double w, int n)
     {
@@ -315,7 +322,7 @@ struct KernF<SPH_KERNEL_SINC> {
         double sn, cs;
         sincos(x, &sn, &cs);
         const double S = x > 0.0 ? sn / x : 1.0;
-        return w5 * ipowd(S, n - 1) * sinc_g(x, sn, cs);
+        return w5 * ipow(S, n - 1) * sinc_g(x, sn, cs);
     }
     static __host__ __device__ double grad_scale(double kb, int n) { return 4.0 * kb * n * kPi * kPi; }
     // grad-h weight -v d(S^n)/dv = n S^(n-1) x^2 g(x) (x = pi v / 2), never
@@ -327,7 +334,7 @@ struct KernF<SPH_KERNEL_SINC> {
         float sn, cs;
         __sincosf(x, &sn, &cs);
         const float S = x > 0.0f ? __fdividef(sn, x) : 1.0f;
-        return (float)n * ipowf(S, n - 1) * (x * x) * sinc_g(x, sn, cs);
+        return (float)n * ipow(S, n - 1) * (x * x) * sinc_g(x, sn, cs);
     }
     static __device__ __forceinline__ double omega_w(double r, double w, int n)
     {
@@ -336,7 +343,7 @@ struct KernF<SPH_KERNEL_SINC> {
         double sn, cs;
         sincos(x, &sn, &cs);
         const double S = x > 0.0 ? sn / x : 1.0;
-        return n * ipowd(S, n - 1) * (x * x) * sinc_g(x, sn, cs);
+        return n * ipow(S, n - 1) * (x * x) * sinc_g(x, sn, cs);
     }
     // dens and omega_w from one sin/cos and one power S^(n-1)
     static __device__ __forceinline__ void dens_omega(float r, float w, int n, float& d, float& g)
@@ -349,7 +356,7 @@ struct KernF<SPH_KERNEL_SINC> {
         float sn, cs;
         __sincosf(x, &sn, &cs);
         const float S = x > 0.0f ? __fdividef(sn, x) : 1.0f;
-        const float Sn1 = ipowf(S, n - 1);
+        const float Sn1 = ipow(S, n - 1);
         d = Sn1 * S;
         g = (float)n * Sn1 * (x * x) * sinc_g(x, sn, cs);
     }
@@ -363,7 +370,7 @@ struct KernF<SPH_KERNEL_SINC> {
         double sn, cs;
         sincos(x, &sn, &cs);
         const double S = x > 0.0 ? sn / x : 1.0;
-        const double Sn1 = ipowd(S, n - 1);
+        const double Sn1 = ipow(S, n - 1);
         d = Sn1 * S;
         g = n * Sn1 * (x * x) * sinc_g(x, sn, cs);
     }
@@ -666,6 +673,10 @@ __device__ __forceinline__ void momentum_chunk(const PairSrc& src, const PairSid
         bz = pz.x + pz.y;
         bu = pu.x + pu.y;
     } else {
+        // the chunk's words within the stencil (words past nv do not matter)
+        bool coded = true;
+#pragma unroll
+        for (int u = 0; u < 4; u++) coded = coded && ((uint32_t)u >= nv || (cws[u] >> kColBits) != kFarCode);
 #pragma unroll
         for (int u = 0; u < 4; u++) {
             if ((uint32_t)u >= nv) break;
@@ -673,7 +684,8 @@ __device__ __forceinline__ void momentum_chunk(const PairSrc& src, const PairSid
             float4 q, vj, tj;
             R.load(u, cw, q, vj, tj);
             float dx, dy, dz;
-            col_dx<ZW>(src, I, cw, q, dx, dy, dz);
+            if (coded) rel_dx<ZW>(stencil_offset(cw >> kColBits), I.s_f, I.sz_f, I.lz_f, I.ncz_f, I.ri.x, I.ri.y, I.ri.z, q, dx, dy, dz);
+            else col_dx<ZW>(src, I, cw, q, dx, dy, dz);
             const PairTerms t = momentum_pair<KERN, GH>(dx, dy, dz, vi, ti, wi5, vj, tj, q.w, K, kn);
             bx += t.ax;
             by += t.ay;
