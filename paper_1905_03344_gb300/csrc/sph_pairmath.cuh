@@ -157,17 +157,28 @@ __device__ __forceinline__ T ipow(T b, int e)
     return r;
 }
 
-// g(x) = (sin x - x cos x)/x^3: its Taylor series sum_m (-1)^(m+1) 2m x^(2m-2)
-// / (2m+1)! below x = 1, where the direct form loses digits to cancellation
-__device__ __forceinline__ float sinc_g(float x, float sn, float cs)
+// 1/x with one Newton step on the approximate reciprocal (x = 0 gives NaN,
+// which no caller uses)
+__device__ __forceinline__ float recip(float x)
 {
-    if (x < 1.0f) {
+    const float y = __fdividef(1.0f, x);
+    return fmaf(y, fmaf(-x, y, 1.0f), y);
+}
+
+// g(x) = (sin x - x cos x)/x^3 (rx: 1/x): its Taylor series sum_m (-1)^(m+1)
+// 2m x^(2m-2) / (2m+1)! below x = 2 (FP64: 1), where the direct form loses
+// digits to cancellation and to the fast sine's absolute error (3e-6 of g at
+// x = 1; the six terms leave 2e-7 at 2)
+__device__ __forceinline__ float sinc_g(float x, float rx, float sn, float cs)
+{
+    if (x < 2.0f) {
         const float x2 = x * x;
-        return fmaf(x2, fmaf(x2, fmaf(x2, fmaf(x2, 1.0f / 3991680.0f, -1.0f / 45360.0f), 1.0f / 840.0f),
+        return fmaf(x2, fmaf(x2, fmaf(x2, fmaf(x2, fmaf(x2, -1.0f / 518918400.0f, 1.0f / 3991680.0f), -1.0f / 45360.0f),
+                                      1.0f / 840.0f),
                              -1.0f / 30.0f),
                     1.0f / 3.0f);
     }
-    return __fdividef(fmaf(-x, cs, sn), x * x * x);
+    return fmaf(-x, cs, sn) * (rx * rx * rx);
 }
 __device__ __forceinline__ double sinc_g(double x, double sn, double cs)
 {
@@ -312,8 +323,9 @@ struct KernF<SPH_KERNEL_SINC> {
         if (!(x < kPif)) return 0.0f;
         float sn, cs;
         __sincosf(x, &sn, &cs);
-        const float S = x > 0.0f ? __fdividef(sn, x) : 1.0f;
-        return w5 * ipow(S, n - 1) * sinc_g(x, sn, cs);
+        const float rx = recip(x);
+        const float S = x > 0.0f ? sn * rx : 1.0f;
+        return w5 * ipow(S, n - 1) * sinc_g(x, rx, sn, cs);
     }
     static __device__ __forceinline__ double grad(double r, double w5, double w, int n)
     {
@@ -333,8 +345,9 @@ struct KernF<SPH_KERNEL_SINC> {
         if (!(x < kPif)) return 0.0f;
         float sn, cs;
         __sincosf(x, &sn, &cs);
-        const float S = x > 0.0f ? __fdividef(sn, x) : 1.0f;
-        return (float)n * ipow(S, n - 1) * (x * x) * sinc_g(x, sn, cs);
+        const float rx = recip(x);
+        const float S = x > 0.0f ? sn * rx : 1.0f;
+        return (float)n * ipow(S, n - 1) * (x * x) * sinc_g(x, rx, sn, cs);
     }
     static __device__ __forceinline__ double omega_w(double r, double w, int n)
     {
@@ -358,7 +371,7 @@ struct KernF<SPH_KERNEL_SINC> {
         const float S = x > 0.0f ? __fdividef(sn, x) : 1.0f;
         const float Sn1 = ipow(S, n - 1);
         d = Sn1 * S;
-        g = (float)n * Sn1 * (x * x) * sinc_g(x, sn, cs);
+        g = (float)n * Sn1 * (x * x) * sinc_g(x, recip(x), sn, cs);
     }
     static __device__ __forceinline__ void dens_omega(double r, double w, int n, double& d, double& g)
     {
