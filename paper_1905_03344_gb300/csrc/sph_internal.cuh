@@ -319,6 +319,37 @@ __device__ __forceinline__ double block_neumaier(const double* part, int n, int 
 }
 #endif
 
+#ifdef __CUDACC__
+// The kernels of a step follow one another on one stream, and for a few
+// thousand particles most of them run for less time than the next one's launch
+// takes.  So they are launched with programmatic stream serialization: the
+// next kernel's launch is under way while the one before it ends, and its
+// threads begin with wait_before(), which holds them until that kernel is
+// complete and its writes are visible.  Every kernel launched by launch_next()
+// begins with it, so each is complete before a later one reads or writes; none
+// of them reads through the non-coherent path, whose loads could move above
+// it.  Ten steps of 20^3 particles in FP64 3467 -> 3092 us, of 33^3 mixed
+// 2773 -> 2439 us, sort and lists of 45^3 326 -> 302 us; 64 patches and 100^3
+// as before.
+__device__ __forceinline__ void wait_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline void launch_next(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+#endif
+
 // ---- launch wrappers (each returns the number of kernels launched) --------
 struct Launch {
     cudaStream_t stream;

@@ -44,6 +44,7 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, int lane)
 template <bool EXACT>
 __global__ void __launch_bounds__(32 * kNbtWarps, SPH_NB_MINB) k_nb_thread(NbArgs a)
 {
+    wait_before();
     extern __shared__ __align__(16) uint32_t nb_ring[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t* ring = nb_ring + warp * (32 * (kRing + kPend)) + lane;
@@ -131,7 +132,7 @@ void launch_nb_thread(const Launch& L, const NbArgs& a)
             cudaFuncSetAttribute(k_nb_thread<EXACT>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
         }
     }
-    k_nb_thread<EXACT><<<L.sms * per_sm, 32 * kNbtWarps, smem, L.stream>>>(a);
+    launch_next(k_nb_thread<EXACT>, L.sms * per_sm, 32 * kNbtWarps, smem, L.stream, a);
 }
 
 // ---- a team of lanes per particle ------------------------------------------
@@ -369,6 +370,7 @@ __device__ __forceinline__ void team_search(const NbArgs& a, const PatchDev* P, 
 template <bool EXACT>
 __global__ void __launch_bounds__(32 * kNbtWarps, 5) k_nb_team(const __grid_constant__ NbArgs a, int sub_log)
 {
+    wait_before();
     __shared__ TeamShared shared[kNbtWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     TeamShared& sh = shared[warp];
@@ -486,7 +488,7 @@ static void launch_nb_team(const Launch& L, const NbArgs& a)
     int sub_log = 0;
     while (sub_log < 3 && (a.nunits << sub_log) < 2 * resident) sub_log++;
     const int64_t need = ((a.nunits << sub_log) + kNbtWarps - 1) / kNbtWarps, cap = (int64_t)L.sms * per_sm;
-    k_nb_team<EXACT><<<(unsigned)(need < cap ? need : cap), 32 * kNbtWarps, 0, L.stream>>>(a, sub_log);
+    launch_next(k_nb_team<EXACT>, (unsigned)(need < cap ? need : cap), 32 * kNbtWarps, 0, L.stream, a, sub_log);
 }
 
 template <bool EXACT>

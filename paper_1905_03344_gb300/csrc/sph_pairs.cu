@@ -157,6 +157,7 @@ __device__ __forceinline__ void density_row(const PairArgs& a, const uint32_t* r
 template <int TPP, int KERN, bool GH>
 __global__ void __launch_bounds__(256, SPH_DEN_MINB) k_density_mixed(PairArgs a)
 {
+    wait_before();
     const float kb8 = (float)(8.0 * a.kb);
     if (*a.status & kStBad) return;
     const GroupIdx G = group_idx<TPP>();
@@ -190,6 +191,7 @@ __global__ void __launch_bounds__(256, SPH_DEN_MINB) k_density_mixed(PairArgs a)
 template <int TPP, int KERN, bool GH>
 __global__ void __launch_bounds__(256) k_density_fp64(PairArgs a)
 {
+    wait_before();
     const int kn = a.kernel_n;
     if (*a.status & kStBad) return;
     const GroupIdx G = group_idx<TPP>();
@@ -260,6 +262,7 @@ __device__ __forceinline__ void momentum_row(const PairArgs& a, const uint32_t* 
 template <int TPP, int KERN, bool GH>
 __global__ void __launch_bounds__(256, SPH_MOM_MINB) k_momentum_mixed(PairArgs a)
 {
+    wait_before();
     const float gscale = (float)KernF<KERN>::grad_scale(a.kb, a.kernel_n);
     if (*a.status & kStBad) return;
     const GroupIdx G = group_idx<TPP>();
@@ -298,6 +301,7 @@ __global__ void __launch_bounds__(256, SPH_MOM_MINB) k_momentum_mixed(PairArgs a
 template <int TPP, int KERN, bool GH>
 __global__ void __launch_bounds__(256) k_momentum_fp64(PairArgs a)
 {
+    wait_before();
     if (*a.status & kStBad) return;
     const GroupIdx G = group_idx<TPP>();
     const int64_t gs = ((int64_t)gridDim.x * blockDim.x) / TPP;
@@ -321,26 +325,26 @@ __global__ void __launch_bounds__(256) k_momentum_fp64(PairArgs a)
     }
 }
 
-#define SPH_DISPATCH_TPP(KERNEL, KERN, GH, tpp, g, L, a)                                        \
-    switch (tpp) {                                                                              \
-    case 1: KERNEL<1, KERN, GH><<<(g).x, (g).y, 0, (L).stream>>>(a); break;                     \
-    case 2: KERNEL<2, KERN, GH><<<(g).x, (g).y, 0, (L).stream>>>(a); break;                     \
-    case 4: KERNEL<4, KERN, GH><<<(g).x, (g).y, 0, (L).stream>>>(a); break;                     \
-    case 16: KERNEL<16, KERN, GH><<<(g).x, (g).y, 0, (L).stream>>>(a); break;                   \
-    case 32: KERNEL<32, KERN, GH><<<(g).x, (g).y, 0, (L).stream>>>(a); break;                   \
-    default: KERNEL<8, KERN, GH><<<(g).x, (g).y, 0, (L).stream>>>(a); break;                    \
+#define SPH_DISPATCH_TPP(KERNEL, KERN, GH, tpp, g, L, a)                                \
+    switch (tpp) {                                                                      \
+    case 1: launch_next(KERNEL<1, KERN, GH>, (g).x, (g).y, 0, (L).stream, a); break;    \
+    case 2: launch_next(KERNEL<2, KERN, GH>, (g).x, (g).y, 0, (L).stream, a); break;    \
+    case 4: launch_next(KERNEL<4, KERN, GH>, (g).x, (g).y, 0, (L).stream, a); break;    \
+    case 16: launch_next(KERNEL<16, KERN, GH>, (g).x, (g).y, 0, (L).stream, a); break;  \
+    case 32: launch_next(KERNEL<32, KERN, GH>, (g).x, (g).y, 0, (L).stream, a); break;  \
+    default: launch_next(KERNEL<8, KERN, GH>, (g).x, (g).y, 0, (L).stream, a); break;   \
     }
-#define SPH_DISPATCH_GH(KERNEL, KERN, tpp, g, L, a)                                        \
-    if ((a).grad_h) {                                                                           \
-        SPH_DISPATCH_TPP(KERNEL, KERN, true, tpp, g, L, a);                                \
-    } else {                                                                                    \
-        SPH_DISPATCH_TPP(KERNEL, KERN, false, tpp, g, L, a);                               \
+#define SPH_DISPATCH_GH(KERNEL, KERN, tpp, g, L, a)                                     \
+    if ((a).grad_h) {                                                                   \
+        SPH_DISPATCH_TPP(KERNEL, KERN, true, tpp, g, L, a);                             \
+    } else {                                                                            \
+        SPH_DISPATCH_TPP(KERNEL, KERN, false, tpp, g, L, a);                            \
     }
-#define SPH_DISPATCH(KERNEL, tpp, g, L, a)                                                 \
-    if ((a).kernel == SPH_KERNEL_SINC) {                                                        \
-        SPH_DISPATCH_GH(KERNEL, SPH_KERNEL_SINC, tpp, g, L, a);                            \
-    } else {                                                                                    \
-        SPH_DISPATCH_GH(KERNEL, SPH_KERNEL_WENDLAND, tpp, g, L, a);                        \
+#define SPH_DISPATCH(KERNEL, tpp, g, L, a)                                              \
+    if ((a).kernel == SPH_KERNEL_SINC) {                                                \
+        SPH_DISPATCH_GH(KERNEL, SPH_KERNEL_SINC, tpp, g, L, a);                         \
+    } else {                                                                            \
+        SPH_DISPATCH_GH(KERNEL, SPH_KERNEL_WENDLAND, tpp, g, L, a);                     \
     }
 
 // {blocks, threads}: blocks of 256 threads that stride over the particles,

@@ -35,6 +35,7 @@ __device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsig
 __global__ void __launch_bounds__(256) k_reduce_bbox(State s, const WorkItem* items, int nitems,
                                                      PatchRed* red)
 {
+    wait_before();
     __shared__ unsigned long long sh[5][8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
@@ -84,13 +85,14 @@ int launch_reduce_bbox(const Launch& L, const State& s, const WorkItem* items, i
 {
     if (nitems <= 0) return 0;
     int grid = nitems < L.sms * 8 ? nitems : L.sms * 8;
-    k_reduce_bbox<<<grid, 256, 0, L.stream>>>(s, items, nitems, red);
+    launch_next(k_reduce_bbox, grid, 256, 0, L.stream, s, items, nitems, red);
     return 1;
 }
 
 // (and clears the radix sort's counters)
 __global__ void k_reset_red(int npatch, PatchRed* red, uint32_t* zero, int64_t words)
 {
+    wait_before();
     int p = blockIdx.x * blockDim.x + threadIdx.x;
     for (int64_t k = p; k < words; k += (int64_t)gridDim.x * blockDim.x) zero[k] = 0u;
     if (p < npatch) {
@@ -112,6 +114,7 @@ __global__ void k_reset_red(int npatch, PatchRed* red, uint32_t* zero, int64_t w
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_h_hist(State s, const WorkItem* items, int nitems, PatchRed* red)
 {
+    wait_before();
     __shared__ uint32_t hist[kHBins];
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const WorkItem w = items[it];
@@ -152,13 +155,14 @@ int launch_h_hist(const Launch& L, const State& s, const WorkItem* items, int ni
 {
     if (nitems <= 0) return 0;
     int grid = nitems < L.sms * 8 ? nitems : L.sms * 8;
-    k_h_hist<<<grid, 256, 0, L.stream>>>(s, items, nitems, red);
+    launch_next(k_h_hist, grid, 256, 0, L.stream, s, items, nitems, red);
     return 1;
 }
 
 int launch_reset_red(const Launch& L, int npatch, PatchRed* red, uint32_t* zero, int64_t words)
 {
-    k_reset_red<<<blocks_for(words > npatch ? words : npatch, 256, L.sms, 8), 256, 0, L.stream>>>(npatch, red, zero, words);
+    launch_next(k_reset_red, blocks_for(words > npatch ? words : npatch, 256, L.sms, 8), 256, 0, L.stream, npatch, red,
+                zero, words);
     return 1;
 }
 
@@ -178,6 +182,7 @@ int launch_reset_red(const Launch& L, int npatch, PatchRed* red, uint32_t* zero,
 __global__ void k_grid_params(int npatch, const PatchRed* red, PatchDev* pd, double cell_factor,
                               int* status, unsigned long long* vote)
 {
+    wait_before();
     int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p < 2) vote[p] = 0ull;          // counted afresh by k_cell_hnb
     if (p >= npatch) return;
@@ -302,7 +307,7 @@ __global__ void k_grid_params(int npatch, const PatchRed* red, PatchDev* pd, dou
 int launch_grid_params(const Launch& L, int npatch, const PatchRed* red, PatchDev* pd,
                        double cell_factor, int* status, unsigned long long* vote)
 {
-    k_grid_params<<<(npatch + 127) / 128, 128, 0, L.stream>>>(npatch, red, pd, cell_factor, status, vote);
+    launch_next(k_grid_params, (npatch + 127) / 128, 128, 0, L.stream, npatch, red, pd, cell_factor, status, vote);
     return 1;
 }
 
@@ -329,6 +334,7 @@ __device__ __forceinline__ void add_digits(int passes, const uint32_t (*sh)[256]
 __global__ void __launch_bounds__(256) k_keys(int64_t n, State s, const uint16_t* patch_of,
                                               PatchDev* pd, uint32_t* keys, uint32_t* vals, int passes, uint32_t* hist)
 {
+    wait_before();
     __shared__ uint32_t sh[kRsMaxPasses][256];
     for (int k = threadIdx.x; k < kRsMaxPasses * 256; k += blockDim.x) (&sh[0][0])[k] = 0u;
     __syncthreads();
@@ -366,7 +372,7 @@ int launch_keys(const Launch& L, int64_t n, const State& s, const uint16_t* patc
     if (n <= 0) return 0;
     uint32_t *k, *v;
     rs.input(passes, k, v);
-    k_keys<<<blocks_for(n, 256, L.sms, 8), 256, 0, L.stream>>>(n, s, patch_of, pd, k, v, passes, rs.work);
+    launch_next(k_keys, blocks_for(n, 256, L.sms, 8), 256, 0, L.stream, n, s, patch_of, pd, k, v, passes, rs.work);
     return 1;
 }
 
@@ -509,10 +515,11 @@ constexpr int kRsSpins = 1 << 22;
 constexpr int kRsItems = 12;            // keys a thread takes in the larger tiles
 
 template <int ITEMS>
-__global__ void __launch_bounds__(kRsThreads, ITEMS == 4 ? 6 : 5) k_rs_pass(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-                                                       int64_t n, int shift, const uint32_t* __restrict__ ghist, uint32_t* ticket,
-                                                       volatile uint32_t* state, uint32_t* kout, uint32_t* vout, int* status)
+__global__ void __launch_bounds__(kRsThreads, ITEMS == 4 ? 6 : 5) k_rs_pass(const uint32_t* kin,
+        const uint32_t* vin, int64_t n, int shift, const uint32_t* ghist, uint32_t* ticket,
+        volatile uint32_t* state, uint32_t* kout, uint32_t* vout, int* status)
 {
+    wait_before();
     constexpr int kTile = kRsThreads * ITEMS;
     __shared__ uint32_t s_keys[kTile];
     __shared__ uint32_t s_vals[kTile];
@@ -636,8 +643,8 @@ int launch_radix_sort(const Launch& L, int64_t n, int passes, const RadixSort& r
         uint32_t* tickets = rs.work + kRsMaxPasses * 256;
         uint32_t* state = tickets + kRsMaxPasses * 16 + (int64_t)ps * 256 * tiles;
         const auto kern = rs_items(n) == 4 ? k_rs_pass<4> : k_rs_pass<kRsItems>;
-        kern<<<(unsigned)tiles, kRsThreads, 0, L.stream>>>(ki, vi, n, 8 * ps, rs.work + 256 * ps, tickets + 16 * ps, state, ko, vo,
-                                                           status);
+        launch_next(kern, (unsigned)tiles, kRsThreads, 0, L.stream, ki, vi, n, 8 * ps, rs.work + 256 * ps, tickets + 16 * ps,
+                    state, ko, vo, status);
         ki = ko;
         vi = vo;
     }
@@ -747,6 +754,7 @@ __global__ void __launch_bounds__(256) k_gather(int64_t n, const uint32_t* skeys
                                                 Recs r, Fp64 f, int mixed, int kernel, RowHint hint,
                                                 const double* hsearch, double* hsearch_out, const int* status)
 {
+    wait_before();
     const bool have_hint = *hint.valid != 0;
     // a sort whose wait ran out: the particles keep their order, and the step
     // ends with its status
@@ -811,9 +819,8 @@ int launch_gather(const Launch& L, int64_t n, const uint32_t* skeys, const uint3
                   const RowHint& hint, const int* status, const double* hsearch, double* hsearch_out)
 {
     if (n <= 0) return 0;
-    k_gather<<<blocks_for(n, 256, L.sms, 16), 256, 0, L.stream>>>(n, skeys, svals, src, dst, perm_src,
-                                                                 perm_dst, pd, g, r, f, mixed, kernel, hint, hsearch,
-                                                                 hsearch_out, status);
+    launch_next(k_gather, blocks_for(n, 256, L.sms, 16), 256, 0, L.stream, n, skeys, svals, src, dst, perm_src, perm_dst,
+                pd, g, r, f, mixed, kernel, hint, hsearch, hsearch_out, status);
     return 1;
 }
 
@@ -852,6 +859,7 @@ int launch_refresh_records(const Launch& L, int64_t n, const State& s, const uin
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_cell_rows(PatchDev* pd, Grid g, const float4* r4, int K, float* hnb_x)
 {
+    wait_before();
     constexpr int kPad = 4;             // at least K
     __shared__ float sh[8][kMaxCellsAxis + 2 * kPad];
     PatchDev* P = pd + blockIdx.y;
@@ -921,6 +929,7 @@ __global__ void __launch_bounds__(256) k_cell_rows(PatchDev* pd, Grid g, const f
 // (h varying from particle to particle) favour cells of edge h_s.
 __global__ void __launch_bounds__(256) k_cell_hnb(const PatchDev* pd, Grid g, int K, const float* hnb_x, unsigned long long* vote)
 {
+    wait_before();
     const PatchDev* P = pd + blockIdx.y;
     const int ncx = P->ncx, ncy = P->ncy, ncz = P->ncz;
     const int64_t nxy = (int64_t)ncx * ncy;
@@ -964,8 +973,8 @@ int launch_cell_tables(const Launch& L, int npatch, PatchDev* pd, const Grid& g,
     if (npatch <= 0) return 0;
     const int rows_x = npatch > 8 ? 64 : (L.sms * 8 + npatch - 1) / npatch;
     const int cells_x = npatch > 8 ? 16 : (L.sms * 8 + npatch - 1) / npatch;
-    k_cell_rows<<<dim3((unsigned)rows_x, (unsigned)npatch), 256, 0, L.stream>>>(pd, g, r4, K, tmp);
-    k_cell_hnb<<<dim3((unsigned)cells_x, (unsigned)npatch), 256, 0, L.stream>>>(pd, g, K, tmp, vote);
+    launch_next(k_cell_rows, dim3((unsigned)rows_x, (unsigned)npatch), 256, 0, L.stream, pd, g, r4, K, tmp);
+    launch_next(k_cell_hnb, dim3((unsigned)cells_x, (unsigned)npatch), 256, 0, L.stream, pd, g, K, tmp, vote);
     return 2;
 }
 

@@ -23,6 +23,7 @@ namespace sphg {
 // 2 to 4 % of their time.)
 __global__ void __launch_bounds__(256) k_dt(StepArgs a)
 {
+    wait_before();
     __shared__ unsigned long long sh[8];
     __shared__ bool last;
     if (*a.status & kStBad) return;
@@ -87,13 +88,14 @@ __global__ void __launch_bounds__(256) k_dt(StepArgs a)
 int launch_dt(const Launch& L, const StepArgs& a)
 {
     const int cap = L.sms * 8;
-    k_dt<<<a.nitems < 1 ? 1 : (a.nitems < cap ? a.nitems : cap), 256, 0, L.stream>>>(a);
+    launch_next(k_dt, a.nitems < 1 ? 1 : (a.nitems < cap ? a.nitems : cap), 256, 0, L.stream, a);
     return 1;
 }
 
 // ---- kick, drift, Adams-Bashforth, h, conserved partials --------------------
 __global__ void __launch_bounds__(256) k_update(StepArgs a)
 {
+    wait_before();
     __shared__ double sh[7][8];
     if (*a.status & kStBad) return;
     for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
@@ -150,7 +152,7 @@ int launch_update(const Launch& L, const StepArgs& a)
 {
     if (a.nitems <= 0) return 0;
     const int grid = a.nitems < L.sms * 8 ? a.nitems : L.sms * 8;
-    k_update<<<grid, 256, 0, L.stream>>>(a);
+    launch_next(k_update, grid, 256, 0, L.stream, a);
     return 1;
 }
 
@@ -180,6 +182,7 @@ int launch_conserved_items(const Launch& L, const StepArgs& a)
 // also closes the step.
 __global__ void __launch_bounds__(256) k_conserved_finalize(StepArgs a, int advance)
 {
+    wait_before();
     __shared__ double sh_s[256], sh_c[256];
     const int t = blockIdx.x;
     if (t >= a.npatch * 7) return;
@@ -198,13 +201,13 @@ __global__ void __launch_bounds__(256) k_conserved_finalize(StepArgs a, int adva
 
 int launch_conserved_finalize(const Launch& L, const StepArgs& a)
 {
-    k_conserved_finalize<<<a.npatch * 7, 256, 0, L.stream>>>(a, 0);
+    launch_next(k_conserved_finalize, a.npatch * 7, 256, 0, L.stream, a, 0);
     return 1;
 }
 
 int launch_step_finalize(const Launch& L, const StepArgs& a)
 {
-    k_conserved_finalize<<<a.npatch * 7, 256, 0, L.stream>>>(a, 1);
+    launch_next(k_conserved_finalize, a.npatch * 7, 256, 0, L.stream, a, 1);
     return 1;
 }
 
