@@ -256,11 +256,21 @@ __device__ __forceinline__ void momentum_row(const PairArgs& a, const uint32_t* 
     }
 }
 
-#ifndef SPH_MOM_MINB
-#define SPH_MOM_MINB 2                  // resident 256-thread CTAs per SM the registers are sized for
-#endif
+// Resident 256-thread CTAs per SM that the registers are sized for.  The packed
+// pairs of the Wendland kernel need 112 registers (at 80 they spill: 10^6
+// particles 512 -> 557 us).  The scalar loop of the Sinc kernel and of the
+// grad-h form needs 100 to 105, waits on its gathers and special functions,
+// and gains more from the third CTA than its 8 bytes of spill cost: 250,000
+// particles, Sinc 209 -> 189 us, Wendland with grad-h 148 -> 127 us; with h
+// varying 10 to 1, 491 -> 420 us and 322 -> 261 us.
+template <int KERN, bool GH>
+constexpr int mom_minb()
+{
+    return KERN == SPH_KERNEL_WENDLAND && !GH ? 2 : 3;
+}
+
 template <int TPP, int KERN, bool GH>
-__global__ void __launch_bounds__(256, SPH_MOM_MINB) k_momentum_mixed(PairArgs a)
+__global__ void __launch_bounds__(256, mom_minb<KERN, GH>()) k_momentum_mixed(PairArgs a)
 {
     wait_before();
     const float gscale = (float)KernF<KERN>::grad_scale(a.kb, a.kernel_n);
