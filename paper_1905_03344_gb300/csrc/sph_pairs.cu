@@ -360,9 +360,15 @@ __global__ void __launch_bounds__(256) k_momentum_fp64(PairArgs a)
 // {blocks, threads}: blocks of 256 threads that stride over the particles,
 // of 64 while 256 would leave the SMs unevenly filled (8000 particles at 8
 // lanes are 250 blocks of 256 for 152 SMs: some get two, some one)
-static uint2 pair_grid(const Launch& L, int64_t n, int tpp)
+// per_sm: blocks of 256 for each SM.  The mixed sums, whose two to four
+// resident blocks hide latency, are best at 8 (from 16 on 2 to 8 % slower: a
+// block is done before its prefetches pay); the FP64 momentum sum is bound by
+// the FP64 pipe and loses only in its last round, so it takes 16 (125,000
+// particles 1234 -> 1196 us, 64,000 with h 10 to 1 1375 -> 1346 us, 10^6 as
+// before).
+static uint2 pair_grid(const Launch& L, int64_t n, int tpp, int per_sm = 8)
 {
-    const int64_t cap = (int64_t)L.sms * 8;
+    const int64_t cap = (int64_t)L.sms * per_sm;
     int64_t blocks = (n * tpp + 255) / 256;
     if (blocks < cap) return make_uint2((unsigned)((n * tpp + 63) / 64), 64u);
     return make_uint2((unsigned)cap, 256u);
@@ -383,7 +389,7 @@ int launch_density(const Launch& L, const PairArgs& a, int tpp, int mixed)
 int launch_momentum(const Launch& L, const PairArgs& a, int tpp, int mixed)
 {
     if (a.n <= 0) return 0;
-    const uint2 g = pair_grid(L, a.n, tpp);
+    const uint2 g = pair_grid(L, a.n, tpp, mixed ? 8 : 16);
     if (mixed) {
         SPH_DISPATCH(k_momentum_mixed, tpp, g, L, a);
     } else {
