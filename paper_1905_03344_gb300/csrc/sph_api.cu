@@ -125,6 +125,7 @@ struct sph_ctx {
     int64_t nunits = 0, cap_units = 0;
     unsigned long long *rowstart = nullptr, *pool_used = nullptr;  // pool_used: [reserved, listed]
     uint32_t* rowcap = nullptr;    // row-length hints in the current sorted order
+    bool pool_clear = false;       // the last enqueued sort left pool_used cleared
     int* hint_ok = nullptr;        // device flag: cnt holds row lengths of the current order
     bool cnt_valid = false;        // host: cnt holds the row lengths of the current order
     uint32_t* cnt_orig = nullptr;  // row lengths carried to the caller's order (set_particles)
@@ -310,6 +311,7 @@ NbArgs nb_args(sph_ctx* ctx)
     a.col = ctx->col;
     a.rowcap = ctx->rowcap;
     a.pool_used = ctx->pool_used;
+    a.hint_ok = ctx->hint_ok;
     a.max_pairs = ctx->max_pairs;
     a.pool_cap = ctx->pool_cap;
     a.status = ctx->status;
@@ -397,7 +399,9 @@ void enqueue_sort(sph_ctx* ctx, bool superset = false)
     }
     {
         Phase p(ctx, SPH_PHASE_BBOX);
-        ctx->launches += launch_reset_red(L, ctx->npatch, ctx->red, ctx->hist, (int64_t)radix_work_words(ctx->n));
+        ctx->launches += launch_reset_red(L, ctx->npatch, ctx->red,
+                                          SortClear{ctx->hist, (int64_t)radix_work_words(ctx->n), ctx->grid.cell,
+                                                    ctx->cells_used, ctx->pool_used});
         ctx->launches += launch_reduce_bbox(L, s, ctx->items, ctx->nitems, ctx->red);
         ctx->launches += launch_h_hist(L, s, ctx->items, ctx->nitems, ctx->red);
         ctx->launches += launch_grid_params(L, ctx->npatch, ctx->red, ctx->pd, ctx->cell_factor, ctx->status,
@@ -413,7 +417,6 @@ void enqueue_sort(sph_ctx* ctx, bool superset = false)
     }
     {
         Phase p(ctx, SPH_PHASE_GATHER);
-        cudaMemsetAsync(ctx->grid.cell, 0, (size_t)ctx->cells_used * sizeof(uint4), ctx->stream);
         const int nxt = 1 - ctx->cur;
         ctx->launches += launch_gather(L, ctx->n, ctx->keys, ctx->vals, ctx->st[ctx->cur], ctx->st[nxt],
                                        ctx->perm[ctx->cur], ctx->perm[nxt], ctx->pd, ctx->grid, ctx->rec,
@@ -427,24 +430,31 @@ void enqueue_sort(sph_ctx* ctx, bool superset = false)
         ctx->cur = nxt;
     }
     ctx->fresh = false;
+    ctx->pool_clear = true;
+}
+
+// an empty list pool: left by the sort that was enqueued last, or (a second
+// search on one grid) cleared here
+void enqueue_pool_reset(sph_ctx* ctx)
+{
+    if (!ctx->pool_clear) {
+        Phase p(ctx, SPH_PHASE_NB_RESET);
+        cudaMemsetAsync(ctx->pool_used, 0, 2 * sizeof(unsigned long long), ctx->stream);
+    }
+    ctx->pool_clear = false;
 }
 
 void enqueue_lists(sph_ctx* ctx)
 {
     const Launch L = launch_of(ctx);
     const NbArgs a = nb_args(ctx);
-    {
-        Phase p(ctx, SPH_PHASE_NB_RESET);
-        cudaMemsetAsync(ctx->pool_used, 0, 2 * sizeof(unsigned long long), ctx->stream);
-    }
+    enqueue_pool_reset(ctx);
     ctx->canon_valid = false;
     {
         Phase p(ctx, SPH_PHASE_NB);
         ctx->launches += launch_nb_lists(L, a, 1);
     }
     ctx->bins_valid = false;
-    // the row lengths now belong to the current order: hints for the next sort
-    cudaMemsetAsync(ctx->hint_ok, 1, sizeof(int), ctx->stream);
 }
 
 // the particles binned by row length, once per set of lists (counted in the
@@ -469,6 +479,7 @@ void enqueue_density(sph_ctx* ctx)
     if (ctx->fused) {
         {
             // the density pass counts the pairs again
+            ctx->pool_clear = false;
             Phase p(ctx, SPH_PHASE_NB_RESET);
             cudaMemsetAsync(ctx->pool_used + 1, 0, sizeof(unsigned long long), ctx->stream);
         }
@@ -510,16 +521,13 @@ void enqueue_superset(sph_ctx* ctx)
     a.col = ctx->col_s;
     a.cnt = ctx->cnt_s;
     a.max_pairs = ctx->max_pairs_s;
-    {
-        Phase p(ctx, SPH_PHASE_NB_RESET);
-        cudaMemsetAsync(ctx->pool_used, 0, 2 * sizeof(unsigned long long), ctx->stream);
-    }
+    a.hint_ok = ctx->hint_ok_s;
+    enqueue_pool_reset(ctx);
     {
         Phase p(ctx, SPH_PHASE_NB);
         ctx->launches += launch_nb_lists(L, a, 0);
         ctx->launches += launch_skin_snapshot(L, ctx->n, ctx->st[ctx->cur], ctx->skinref);
     }
-    cudaMemsetAsync(ctx->hint_ok_s, 1, sizeof(int), ctx->stream);
 }
 
 // the exact lists of the current state from the superset: records of the

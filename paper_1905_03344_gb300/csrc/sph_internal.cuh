@@ -424,6 +424,7 @@ struct NbArgs {
     uint32_t* col;                       // the list pool
     const uint32_t* rowcap;              // row-length hints (kNoHint: none)
     unsigned long long* pool_used;       // [0] entries reserved, [1] entries listed (nnz)
+    int* hint_ok;                        // set: the row lengths belong to the current order
     int64_t max_pairs;                   // bound on nnz
     int64_t pool_cap;                    // entries the pool holds (max_pairs + slack)
     int* status;
@@ -542,6 +543,14 @@ int launch_unpermute_u32(const Launch& L, int64_t n, const uint32_t* src, const 
 // new particles: src (x y z vx vy vz m h u; may be s's own arrays) into s, the
 // time fields cleared, perm the identity; status: kStNonFinite for bad values
 int launch_load(const Launch& L, int64_t n, const double* const src[9], const State& s, uint32_t* perm, int* status);
-int launch_reset_red(const Launch& L, int npatch, PatchRed* red, uint32_t* zero, int64_t words);
+// what k_reset_red clears besides the reductions
+struct SortClear {
+    uint32_t* work;                // radix sort's histograms, tickets and tile states
+    int64_t words;
+    uint4* cell;                   // cell table
+    int64_t cells;
+    unsigned long long* pool_used;
+};
+int launch_reset_red(const Launch& L, int npatch, PatchRed* red, const SortClear& c);
 
 }  // namespace sphg

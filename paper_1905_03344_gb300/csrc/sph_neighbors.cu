@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_NB_MINB) k_nb_thread(NbArg
     extern __shared__ __align__(16) uint32_t nb_ring[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t* ring = nb_ring + warp * (32 * (kRing + kPend)) + lane;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.hint_ok = 1;
     if (*a.status & kStBad) return;
     const unsigned long long pool_cap = (unsigned long long)a.pool_cap;
     for (int64_t q = (int64_t)blockIdx.x * kNbtWarps + warp; q < a.nunits; q += (int64_t)gridDim.x * kNbtWarps) {
@@ -374,6 +375,7 @@ __global__ void __launch_bounds__(32 * kNbtWarps, 5) k_nb_team(const __grid_cons
     __shared__ TeamShared shared[kNbtWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     TeamShared& sh = shared[warp];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.hint_ok = 1;
     if (*a.status & kStBad) return;
     const int width = 32 >> sub_log;
     const int64_t nparts = a.nunits << sub_log;
