@@ -915,7 +915,8 @@ sph_status sph_create(const sph_config* cfg_in, sph_ctx** out)
     uint32_t* cellxyz = nullptr;
     ok = ok && dalloc(ctx, cellrec, (size_t)ctx->cap_cells) && dalloc(ctx, cellxyz, N) &&
          dalloc(ctx, ctx->grid.row, (size_t)ctx->cap_cells) && dalloc(ctx, ctx->grid.row_rec, N + 16) &&
-         dalloc(ctx, ctx->grid.row_id, N + 16) && dalloc(ctx, ctx->grid.hnb, (size_t)ctx->cap_cells) && dalloc(ctx, ctx->hnb_tmp, (size_t)ctx->cap_cells);
+         dalloc(ctx, ctx->grid.row_id, N + 16) && dalloc(ctx, ctx->grid.row_box, (size_t)ctx->cap_cells) &&
+         dalloc(ctx, ctx->grid.hnb, (size_t)ctx->cap_cells) && dalloc(ctx, ctx->hnb_tmp, (size_t)ctx->cap_cells);
     ctx->grid.cell = cellrec;
     ctx->grid.cellxyz = cellxyz;
     // kGroup-style padding: the list search reads groups of records past a cell

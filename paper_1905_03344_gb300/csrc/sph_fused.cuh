@@ -51,6 +51,7 @@ __device__ __forceinline__ bool union_decision(const NbArgs& a, const PatchDev* 
 // ---- mixed precision --------------------------------------------------------
 template <int KERN, bool GH>
 struct DensSink {
+    static constexpr bool kBoxes = false;
     PairSrc src;
     PairSide I;
     float inv2h;
@@ -75,6 +76,7 @@ struct DensSink {
 
 template <int KERN, bool GH>
 struct MomSink {
+    static constexpr bool kBoxes = false;
     PairSrc src;
     PairSide I;
     float4 vi, ti;
@@ -120,6 +122,7 @@ struct MomSink {
 // ---- FP64 -------------------------------------------------------------------
 template <int KERN, bool GH>
 struct DensSinkD {
+    static constexpr bool kBoxes = false;
     const PairArgs* pa;
     double xi, yi, zi, w, lz;
     int kn;
@@ -141,6 +144,7 @@ struct DensSinkD {
 
 template <int KERN, bool GH>
 struct MomSinkD {
+    static constexpr bool kBoxes = false;
     const PairArgs* pa;
     SideD I;
     int kn;

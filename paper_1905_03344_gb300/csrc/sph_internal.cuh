@@ -94,6 +94,9 @@ struct PatchDev {
     int32_t ncxc, ncyc, nczc;    // coarse grid
     int32_t zmode_c;             // 0: 3 distinct coarse z cells; 1: all of them
     int64_t coarse_base;         // first coarse cell in the cell tables
+    // of the row boxes (Grid::row_box): the sum of the four insets over the
+    // fine cells that have one, << 32, and the count of these
+    unsigned long long row_inset;
     // time state
     double dt, dt_prev;
     int64_t step;
@@ -131,6 +134,10 @@ struct Grid {
     uint2* row;          // [fine cell]
     float4* row_rec;     // [slot], padded past the end (read in groups)
     uint32_t* row_id;    // [slot], padded likewise
+    uint32_t* row_box;   // [fine cell] where in y and z the particles of the
+                         // row lie, K cells to each side of this one: insets
+                         // from the cell's low and high y, low and high z
+                         // face, a byte each, in 1/255 of the edge
     uint32_t* cellxyz;   // [particle] cx | cy << 8 | cz << 16
     const uint16_t* patch_of;  // [particle] patch index
     float* hnb;          // [fine cell] the largest h of the fine cells within

@@ -280,24 +280,21 @@ __device__ __forceinline__ void team_search(const NbArgs& a, const PatchDev* P, 
                     int czj = cz + dcz;
                     if (czj < 0) czj += ncz;
                     else if (czj >= ncz) czj -= ncz;
-                    const float ysh = (float)dcy * s_f, zsh = (float)dcz * sz_f;
-                    float gz = 0.0f, gy = 0.0f;
-                    if (!zw && dcz != 0) gz = fmaxf(dcz > 0 ? zsh - C.zi : C.zi - (zsh + sz_f), 0.0f);
-                    if (dcy != 0) gy = fmaxf(dcy > 0 ? ysh - C.yi : C.yi - (ysh + s_f), 0.0f);
-                    const float rem2 = R.Rg2 - fmaf(gy, gy, gz * gz);
+                    const uint32_t lrow = cbase + ((uint32_t)czj * (uint32_t)ncy + (uint32_t)(cy + dcy)) * (uint32_t)ncx;
+                    const uint32_t box = R.kx <= P->K && use_boxes(P) ? a.g.row_box[lrow + (uint32_t)cx] : 0u;
+                    f = make_float2(C.yi - (float)dcy * s_f, C.zi - (float)dcz * sz_f);
+                    const float rem2 = R.Rg2 - (zw ? row_gap2<false>(box, f.x, f.y, s_f, sz_f) : row_gap2<true>(box, f.x, f.y, s_f, sz_f));
                     if (rem2 > 0.0f) {
                         // the chord, in cells (Rg's margins cover the rounding
                         // and the FP32 cell assignment)
                         const float half = __fsqrt_rn(rem2) * inv_s;
                         const int x0 = max((int)floorf(xs - half), xlo), x1 = min((int)floorf(xs + half), xhi);
                         if (x0 <= x1) {
-                            const uint32_t lrow = cbase + ((uint32_t)czj * (uint32_t)ncy + (uint32_t)(cy + dcy)) * (uint32_t)ncx;
                             k = a.g.row[lrow + (uint32_t)x0].x;
                             ke = a.g.row[lrow + (uint32_t)x1].y;
                             const int zd = zw ? (P->zmode ? iz : 5) : dcz + 2;
                             if ((uint32_t)(dcy + 2) <= 4u && (uint32_t)zd <= 4u)
                                 add = (uint32_t)(2 + 5 * (dcy + 2) + 25 * zd - cx) << kColBits;
-                            f = make_float2(C.yi - ysh, C.zi - zsh);
                         }
                     }
                 }

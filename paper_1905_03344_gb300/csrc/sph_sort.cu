@@ -301,6 +301,7 @@ __global__ void k_grid_params(int npatch, const PatchRed* red, PatchDev* pd, dou
     P.hmed = hmed;
     P.nbig = 0;
     P.row_fill = 0;
+    P.row_inset = 0;
     P.kc = kc;
     P.ncxc = (int)ncxc;
     P.ncyc = (int)ncyc;
@@ -868,16 +869,20 @@ __global__ void __launch_bounds__(256) k_cell_rows(PatchDev* pd, Grid g, const f
     wait_before();
     constexpr int kPad = 4;             // at least K
     __shared__ float sh[8][kMaxCellsAxis + 2 * kPad];
+    __shared__ uint32_t box[8][kMaxCellsAxis + 2 * kPad];
     PatchDev* P = pd + blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ncx = P->ncx, nrows = P->ncy * P->ncz;
-    const float s_f = P->s_f;
+    const float s_f = P->s_f, qy = 255.0f * P->inv_s_f, qz = 255.0f * P->inv_sz_f;
     const uint32_t first = (uint32_t)P->begin;
     for (int r = (int)blockIdx.x * 8 + warp; r < nrows; r += (int)gridDim.x * 8) {
         const int64_t lin = P->cell_base + (int64_t)r * ncx;
         // at most kMaxCellsAxis cells: four per lane, 32 apart
         uint32_t beg[4], off[4], cnt[4], tot = 0;
-        if (lane < kPad) sh[warp][lane] = sh[warp][kPad + ncx + lane] = 0.0f;
+        if (lane < kPad) {
+            sh[warp][lane] = sh[warp][kPad + ncx + lane] = 0.0f;
+            box[warp][lane] = box[warp][kPad + ncx + lane] = ~0u;
+        }
 #pragma unroll
         for (int k = 0; k < 4; k++) {
             const int x = k * 32 + lane;
@@ -911,13 +916,36 @@ __global__ void __launch_bounds__(256) k_cell_rows(PatchDev* pd, Grid g, const f
             float m = 0.0f;
             for (int d = -K; d <= K; d++) m = fmaxf(m, sh[warp][kPad + x + d]);
             hnb_x[lin + x] = m;
+            float ylo = 255.0f, yhi = 0.0f, zlo = 255.0f, zhi = 0.0f;
             for (uint32_t u = 0; u < cnt[k]; u++) {
                 const uint32_t j = beg[k] + u;
                 const float4 q = r4[j];
+                ylo = fminf(ylo, q.y * qy);
+                yhi = fmaxf(yhi, q.y * qy);
+                zlo = fminf(zlo, q.z * qz);
+                zhi = fmaxf(zhi, q.z * qz);
                 g.row_rec[b + u] = make_float4(fmaf((float)x, s_f, q.x), q.y, q.z, q.w);
                 g.row_id[b + u] = j | ((uint32_t)x << kColBits);
             }
+            // rounded outwards (no particle: all ones, which any other undercuts)
+            box[warp][kPad + x] = cnt[k] == 0 ? ~0u
+                : __float2uint_rd(fmaxf(ylo, 0.0f)) | __float2uint_rd(fmaxf(255.0f - yhi, 0.0f)) << 8 |
+                  __float2uint_rd(fmaxf(zlo, 0.0f)) << 16 | __float2uint_rd(fmaxf(255.0f - zhi, 0.0f)) << 24;
         }
+        __syncwarp();
+        uint32_t inset = 0, nbox = 0;
+        for (int x = lane; x < ncx; x += 32) {
+            uint32_t m = ~0u;
+            for (int d = -K; d <= K; d++) m = __vminu4(m, box[warp][kPad + x + d]);
+            g.row_box[lin + x] = m;
+            if (m != ~0u) {
+                inset += __dp4a(m, 0x01010101u, 0u);
+                nbox++;
+            }
+        }
+        inset = __reduce_add_sync(0xffffffffu, inset);
+        nbox = __reduce_add_sync(0xffffffffu, nbox);
+        if (lane == 0 && nbox) atomicAdd(&P->row_inset, (unsigned long long)inset << 32 | nbox);
         __syncwarp();
     }
 }

@@ -130,6 +130,9 @@ __device__ __forceinline__ uint32_t round8(uint32_t v) { return (v + 7u) & ~7u; 
 template <int MODE, bool EXACT = true>
 struct RowSink {
     static constexpr bool kDefer = MODE == kWalkRing && EXACT;
+    // rows pruned by their boxes (not in the counting and repair walks, which
+    // would spill)
+    static constexpr bool kBoxes = MODE == kWalkRing;
     uint32_t* col;      // the row's first pool entry; flat mode: nullptr = count only
     uint32_t* ring;     // this lane's ring (ring mode): slot k at ring[32 k], then
                         // kPend slots of deferred positions at ring[32 (kRing + k)]
@@ -229,9 +232,10 @@ __device__ __forceinline__ uint32_t stencil_code(const PatchDev* P, int dcx, int
 
 // ---- any i, small j: the rows of fine cells within reach -------------------
 // (2 kx + 1) x (2 kz + 1) rows around i's cell (every z plane with ZW), each
-// clipped to the chord of the search sphere: one run of the row copy.  Bound
-// by instruction issue (70 % of cycles) and by the L1's gathers (71 %).  A
-// walk over cells, pruned by each cell's tight box, tested about as many
+// clipped to the chord of the search sphere, whose distance from the row is
+// that from the row's particles (row_gap2) where these lie in layers: one run
+// of the row copy.  Bound by instruction issue (70 % of cycles) and by the
+// L1's gathers (71 %).  A walk over cells, pruned by each cell's tight box, tested about as many
 // candidates but paid ~35 instructions for each of ~82 cells and ended a
 // group of four in every one of them; the rows come to 13-21 runs.  Search of
 // 8 M particles (a 200^3 lattice disturbed by 4 %) 10.24 -> 8.63 ms, of the
@@ -291,6 +295,40 @@ __device__ __forceinline__ RowCtx row_ctx(const NbArgs& a, const PatchDev* P, in
     return c;
 }
 
+// byte k of w as a float
+template <int k>
+__device__ __forceinline__ float byte_f32(uint32_t w)
+{
+    return __uint_as_float(__byte_perm(w, 0x4b000000u, 0x7650u + k)) - 8388608.0f;
+}
+
+// the gap between a position at (y, z) of a row's frame and the particles of
+// the row, squared, from its box (Grid::row_box; 0: the whole cell); WZ: z too
+template <bool WZ>
+__device__ __forceinline__ float row_gap2(uint32_t b, float y, float z, float s_f, float sz_f)
+{
+    const float uy = s_f * (1.0f / 255.0f);
+    const float gy = fmaxf(fmaxf(fmaf(byte_f32<0>(b), uy, -y), fmaf(byte_f32<1>(b), uy, y - s_f)), 0.0f);
+    if (!WZ) return gy * gy;
+    const float uz = sz_f * (1.0f / 255.0f);
+    const float gz = fmaxf(fmaxf(fmaf(byte_f32<2>(b), uz, -z), fmaf(byte_f32<3>(b), uz, z - sz_f)), 0.0f);
+    return fmaf(gy, gy, gz * gz);
+}
+
+// Whether the boxes are worth their look-up, which costs a row some 20
+// instructions: a mean inset above 1/8 of the edge.  Layers of a lattice, also
+// of a sheared one, leave 0.2 to 0.35, random positions 0.02.  Search of the
+// 200^3 patch, without / with boxes: undisturbed 7.9 / 6.9 ms, over 50 steps
+// 8.32 / 7.49; 33^3 72 / 64 us; 100^3 disturbed, h raised behind the surface
+// 1121 / 1072 us; 200^3 disturbed by 4 %, which leaves 0.26 but fewer rows that
+// a whole warp skips, 8.57 / 8.76 ms.  The irregular patch, where they are not
+// used, would take 6 % longer with them.
+constexpr uint32_t kBoxInset = 1020u / 8u;   // of the four insets' sum, 4 x 255
+__device__ __forceinline__ bool use_boxes(const PatchDev* P)
+{
+    return (uint32_t)(P->row_inset >> 32) > kBoxInset * (uint32_t)P->row_inset;
+}
+
 // the z plane iz of the walk
 struct RowPlane {
     int czj, zd;
@@ -323,22 +361,26 @@ __device__ __forceinline__ RowPlane row_plane(const RowCtx& c, int iz)
 }
 
 // the row dcy of plane p: its run of the row copy, tested
-template <class S, int ZW>
+template <class S, int ZW, bool BOX>
 __device__ __forceinline__ void walk_row(const NbArgs& a, const PatchDev* P, int64_t i, const RowCtx& c, const RowPlane& p,
-                                         int dcy, S& row)
+                                         int dcy, uint32_t lrow, uint32_t box, S& row)
 {
-    const float ysh = (float)dcy * c.s_f;
-    const float gy = fmaxf(dcy > 0 ? ysh - c.yi : (dcy < 0 ? c.yi - (ysh + c.s_f) : 0.0f), 0.0f);
-    const float rem2 = c.Rg2 - fmaf(gy, gy, p.gz2);
+    const float yo = c.yi - (float)dcy * c.s_f;
+    float gap2;
+    if (BOX) {
+        gap2 = row_gap2<!ZW>(box, yo, p.zo, c.s_f, c.sz_f);
+    } else {
+        const float gy = fmaxf(dcy > 0 ? -yo : (dcy < 0 ? yo - c.s_f : 0.0f), 0.0f);
+        gap2 = fmaf(gy, gy, p.gz2);
+    }
+    const float rem2 = c.Rg2 - gap2;
     if (!(rem2 > 0.0f)) return;
     // the chord, in cells (Rg's margins cover the rounding and the FP32 cell
     // assignment)
     const float half = __fsqrt_rn(rem2) * c.inv_s;
     const int x0 = max((int)floorf(c.xs - half), c.xlo), x1 = min((int)floorf(c.xs + half), c.xhi);
     if (x0 > x1) return;
-    const uint32_t lrow = c.cbase + ((uint32_t)p.czj * (uint32_t)c.ncy + (uint32_t)(c.cy + dcy)) * (uint32_t)c.ncx;
     const uint32_t kb = a.g.row[lrow + (uint32_t)x0].x, ke = a.g.row[lrow + (uint32_t)x1].y;
-    const float yo = c.yi - ysh;
     const bool rowcode = (uint32_t)(dcy + 2) <= 4u && (uint32_t)p.zd <= 4u;
     // row_id + add: the column word where the code exists
     const uint32_t add = (uint32_t)(2 + 5 * (dcy + 2) + 25 * p.zd - c.cx) << kColBits;
@@ -382,14 +424,21 @@ __device__ __forceinline__ void walk_row(const NbArgs& a, const PatchDev* P, int
     }
 }
 
-template <class S, int ZW>
+template <class S, int ZW, bool BOX>
 __device__ __forceinline__ void walk_rows(const NbArgs& a, const PatchDev* P, int64_t i, int kx, int kz, float Rg2, S& row)
 {
     const RowCtx c = row_ctx<ZW>(a, P, i, kx, kz, Rg2);
     for (int iz = 0; iz < c.nz; iz++) {
         const RowPlane p = row_plane<ZW>(c, iz);
         if (p.gz2 >= Rg2) continue;
-        for (int dcy = c.ylo; dcy <= c.yhi; dcy++) walk_row<S, ZW>(a, P, i, c, p, dcy, row);
+        uint32_t lrow = c.cbase + ((uint32_t)p.czj * (uint32_t)c.ncy + (uint32_t)(c.cy + c.ylo)) * (uint32_t)c.ncx;
+        uint32_t next = BOX ? a.g.row_box[lrow + (uint32_t)c.cx] : 0u;
+        for (int dcy = c.ylo; dcy <= c.yhi; dcy++) {
+            const uint32_t box = next;
+            if (BOX && dcy < c.yhi) next = a.g.row_box[lrow + (uint32_t)(c.ncx + c.cx)];
+            walk_row<S, ZW, BOX>(a, P, i, c, p, dcy, lrow, box, row);
+            lrow += (uint32_t)c.ncx;
+        }
     }
 }
 
@@ -494,8 +543,10 @@ template <class S>
 __device__ __forceinline__ void walk_all(const NbArgs& a, const PatchDev* P, int64_t i, bool big, S& row)
 {
     const RowReach R = row_reach(a, P, a.g.cellxyz[i], (float)a.h[i], big);
-    if (R.zw) walk_rows<S, 1>(a, P, i, R.kx, R.kz, R.Rg2, row);
-    else walk_rows<S, 0>(a, P, i, R.kx, R.kz, R.Rg2, row);
+    // (the boxes hold the rows as far as K cells)
+    if (R.zw) walk_rows<S, 1, false>(a, P, i, R.kx, R.kz, R.Rg2, row);
+    else if (S::kBoxes && R.kx <= P->K && use_boxes(P)) walk_rows<S, 0, S::kBoxes>(a, P, i, R.kx, R.kz, R.Rg2, row);
+    else walk_rows<S, 0, false>(a, P, i, R.kx, R.kz, R.Rg2, row);
     if (P->nbig > 0) row = walk_coarse<S>(a, P, i, row);
 }
 

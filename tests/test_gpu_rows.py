@@ -65,3 +65,41 @@ def test_rows(B, orc, kind, n, cf):
         assert np.array_equal(o, nb.off) and np.array_equal(c, nb.col)
         assert np.array_equal(sim.field("nown").astype(np.int64), nb.nown)
     sim.close()
+
+
+def _layers(kind, e):
+    """A lattice of e^3 particles whose rows are pruned by where their particles lie."""
+    rng = np.random.default_rng(5)
+    dx, n = 1.0 / e, e ** 3
+    g = (np.arange(e) + 0.5) * dx - 0.5
+    z, y, x = (t.ravel().copy() for t in np.meshgrid(g, g, g, indexing="ij"))
+    h = np.full(n, 1.44 * dx)
+    if kind == "sheared":        # layers along z, rows at an angle to y
+        y += 0.3 * x
+    elif kind == "jittered":     # with particles whose radius outgrows the stencil
+        for t in (x, y):
+            t += rng.uniform(-0.1, 0.1, n) * dx
+        h *= rng.uniform(0.9, 1.1, n)
+        h[::101] *= rng.uniform(2.0, 4.0, len(h[::101]))
+    elif kind == "periodic":     # layers on the period's ends, gaps between them
+        z = np.floor((z + 0.5) * e / 3.0) * 3.0 * dx - 0.5
+        x += rng.uniform(-0.3, 0.3, n) * dx
+    v = np.zeros(n)
+    return {"x": x, "y": y, "z": z, "vx": v, "vy": v, "vz": v, "m": np.full(n, 1.0 / n), "h": h, "u": np.ones(n)}
+
+
+@pytest.mark.parametrize("e,cf", [(18, 0.0), (18, 0.4), (37, 0.0), (37, 0.4), (37, 1.0)])
+@pytest.mark.parametrize("kind", ["lattice", "sheared", "jittered", "periodic"])
+def test_layers(B, orc, kind, e, cf):
+    f = _layers(kind, e)
+    n = e ** 3
+    sim = B.SPH(n, cell_factor=cf, max_pairs=800 * n)
+    sim.set_particles(f)
+    nb = orc.neighbors(f["x"], f["y"], f["z"], f["h"], 1.0, nthreads=os.cpu_count() or 1)
+    for _ in range(2):
+        sim.find_neighbors()
+        off, col, perm = sim.neighbors()
+        o, c = lists_to_original(off, col, perm, n)
+        assert np.array_equal(o, nb.off) and np.array_equal(c, nb.col)
+        assert np.array_equal(sim.field("nown").astype(np.int64), nb.nown)
+    sim.close()
