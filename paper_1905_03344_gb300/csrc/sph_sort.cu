@@ -860,9 +860,10 @@ int launch_refresh_records(const Launch& L, int64_t n, const State& s, const uin
 // The row copy of the small particles' search records (see Grid): one warp
 // per row of fine cells, which reserves the row's slots (where in the copy a
 // row lies depends on scheduling, its contents do not), scans the cells'
-// counts and copies their particles: 36 bytes a particle, 0.11 ms at 8 M.
-// The warp also leaves the row's running maximum of h over K cells to each
-// side in hnb_x.  blockIdx.y is the patch.
+// counts and copies their particles: 36 bytes a particle, 0.15 ms at 8 M
+// (0.13 without the boxes).  The warp also leaves, over K cells to each side of
+// every cell, the row's largest h in hnb_x and where its particles lie in y and
+// z in row_box.  blockIdx.y is the patch.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_cell_rows(PatchDev* pd, Grid g, const float4* r4, int K, float* hnb_x)
 {
