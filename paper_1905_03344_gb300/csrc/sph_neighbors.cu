@@ -219,22 +219,24 @@ __device__ __forceinline__ void team_tests(const NbArgs& a, const PatchDev* P, c
                 dz = f.y - q.z;
             }
             if (wrap) dz = fmaf(-lz_f, rintf(dz * inv_lz), dz);
-            float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            if (!in_run || j == C.i) r2 = 1e30f;
+            // (masked by a predicate: no value of r2 is beyond every threshold,
+            // which are in the caller's units)
+            const bool valid = in_run && j != C.i;
+            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
             float d = r2 - fmaxf(C.Ti, q.w), o = r2 - C.Ti;
             if (EXACT) {
                 // the guard band: decided exactly
                 const float eps = C.eps * fmaxf(C.Ti, q.w);
-                if (fminf(fabsf(d), fabsf(o)) <= eps) {
+                if (valid && fminf(fabsf(d), fabsf(o)) <= eps) {
                     const int x = exact_pair_at(a, (int64_t)C.i, j, P->lz);
                     d = x & 1 ? -1.0f : 1.0f;
                     o = x & 2 ? -1.0f : 1.0f;
                 }
-                C.own += (uint32_t)(o < 0.0f);
+                C.own += (uint32_t)(valid && o < 0.0f);
             } else {
                 d -= C.eps * fmaxf(C.Ti, q.w);
             }
-            const bool in = d < 0.0f;
+            const bool in = valid && d < 0.0f;
             const uint32_t m = (__ballot_sync(0xffffffffu, in) >> tsh) & ((1u << kTeam) - 1u);
             const uint32_t p = C.cnt + (uint32_t)__popc(m & lt);
             if (in && p < C.lim) __stcs(C.col + p, w);
