@@ -176,6 +176,7 @@ sph_status fail(sph_ctx* c, sph_status s, const std::string& msg)
 sph_status cuda_fail(sph_ctx* c, cudaError_t e, const char* where)
 {
     std::string msg = std::string(where) + ": " + cudaGetErrorString(e);
+    if (c) c->bins_valid = false;   // a launch that failed may be the binning's
     if (is_sticky(e)) {
         if (c) c->poisoned = true;
         return fail(c, SPH_ESTATE, msg + " (context poisoned)");
@@ -601,6 +602,9 @@ sph_status check_status(sph_ctx* ctx, const char* where)
     if (e != cudaSuccess) return cuda_fail(ctx, e, where);
     collect_profile(ctx);
     const int st = *ctx->h_status;
+    // the binning's sort may be what gave up: its order is not written then,
+    // and the lists, which a sum that failed keeps, are binned again
+    if (st & kStBad) ctx->bins_valid = false;
     if (st & kStOverflow)
         return fail(ctx, SPH_EOVERFLOW, std::string(where) + ": neighbour lists exceed max_pairs");
     if (st & kStNonFinite) return fail(ctx, SPH_ENONFINITE, std::string(where) + ": non-finite value");

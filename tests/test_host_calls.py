@@ -1,0 +1,88 @@
+"""The host side of the C ABI on a device that runs nothing (fake_runtime.cpp, fake_launches.cu):
+what a call launches after an earlier one failed.  A failing launch, copy or
+wait is a value the fake returns, so no GPU is needed or harmed."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_1905_03344_gb300 import binding, build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+OVERFLOW, NONFINITE, TIMEOUT = 1, 2, 4      # bits of the device status word
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    out = tmp_path_factory.mktemp("host_calls")
+    objs = []
+    jobs = []
+    for src in (os.path.join(build.CSRC, "sph_api.cu"), os.path.join(HERE, "fake_launches.cu"),
+                os.path.join(HERE, "fake_runtime.cpp")):
+        objs.append(str(out / (os.path.basename(src) + ".o")))
+        jobs.append(subprocess.Popen([build.nvcc()] + build.ARCH + ["-std=c++17", "-Xcompiler", "-fPIC",
+                                      "--expt-relaxed-constexpr", "-I", build.CSRC, "-c", src, "-o", objs[-1]]))
+    assert all(j.wait() == 0 for j in jobs)
+    so = str(out / "libfake.so")
+    # bound to its own symbols, whatever CUDA runtime the process has loaded
+    subprocess.run(["g++", "-shared", "-Wl,-Bsymbolic", "-o", so] + objs, check=True)
+    L = ctypes.CDLL(so)
+    for name, (res, args) in binding.SIGNATURES.items():
+        if hasattr(L, name):
+            getattr(L, name).restype, getattr(L, name).argtypes = res, args
+    L.fake_log.restype = ctypes.c_char_p
+    L.fake_alloc.restype, L.fake_alloc.argtypes = ctypes.c_void_p, [ctypes.c_size_t, ctypes.c_int]
+    return L
+
+
+class Fake:
+    def __init__(self, lib, n=64, **kw):
+        self.lib = lib
+        lib.fake_reset(b"", 0, -1)
+        cfg = binding.SphConfig()
+        lib.sph_config_default(ctypes.byref(cfg))
+        cfg.max_particles = n
+        for k, v in kw.items():
+            setattr(cfg, k, v)
+        self.ctx = ctypes.c_void_p()
+        assert lib.sph_create(ctypes.byref(cfg), ctypes.byref(self.ctx)) == binding.SPH_OK
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *exc):
+        self.lib.sph_destroy(self.ctx)
+
+    def expect(self, status_at="", bits=0, copies_left=-1):
+        """Clears the log; the launch of that name will report bits."""
+        self.lib.fake_reset(status_at.encode(), bits, copies_left)
+
+    def log(self):
+        return self.lib.fake_log().decode().split()
+
+    def set_particles(self, n, ptrs=None, on_device=0):
+        if ptrs is None:
+            self.buf = np.ones((9, n))
+            ptrs = [self.buf[k].ctypes.data for k in range(9)]
+        return self.lib.sph_set_particles(self.ctx, n, *ptrs, on_device)
+
+    def step(self, n=1):
+        return self.lib.sph_step(self.ctx, n, None)
+
+
+def test_bins_of_a_failed_call_are_not_used(lib):
+    """A binning pass that gave up leaves its order unwritten; the next sum
+    bins again instead of reading it."""
+    with Fake(lib, pair_bins=32) as f:
+        assert f.set_particles(40) == binding.SPH_OK
+        assert lib.sph_find_neighbors(f.ctx) == binding.SPH_OK
+        f.expect("bins", TIMEOUT)
+        assert lib.sph_density(f.ctx) == binding.SPH_ETIMEOUT
+        assert f.log() == ["bins", "density_binned"]
+        f.expect()
+        assert lib.sph_density(f.ctx) == binding.SPH_OK
+        assert f.log() == ["bins", "density_binned"]
+        assert lib.sph_momentum_energy(f.ctx) == binding.SPH_OK
+        assert f.log() == ["bins", "density_binned", "momentum_binned"]     # the same bins
