@@ -1194,6 +1194,7 @@ sph_status sph_step(sph_ctx* ctx, int32_t nsteps, double* dt_last)
         // with reused lists: sort and search only when the superset no longer
         // holds every pair (the previous step's check says so)
         const bool rebuild = !reuse || !ctx->sup_valid;
+        ctx->sup_valid = false;         // until this step's own check
         // the first step after new particles runs outside the graphs: a
         // captured step must not depend on the state having no search yet
         if (graph && !ctx->fresh) {
@@ -1238,8 +1239,10 @@ sph_status sph_step(sph_ctx* ctx, int32_t nsteps, double* dt_last)
         }
     }
     st = after_launches(ctx, "sph_step");
-    if (st != SPH_OK) return st;
-    st = check_status(ctx, "sph_step");
+    if (st == SPH_OK) st = check_status(ctx, "sph_step");
+    // the superset of a step that failed may be incomplete, whatever the check
+    // of the particles' moves said
+    if (st != SPH_OK) ctx->sup_valid = false;
     ctx->nb_valid = false;
     ctx->rho_valid = ctx->acc_valid = (st == SPH_OK);
     ctx->cnt_valid = st == SPH_OK;

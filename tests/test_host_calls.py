@@ -86,3 +86,20 @@ def test_bins_of_a_failed_call_are_not_used(lib):
         assert f.log() == ["bins", "density_binned"]
         assert lib.sph_momentum_energy(f.ctx) == binding.SPH_OK
         assert f.log() == ["bins", "density_binned", "momentum_binned"]     # the same bins
+
+
+@pytest.mark.parametrize("failing", ["sort", "superset", "filter"])
+def test_superset_of_a_failed_step_is_not_used(lib, failing):
+    """A step that fails may leave its candidate superset incomplete, with rows
+    outside the pool; no particle moves, so the check that follows every step
+    finds that the superset would still hold."""
+    with Fake(lib, list_skin=0.2) as f:
+        assert f.set_particles(40) == binding.SPH_OK
+        f.expect(failing, TIMEOUT if failing == "sort" else OVERFLOW)
+        assert f.step() == (binding.SPH_ETIMEOUT if failing == "sort" else binding.SPH_EOVERFLOW)
+        f.expect()
+        assert f.step() == binding.SPH_OK
+        assert "superset" in f.log()
+        f.expect()
+        assert f.step() == binding.SPH_OK       # while a good one is used again
+        assert "superset" not in f.log() and "filter" in f.log()
