@@ -1013,7 +1013,6 @@ sph_status sph_set_particles(sph_ctx* ctx, int64_t n, const double* x, const dou
     // others are copied first and checked where they land
     bool direct = on_device && n > 0;
     for (int k = 0; k < 9; k++) direct = direct && (uintptr_t)src[k] % sizeof(double) == 0;
-    ctx->n = n;
     if (direct) {
         launch_load(launch_of(ctx), n, src, s, ctx->perm[0], ctx->status);
     } else {
@@ -1023,6 +1022,7 @@ sph_status sph_set_particles(sph_ctx* ctx, int64_t n, const double* x, const dou
         const double* own[9] = {s.x, s.y, s.z, s.vx, s.vy, s.vz, s.m, s.h, s.u};
         if (n > 0) launch_load(launch_of(ctx), n, own, s, ctx->perm[0], ctx->status);
     }
+    ctx->n = n;             // (a copy that failed leaves the count the patch tables are made for)
     int64_t offs[2] = {0, n};
     st = setup_patches(ctx, 1, offs);
     if (st != SPH_OK) return st;

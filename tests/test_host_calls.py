@@ -103,3 +103,16 @@ def test_superset_of_a_failed_step_is_not_used(lib, failing):
         f.expect()
         assert f.step() == binding.SPH_OK       # while a good one is used again
         assert "superset" not in f.log() and "filter" in f.log()
+
+
+@pytest.mark.parametrize("copies", [0, 4])
+def test_failed_upload_leaves_the_particle_count(lib, copies):
+    """The patch tables are sized by the particle count: an upload that fails
+    changes neither."""
+    with Fake(lib) as f:
+        assert f.set_particles(24) == binding.SPH_OK
+        f.expect(copies_left=copies)
+        assert f.set_particles(40) == binding.SPH_ECUDA
+        f.expect()
+        f.step()        # (the runtime's last error is the copy's)
+        assert f.log()[:2] == ["items=24", "keys=24"]
