@@ -70,6 +70,7 @@ struct sph_ctx {
     sph_config cfg;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
+    int device = 0;
     int sms = 1;
     std::string err;
     bool poisoned = false;
@@ -204,6 +205,20 @@ bool dalloc(sph_ctx* ctx, T*& p, size_t count)
     ctx->allocs.push_back(q);
     p = (T*)q;
     return true;
+}
+
+// Whether a kernel may take p: memory of the context's device, aligned.  Other
+// pointers go through copies, which know the memory of any device and refuse
+// what is none, where a kernel would fault.
+bool kernel_memory(const sph_ctx* ctx, const void* p, size_t align)
+{
+    cudaPointerAttributes a;
+    if ((uintptr_t)p % align != 0) return false;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == ctx->device);
 }
 
 Launch launch_of(const sph_ctx* ctx) { return Launch{ctx->stream, ctx->sms}; }
@@ -857,6 +872,7 @@ sph_status sph_create(const sph_config* cfg_in, sph_ctx** out)
     ctx->cfg = cfg;
     int dev = 0;
     cudaGetDevice(&dev);
+    ctx->device = dev;
     cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, dev);
     if (cfg.cuda_stream) {
         ctx->stream = (cudaStream_t)cfg.cuda_stream;
@@ -1009,10 +1025,10 @@ sph_status sph_set_particles(sph_ctx* ctx, int64_t n, const double* x, const dou
     }
     ctx->cur = 0;
     State& s = ctx->st[0];
-    // device arrays (of aligned doubles) are copied and checked in one pass;
-    // others are copied first and checked where they land
+    // arrays on this device are copied and checked in one pass; others are
+    // copied first and checked where they land
     bool direct = on_device && n > 0;
-    for (int k = 0; k < 9; k++) direct = direct && (uintptr_t)src[k] % sizeof(double) == 0;
+    for (int k = 0; k < 9; k++) direct = direct && kernel_memory(ctx, src[k], sizeof(double));
     if (direct) {
         launch_load(launch_of(ctx), n, src, s, ctx->perm[0], ctx->status);
     } else {
@@ -1129,7 +1145,7 @@ sph_status sph_get_neighbors(sph_ctx* ctx, const uint64_t** off, const uint32_t*
 sph_status sph_copy_neighbors(sph_ctx* ctx, uint64_t* off, uint32_t* col, uint32_t* perm, int on_device)
 {
     if (on_device && ctx && !ctx->poisoned && ctx->nb_valid && !ctx->canon_valid && off && col && perm &&
-        (uintptr_t)off % sizeof(uint64_t) == 0 && (uintptr_t)col % sizeof(uint32_t) == 0) {
+        kernel_memory(ctx, off, sizeof(uint64_t)) && kernel_memory(ctx, col, sizeof(uint32_t))) {
         // the rows straight into the caller's buffers
         sph_status st = begin_call(ctx);
         if (st != SPH_OK) return st;

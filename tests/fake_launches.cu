@@ -40,7 +40,12 @@ int launch_gather(const Launch&, int64_t, const uint32_t*, const uint32_t*, cons
 int launch_refresh_records(const Launch&, int64_t, const State&, const uint16_t*, const PatchDev*, const uint32_t*,
                            const Recs&, const Fp64&, int, int) { return 1; }
 int launch_cell_tables(const Launch&, int, PatchDev*, const Grid&, const float4*, int, float*, unsigned long long*) { return 1; }
-int launch_nb_lists(const Launch&, const NbArgs& a, int exact) { note(exact ? "lists" : "superset", a.status); return 1; }
+int launch_nb_lists(const Launch&, const NbArgs& a, int exact)
+{
+    note(exact ? "lists" : "superset", a.status);
+    a.pool_used[1] = 8;
+    return 1;
+}
 int launch_nb_filter(const Launch&, const NbArgs& a, const uint32_t*, const uint32_t*) { note("filter", a.status); return 1; }
 int launch_pair_bins(const Launch&, int64_t, const uint32_t*, const RadixSort&, uint32_t*, int* status) { note("bins", status); return 1; }
 int launch_density(const Launch&, const PairArgs& a, int, int) { note("density", a.status); return 1; }

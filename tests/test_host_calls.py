@@ -116,3 +116,32 @@ def test_failed_upload_leaves_the_particle_count(lib, copies):
         f.expect()
         f.step()        # (the runtime's last error is the copy's)
         assert f.log()[:2] == ["items=24", "keys=24"]
+
+
+@pytest.mark.parametrize("where", ["here", "peer", "host"])
+def test_kernels_take_only_this_devices_memory(lib, where):
+    """on_device pointers are handed to a kernel where they are this device's
+    memory.  Another device's is copied, as the runtime does between any two,
+    and a host pointer is refused by the copy."""
+    n = 32
+    with Fake(lib) as f:
+        def buf(k):
+            if where == "host":
+                f.keep = getattr(f, "keep", []) + [np.ones(k)]
+                return f.keep[-1].ctypes.data
+            return lib.fake_alloc(8 * k, 0 if where == "here" else 1)
+        ptrs = [buf(n) for _ in range(9)]
+        f.expect()
+        st = f.set_particles(n, ptrs, 1)
+        if where == "here":
+            assert st == binding.SPH_OK and f.log() == ["load_direct"]
+        elif where == "peer":
+            assert st == binding.SPH_OK and f.log() == ["copy"] * 9 + ["load_own"]
+        else:
+            assert st == binding.SPH_ECUDA and f.log() == []
+        assert f.set_particles(n) == (binding.SPH_ECUDA if where == "host" else binding.SPH_OK)
+        assert lib.sph_find_neighbors(f.ctx) == binding.SPH_OK
+        f.expect()
+        st = lib.sph_copy_neighbors(f.ctx, buf(n + 1), buf(8), buf(n), 1)
+        assert not [w for w in f.log() if w.endswith("elsewhere")]
+        assert st == (binding.SPH_ECUDA if where == "host" else binding.SPH_OK)
