@@ -225,7 +225,8 @@ __device__ __forceinline__ bool seedable(double x)
 // sqrt(x) by Goldschmidt's iteration from an FP32 reciprocal square root (22
 // bits; one step makes 44), then the residual's correction (Markstein,
 // "Computation of elementary functions on the IBM RISC System/6000
-// processor", 1990): six FP64 operations
+// processor", 1990): six FP64 operations.  Within 0.5 ulp and 2^-29 ulp of the
+// root: the nearest double, or beside a tie its neighbour
 __device__ __forceinline__ double sqrt_fp64(double x)
 {
     if (!seedable(x)) return sqrt(x);
@@ -236,9 +237,10 @@ __device__ __forceinline__ double sqrt_fp64(double x)
     const double g1 = fma(g, e, g), h1 = fma(h, e, h);
     return fma(fma(-g1, g1, x), h1, g1);
 }
-// n / x for a positive x, to about an ulp: the FP32 reciprocal's error
-// e = 1 - x y (23 bits), y (1 + e + e^2) leaves e^3 (Newton's iteration of
-// the third order)
+// n / x for a positive x: the FP32 reciprocal's error e = 1 - x y (21 bits or
+// more), y (1 + e + e^2) leaves e^3 (Newton's iteration of the third order).
+// Within 1.5 ulp and 2^-10 ulp of the quotient (the library's: 0.5), one of
+// them for the rounding of the reciprocal
 __device__ __forceinline__ double div_fp64(double n, double x)
 {
     if (!seedable(x)) return n / x;
