@@ -88,3 +88,15 @@ def test_noalloc_rejects_beyond_its_fixed_scratch(B):
                                        ctypes.c_void_p(out.data_ptr()), None)
     assert st == B.SPH_EINVAL
     assert b"16777216" in B.lib().sph_noalloc_last_error()
+
+
+def test_noalloc_of_more_slots_than_threads(B, orc):
+    """Eight shares for every SM, of 256 particles or more: 400,001 particles
+    fill 782 slots of a 152-SM chip, so that a thread of the closing sum takes
+    several; the next calls (157 slots, one) find them left in the array.  (The
+    sizes of the first test fill 235, 79 and 20.)"""
+    for call, (n, seed) in enumerate(((400001, 4), (40001, 5), (200, 6))):
+        f = _fields(n, seed)
+        want = orc.conserved(*[f[k] for k in NAMES])
+        got = _noalloc(B, f)
+        assert np.all(np.abs(got - want) <= 1e-12 * _scales(f)), (call, got, want)
