@@ -316,6 +316,8 @@ NbArgs nb_args(sph_ctx* ctx)
 {
     NbArgs a;
     a.n = ctx->n;
+    a.K = stencil_k(ctx->cell_factor);
+    a.npatch = ctx->npatch;
     a.pd = ctx->pd;
     a.g = ctx->grid;
     a.r4 = ctx->rec.r4;

@@ -51,7 +51,6 @@ __device__ __forceinline__ bool union_decision(const NbArgs& a, const PatchDev* 
 // ---- mixed precision --------------------------------------------------------
 template <int KERN, bool GH>
 struct DensSink {
-    static constexpr bool kBoxes = false;
     PairSrc src;
     PairSide I;
     float inv2h;
@@ -76,7 +75,6 @@ struct DensSink {
 
 template <int KERN, bool GH>
 struct MomSink {
-    static constexpr bool kBoxes = false;
     PairSrc src;
     PairSide I;
     float4 vi, ti;
@@ -122,7 +120,6 @@ struct MomSink {
 // ---- FP64 -------------------------------------------------------------------
 template <int KERN, bool GH>
 struct DensSinkD {
-    static constexpr bool kBoxes = false;
     const PairArgs* pa;
     double xi, yi, zi, w, lz;
     int kn;
@@ -144,7 +141,6 @@ struct DensSinkD {
 
 template <int KERN, bool GH>
 struct MomSinkD {
-    static constexpr bool kBoxes = false;
     const PairArgs* pa;
     SideD I;
     int kn;
@@ -183,7 +179,7 @@ __device__ __forceinline__ void count_pairs(const NbArgs& a, uint32_t cnt)
 }
 
 // ---- kernels ----------------------------------------------------------------
-template <int KERN, bool GH>
+template <int K, int KERN, bool GH>
 __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_DEN_MINB)
     k_fused_density_mixed(NbArgs a, const __grid_constant__ PairArgs pa)
 {
@@ -200,7 +196,7 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_DEN_MINB)
             const bool big = i >= P->end - (int64_t)P->nbig;
             DensSink<KERN, GH> s = {src, pair_side(pa, P, i), pa.r.rv[i].w, pa.kernel_n, P->zmode,
                                     0.0f, 0.0f, 0.0f, 0.0f, 0u, 0u};
-            walk_all<DensSink<KERN, GH>>(a, P, i, big, s);
+            walk_all<DensSink<KERN, GH>, K>(a, P, i, big, s);
             density_finish<GH>(pa, i, s.I.ri.w, s.inv2h, kb8, gam, s.sum, s.comp, s.sumd, s.compd);
             a.cnt[i] = s.cnt;
             a.nown[i] = s.own;
@@ -210,7 +206,7 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_DEN_MINB)
     }
 }
 
-template <int KERN, bool GH>
+template <int K, int KERN, bool GH>
 __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_MOM_MINB)
     k_fused_momentum_mixed(NbArgs a, const __grid_constant__ PairArgs pa)
 {
@@ -231,14 +227,14 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_MOM_MINB)
             const float wi2 = vi.w * vi.w;
             MomSink<KERN, GH> s = {src, pair_side(pa, P, i), vi, pa.r.rt[i], wi2 * wi2 * vi.w, Kc,
                                    pa.kernel_n, P->zmode, qlane, 0u, 0u, {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}};
-            walk_all<MomSink<KERN, GH>>(a, P, i, big, s);
+            walk_all<MomSink<KERN, GH>, K>(a, P, i, big, s);
             s.finish();
             momentum_finish(pa, i, gscale, s.A);
         }
     }
 }
 
-template <int KERN, bool GH>
+template <int K, int KERN, bool GH>
 __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_DEN_MINB)
     k_fused_density_fp64(NbArgs a, const __grid_constant__ PairArgs pa)
 {
@@ -253,7 +249,7 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_DEN_MINB)
             const bool big = i >= P->end - (int64_t)P->nbig;
             DensSinkD<KERN, GH> s = {&pa, pa.s.x[i], pa.s.y[i], pa.s.z[i], pa.f.w[i], P->lz,
                                      pa.kernel_n, 0.0, 0.0, 0u, 0u};
-            walk_all<DensSinkD<KERN, GH>>(a, P, i, big, s);
+            walk_all<DensSinkD<KERN, GH>, K>(a, P, i, big, s);
             density_finish_fp64<GH>(pa, i, s.sum, s.sumd);
             a.cnt[i] = s.cnt;
             a.nown[i] = s.own;
@@ -263,7 +259,7 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_DEN_MINB)
     }
 }
 
-template <int KERN, bool GH>
+template <int K, int KERN, bool GH>
 __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_MOM_MINB)
     k_fused_momentum_fp64(NbArgs a, const __grid_constant__ PairArgs pa)
 {
@@ -279,7 +275,7 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_FUSED_MOM_MINB)
         if (i < U.end) {
             const bool big = i >= P->end - (int64_t)P->nbig;
             MomSinkD<KERN, GH> s = {&pa, side_fp64(pa, P, i), pa.kernel_n, qlane, 0u, 0u, {0.0, 0.0, 0.0, 0.0}};
-            walk_all<MomSinkD<KERN, GH>>(a, P, i, big, s);
+            walk_all<MomSinkD<KERN, GH>, K>(a, P, i, big, s);
             s.finish();
             momentum_finish_fp64(pa, i, S80, s.A);
         }
@@ -300,13 +296,19 @@ void launch_fused(const Launch& L, Kern kern, const NbArgs& a, const PairArgs& p
     kern<<<(unsigned)blocks, 32 * kNbtWarps, 0, L.stream>>>(a, pa);
 }
 
+#define SPH_FUSED_K(KERNEL, KERN, GH, L, a, pa)                                                   \
+    switch ((a).K) {                                                                              \
+    case 1: launch_fused(L, KERNEL<1, KERN, GH>, a, pa); break;                                   \
+    case 2: launch_fused(L, KERNEL<2, KERN, GH>, a, pa); break;                                   \
+    default: launch_fused(L, KERNEL<3, KERN, GH>, a, pa); break;                                  \
+    }
 #define SPH_FUSED_DISPATCH(KERNEL, L, a, pa)                                                      \
     if ((pa).kernel == SPH_KERNEL_SINC) {                                                         \
-        if ((pa).grad_h) launch_fused(L, KERNEL<SPH_KERNEL_SINC, true>, a, pa);                   \
-        else launch_fused(L, KERNEL<SPH_KERNEL_SINC, false>, a, pa);                              \
+        if ((pa).grad_h) { SPH_FUSED_K(KERNEL, SPH_KERNEL_SINC, true, L, a, pa); }                \
+        else { SPH_FUSED_K(KERNEL, SPH_KERNEL_SINC, false, L, a, pa); }                           \
     } else {                                                                                      \
-        if ((pa).grad_h) launch_fused(L, KERNEL<SPH_KERNEL_WENDLAND, true>, a, pa);               \
-        else launch_fused(L, KERNEL<SPH_KERNEL_WENDLAND, false>, a, pa);                          \
+        if ((pa).grad_h) { SPH_FUSED_K(KERNEL, SPH_KERNEL_WENDLAND, true, L, a, pa); }            \
+        else { SPH_FUSED_K(KERNEL, SPH_KERNEL_WENDLAND, false, L, a, pa); }                       \
     }
 
 }  // namespace sphg

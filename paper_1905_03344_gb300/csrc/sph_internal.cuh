@@ -97,6 +97,9 @@ struct PatchDev {
     // of the row boxes (Grid::row_box): the sum of the four insets over the
     // fine cells that have one, << 32, and the count of these
     unsigned long long row_inset;
+    // ... of hnb / (the cell's largest h) - 1 in 1/256, over the fine cells that
+    // hold particles
+    unsigned long long h_spread;
     // time state
     double dt, dt_prev;
     int64_t step;
@@ -121,7 +124,10 @@ struct State {
 
 // Cell record, 16 bytes: particles [x, y) of the sorted order (x = y: empty;
 // fine cells hold small particles, coarse cells big ones), z = the largest h
-// in the cell (FP32 bits).
+// in the cell (FP32 bits), w = for fine cells the tight box of the cell's
+// particles, as insets from the cell faces in 1/kBoxQ of the cell edge:
+// bits 0-4 low x, 5-9 high x, 10-14 low y, 15-19 high y, 20-24 low z,
+// 25-29 high z (rounded outwards up to the FP32 rounding of the offsets).
 //
 // The search reads its small candidates from a second copy of the records, in
 // which the particles of a row of fine cells (all x at one y, z) are
@@ -129,6 +135,7 @@ struct State {
 // cell in that copy, row_rec = {x from the grid's origin, oy, oz, 4 h^2} and
 // row_id = sorted slot | x cell << kColBits.  A row of the search sphere is
 // then one run of slots, where the Morton order holds one run per cell.
+constexpr int kBoxQ = 32;
 struct Grid {
     uint4* cell;         // [cell] record above
     uint2* row;          // [fine cell]
@@ -419,6 +426,8 @@ int64_t scan_tmp_words(int64_t n);
 
 struct NbArgs {
     int64_t n;
+    int K;                               // stencil half-extent of every patch
+    int npatch;
     const PatchDev* pd;
     Grid g;
     const float4* r4;

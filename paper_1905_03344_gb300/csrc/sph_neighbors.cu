@@ -22,11 +22,11 @@ namespace sphg {
 
 // counting walk (col = nullptr) and repair walk (straight to the pool): one
 // out-of-line copy serves both
-template <bool EXACT>
+template <bool EXACT, int K>
 __device__ __noinline__ RowSink<kWalkFlat, EXACT> walk_all_flat(const NbArgs& a, const PatchDev* P, int64_t i,
                                                              bool big, RowSink<kWalkFlat, EXACT> row)
 {
-    walk_all<RowSink<kWalkFlat, EXACT>>(a, P, i, big, row);
+    walk_all<RowSink<kWalkFlat, EXACT>, K>(a, P, i, big, row);
     return row;
 }
 
@@ -40,8 +40,12 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, int lane)
 }
 
 // EXACT = false: the candidate superset (every candidate within the scaled
-// search radius in FP32, no n_i)
-template <bool EXACT>
+// search radius in FP32, no n_i).  K = 0: the patches searched by rows; else
+// those searched by cells, with stencils of K.  Two kernels, since one that
+// branches between the two walks, at the 64 registers of eight blocks an SM,
+// took 3 % longer in either (200^3 8.85 -> 9.1 ms, 64 patches 5.97 -> 6.17); a
+// launch that finds no patch of its kind is done in 2 us.
+template <bool EXACT, int K>
 __global__ void __launch_bounds__(32 * kNbtWarps, SPH_NB_MINB) k_nb_thread(NbArgs a)
 {
     wait_before();
@@ -51,9 +55,11 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_NB_MINB) k_nb_thread(NbArg
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.hint_ok = 1;
     if (*a.status & kStBad) return;
     const unsigned long long pool_cap = (unsigned long long)a.pool_cap;
+    if (a.npatch == 1 && use_cells(a.pd) != (K > 0)) return;
     for (int64_t q = (int64_t)blockIdx.x * kNbtWarps + warp; q < a.nunits; q += (int64_t)gridDim.x * kNbtWarps) {
         const WorkItem U = a.units[q];
         const PatchDev* P = a.pd + U.patch;
+        if (use_cells(P) != (K > 0)) continue;
         const int64_t i = U.begin + lane;
         const bool act = i < U.end;
         // big particles sit at the end of their patch
@@ -64,7 +70,7 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_NB_MINB) k_nb_thread(NbArg
             const uint32_t hint = a.rowcap[i];
             if (hint == kNoHint) {
                 const RowSink<kWalkFlat, EXACT> rc =
-                    walk_all_flat<EXACT>(a, P, i, big, RowSink<kWalkFlat, EXACT>{nullptr, nullptr, 0u, 0u, 0u, 0u});
+                    walk_all_flat<EXACT, K>(a, P, i, big, RowSink<kWalkFlat, EXACT>{nullptr, nullptr, 0u, 0u, 0u, 0u});
                 res = round8(rc.cnt);
             } else {
                 const uint32_t c = min(hint, (uint32_t)a.n);
@@ -81,7 +87,7 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_NB_MINB) k_nb_thread(NbArg
         unsigned long long r0 = base + (inc - res);
         RowSink<kWalkRing, EXACT> row = {a.col + r0, ring, ok ? res : 0u, 0u, 0u, 0u};
         if (act) {
-            walk_all<RowSink<kWalkRing, EXACT>>(a, P, i, big, row);
+            walk_all<RowSink<kWalkRing, EXACT>, K>(a, P, i, big, row);
             row.finish();
             // only a row that is in the pool (within the sink's reservation,
             // which is 0 for a warp whose reservation did not fit)
@@ -93,7 +99,7 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_NB_MINB) k_nb_thread(NbArg
             const uint32_t need = round8(row.cnt);
             r0 = atomicAdd(&a.pool_used[0], (unsigned long long)need);
             if (r0 + need <= pool_cap) {
-                const RowSink<kWalkFlat, EXACT> rr = walk_all_flat<EXACT>(
+                const RowSink<kWalkFlat, EXACT> rr = walk_all_flat<EXACT, K>(
                     a, P, i, big, RowSink<kWalkFlat, EXACT>{a.col + r0, nullptr, need, 0u, 0u, 0u});
                 row.cnt = rr.cnt;
                 row.own = rr.own;
@@ -114,13 +120,13 @@ __global__ void __launch_bounds__(32 * kNbtWarps, SPH_NB_MINB) k_nb_thread(NbArg
     }
 }
 
-template <bool EXACT>
+template <bool EXACT, int K>
 void launch_nb_thread(const Launch& L, const NbArgs& a)
 {
     const size_t smem = sizeof(uint32_t) * 32 * (kRing + kPend) * kNbtWarps;
     static int per_sm = 0;
     if (!per_sm) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_nb_thread<EXACT>, 32 * kNbtWarps, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_nb_thread<EXACT, K>, 32 * kNbtWarps, smem);
         if (per_sm < 1) per_sm = 1;
         // shared memory only for the rings of the resident CTAs: the rest is L1
         int smem_max = 0, dev = 0;
@@ -130,10 +136,10 @@ void launch_nb_thread(const Launch& L, const NbArgs& a)
             const size_t need = (size_t)per_sm * (smem + 1024);
             int pct = (int)((need * 100 + (size_t)smem_max - 1) / (size_t)smem_max);
             pct = pct < 1 ? 1 : (pct > 100 ? 100 : pct);
-            cudaFuncSetAttribute(k_nb_thread<EXACT>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+            cudaFuncSetAttribute(k_nb_thread<EXACT, K>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
         }
     }
-    launch_next(k_nb_thread<EXACT>, L.sms * per_sm, 32 * kNbtWarps, smem, L.stream, a);
+    launch_next(k_nb_thread<EXACT, K>, L.sms * per_sm, 32 * kNbtWarps, smem, L.stream, a);
 }
 
 // ---- a team of lanes per particle ------------------------------------------
@@ -493,18 +499,23 @@ static void launch_nb_team(const Launch& L, const NbArgs& a)
 }
 
 template <bool EXACT>
-static void launch_nb(const Launch& L, const NbArgs& a)
+static int launch_nb(const Launch& L, const NbArgs& a)
 {
-    if (a.n <= kTeamMost) launch_nb_team<EXACT>(L, a);
-    else launch_nb_thread<EXACT>(L, a);
+    if (a.n <= kTeamMost) {
+        launch_nb_team<EXACT>(L, a);
+        return 1;
+    }
+    launch_nb_thread<EXACT, 0>(L, a);
+    if (a.K == 1) launch_nb_thread<EXACT, 1>(L, a);
+    else if (a.K == 2) launch_nb_thread<EXACT, 2>(L, a);
+    else launch_nb_thread<EXACT, 3>(L, a);
+    return 2;
 }
 
 int launch_nb_lists(const Launch& L, const NbArgs& a, int exact)
 {
     if (a.n <= 0 || a.nunits <= 0) return 0;
-    if (exact) launch_nb<true>(L, a);
-    else launch_nb<false>(L, a);
-    return 1;
+    return exact ? launch_nb<true>(L, a) : launch_nb<false>(L, a);
 }
 
 // ---- exact lists from a reused candidate superset -------------------------

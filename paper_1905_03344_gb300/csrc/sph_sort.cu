@@ -302,6 +302,7 @@ __global__ void k_grid_params(int npatch, const PatchRed* red, PatchDev* pd, dou
     P.nbig = 0;
     P.row_fill = 0;
     P.row_inset = 0;
+    P.h_spread = 0;
     P.kc = kc;
     P.ncxc = (int)ncxc;
     P.ncyc = (int)ncyc;
@@ -863,8 +864,16 @@ int launch_refresh_records(const Launch& L, int64_t n, const State& s, const uin
 // counts and copies their particles: 36 bytes a particle, 0.15 ms at 8 M
 // (0.13 without the boxes).  The warp also leaves, over K cells to each side of
 // every cell, the row's largest h in hnb_x and where its particles lie in y and
-// z in row_box.  blockIdx.y is the patch.
+// z in row_box, and each cell's tight box in its record.  blockIdx.y is the
+// patch.
 // ---------------------------------------------------------------------------
+// a distance from a face of the cell, in 1/255 of the edge, as an inset of a
+// cell's box, rounded down
+__device__ __forceinline__ uint32_t box_inset(float d255)
+{
+    return min(__float2uint_rd(fmaxf(d255, 0.0f) * ((float)kBoxQ / 255.0f)), (uint32_t)kBoxQ - 1u);
+}
+
 __global__ void __launch_bounds__(256) k_cell_rows(PatchDev* pd, Grid g, const float4* r4, int K, float* hnb_x)
 {
     wait_before();
@@ -917,10 +926,12 @@ __global__ void __launch_bounds__(256) k_cell_rows(PatchDev* pd, Grid g, const f
             float m = 0.0f;
             for (int d = -K; d <= K; d++) m = fmaxf(m, sh[warp][kPad + x + d]);
             hnb_x[lin + x] = m;
-            float ylo = 255.0f, yhi = 0.0f, zlo = 255.0f, zhi = 0.0f;
+            float xlo = 255.0f, xhi = 0.0f, ylo = 255.0f, yhi = 0.0f, zlo = 255.0f, zhi = 0.0f;
             for (uint32_t u = 0; u < cnt[k]; u++) {
                 const uint32_t j = beg[k] + u;
                 const float4 q = r4[j];
+                xlo = fminf(xlo, q.x * qy);
+                xhi = fmaxf(xhi, q.x * qy);
                 ylo = fminf(ylo, q.y * qy);
                 yhi = fmaxf(yhi, q.y * qy);
                 zlo = fminf(zlo, q.z * qz);
@@ -928,6 +939,9 @@ __global__ void __launch_bounds__(256) k_cell_rows(PatchDev* pd, Grid g, const f
                 g.row_rec[b + u] = make_float4(fmaf((float)x, s_f, q.x), q.y, q.z, q.w);
                 g.row_id[b + u] = j | ((uint32_t)x << kColBits);
             }
+            if (cnt[k])
+                g.cell[lin + x].w = box_inset(xlo) | box_inset(255.0f - xhi) << 5 | box_inset(ylo) << 10 |
+                                    box_inset(255.0f - yhi) << 15 | box_inset(zlo) << 20 | box_inset(255.0f - zhi) << 25;
             // rounded outwards (no particle: all ones, which any other undercuts)
             box[warp][kPad + x] = cnt[k] == 0 ? ~0u
                 : __float2uint_rd(fmaxf(ylo, 0.0f)) | __float2uint_rd(fmaxf(255.0f - yhi, 0.0f)) << 8 |
@@ -962,10 +976,13 @@ __global__ void __launch_bounds__(256) k_cell_rows(PatchDev* pd, Grid g, const f
 // h_s.  Many such cells (h wide but smooth in space, as behind the free
 // surface of a patch) favour a 3-cell stencil over median-sized cells; few
 // (h varying from particle to particle) favour cells of edge h_s.
-__global__ void __launch_bounds__(256) k_cell_hnb(const PatchDev* pd, Grid g, int K, const float* hnb_x, unsigned long long* vote)
+//
+// And how far hnb is above each cell's own largest h, which decides between
+// the walk over rows and the one over cells (use_cells).
+__global__ void __launch_bounds__(256) k_cell_hnb(PatchDev* pd, Grid g, int K, const float* hnb_x, unsigned long long* vote)
 {
     wait_before();
-    const PatchDev* P = pd + blockIdx.y;
+    PatchDev* P = pd + blockIdx.y;
     const int ncx = P->ncx, ncy = P->ncy, ncz = P->ncz;
     const int64_t nxy = (int64_t)ncx * ncy;
     const int64_t nfine = nxy * ncz;
@@ -973,7 +990,7 @@ __global__ void __launch_bounds__(256) k_cell_hnb(const PatchDev* pd, Grid g, in
     const float lim = 0.8f * P->hs_f;
     // every z plane when they are fewer than 2K+1
     const int kz = 2 * K + 1 > ncz ? (ncz - 1) / 2 + 1 : K;
-    uint32_t ne = 0, nn = 0;
+    uint32_t ne = 0, nn = 0, over = 0;
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nfine; c += (int64_t)gridDim.x * blockDim.x) {
         const int z = (int)(c / nxy), y = (int)(c - z * nxy) / ncx;
         const int ylo = max(-K, -y), yhi = min(K, ncy - 1 - y);
@@ -990,13 +1007,16 @@ __global__ void __launch_bounds__(256) k_cell_hnb(const PatchDev* pd, Grid g, in
         if (cr.x < cr.y) {
             ne++;
             nn += (uint32_t)(wide && m < lim);
+            over += (uint32_t)fminf(fmaf(__fdividef(m, __uint_as_float(cr.z)), 256.0f, -256.0f), 1024.0f);
         }
     }
     for (int o = 16; o > 0; o >>= 1) {
         ne += __shfl_xor_sync(0xffffffffu, ne, o);
         nn += __shfl_xor_sync(0xffffffffu, nn, o);
+        over += __shfl_xor_sync(0xffffffffu, over, o);
     }
     if ((threadIdx.x & 31) == 0 && ne) {
+        atomicAdd(&P->h_spread, (unsigned long long)over << 32 | ne);
         atomicAdd(&vote[0], (unsigned long long)ne);
         atomicAdd(&vote[1], (unsigned long long)nn);
     }

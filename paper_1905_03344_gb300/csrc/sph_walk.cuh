@@ -8,7 +8,8 @@
 // candidate of its kind once:
 //   small i, small j: the rows of fine cells (all x at one y, z) around i's
 //     cell, at most K away, each clipped to the chord of the radius
-//     2 max(h_i, hnb) (hnb: the largest h around i's cell);
+//     2 max(h_i, hnb) (hnb: the largest h around i's cell), or the cells one
+//     by one, pruned by each cell's own largest h (use_cells);
 //   big i, small j:   the same rows as far as 2 max(h_i, h_s) reaches;
 //   any i, big j:     the 3 x 3 x 3 coarse cells around i's coarse cell
 //     (only when the patch has big particles).
@@ -329,6 +330,25 @@ __device__ __forceinline__ bool use_boxes(const PatchDev* P)
     return (uint32_t)(P->row_inset >> 32) > kBoxInset * (uint32_t)P->row_inset;
 }
 
+// Whether a patch's lists are searched cell by cell: where h varies so much
+// from cell to cell that the one radius of a row reaches far beyond what most
+// of its cells need.  The mean over the cells of hnb / (the cell's largest h)
+// tells: above 1.06 for stencils of 1 or 2 cells, above 1.12 for 3.  Search in
+// ms, rows / cells, at a mean of 1.0 (200^3 disturbed by 4 %) 8.9 / 10.5, 1.04
+// (100^3 disturbed, h raised behind the surface) 1.10 / 1.18, 1.05 to 1.06
+// (100^3 after 20 to 50 steps) 1.41 / 1.36, 1.1 to 1.15 (64 patches of 60^3)
+// 21.4 / 19.6, 1.2 to 1.3 (of 35^3) 5.6 / 4.1, 1.5 (of 20^3) 1.8 / 1.1; with 3
+// cells 1.07 (100^3) 1.36 / 1.45, 1.11 to 1.18 (64 patches of 60^3) 22.9 / 23.9
+// and 26.4 / 26.1, more (of 35^3) 4.8 / 4.4.  On the irregular patch (1.16) h
+// varies from particle to particle and a cell's box says little, a mean inset
+// of 0.03 where the others have 0.09 or more: 1.29 / 1.41.
+constexpr uint32_t kCellsInset = 1020u / 16u;
+__device__ __forceinline__ bool use_cells(const PatchDev* P)
+{
+    const uint32_t over = (uint32_t)(P->h_spread >> 32), n = (uint32_t)P->h_spread;   // of the mean - 1, in 1/256
+    return over > (P->K <= 2 ? 15u : 30u) * n && (uint32_t)(P->row_inset >> 32) > kCellsInset * (uint32_t)P->row_inset;
+}
+
 // the z plane iz of the walk
 struct RowPlane {
     int czj, zd;
@@ -538,15 +558,166 @@ __device__ __noinline__ S walk_coarse(const NbArgs& a, const PatchDev* P, int64_
     return row;
 }
 
-// the whole search for particle i
+// ---- small i, small j: the fine cells around i's cell, one by one ----------
+// squared distance from i to the tight box of a fine cell: g*r are the raw
+// distances from i to the cell's near faces (-1e30 along an axis where i is
+// inside the cell's slab), the insets come from the cell record at the given
+// bit offsets, in units qs = s / kBoxQ (qsz = sz / kBoxQ along z)
+__device__ __forceinline__ float tight_gap2(uint32_t box, float gxr, uint32_t xs, float gyr, uint32_t ys, float gzr,
+                                            uint32_t zs, float qs, float qsz)
+{
+    const float tx = fmaxf(fmaf((float)((box >> xs) & 31u), qs, gxr), 0.0f);
+    const float ty = fmaxf(fmaf((float)((box >> ys) & 31u), qs, gyr), 0.0f);
+    const float tz = fmaxf(fmaf((float)((box >> zs) & 31u), qsz, gzr), 0.0f);
+    return fmaf(tx, tx, fmaf(ty, ty, tz * tz));
+}
+
+// The (2K+1)^3 cells in the order of the rows' walk, so that both write the
+// same row: a cell farther than 2 max(h_i, hnb), or whose tight box is farther
+// than 2 max(h_i, the cell's largest h), is left out, the others are tested
+// kGroup candidates at a time.  ~35 instructions for each of ~82 cells: the
+// rows' walk has fewer where h is even.  The list-free sums always search by
+// it (200^3, 10 steps: density 11.2 ms by rows, 10.5 by cells, momentum 16.9
+// and 16.2; 64 patches 7.6 and 7.3, 11.6 and 11.4): they have no registers to
+// spare for the rows' boxes.
+template <class S, int K, int ZW>
+__device__ __forceinline__ void walk_cells(const NbArgs& a, const PatchDev* P, int64_t i, const RowReach& R, S& row)
+{
+    const float s_f = P->s_f, sz_f = P->sz_f, lz_f = P->lz_f, inv_lz = 1.0f / P->lz_f;
+    const int ncx = P->ncx, ncy = P->ncy, ncz = P->ncz;
+    const uint32_t cbase = (uint32_t)P->cell_base;
+    const uint32_t i32 = (uint32_t)i;
+    const float4 ri = a.r4[i];
+    const uint32_t cc = a.g.cellxyz[i];
+    const int cx = cc & 255, cy = (cc >> 8) & 255, cz = cc >> 16;
+    const float hf = (float)a.h[i];
+    const float Ti = ri.w, Rg2 = R.Rg2;
+    // a stencil of at most 2 cells keeps its compile-time bounds
+    const int kx = K <= 2 ? K : R.kx, kz = K <= 2 ? K : R.kz;
+    // every z cell visited (ZW): shifts of up to ncz - 1 cells along z
+    const float tol = guard_tol(s_f / hf, ZW ? max(K, ncz) : K);
+    const float flo = 1.0f - tol, fhi = 1.0f + tol;
+    const float slack = (1.0f / 4096.0f) * s_f;
+    const float Rc = 2.0f * (1.0f + 1.0f / 512.0f);
+    const float qs = s_f * (1.0f / kBoxQ), qsz = sz_f * (1.0f / kBoxQ);
+    const int nz = ZW ? ncz : 2 * kz + 1;
+    for (int iz = 0; iz < nz; iz++) {
+        int czj, zd;
+        float zsh, gz2;
+        // raw distance from i to the near z face of the plane (-big: the own
+        // plane, or every plane)
+        float gzr = -1e30f;
+        uint32_t zshift = 20;
+        if (!ZW) {
+            const int dcz = iz - kz;
+            czj = cz + dcz;
+            if (czj < 0) czj += ncz;
+            else if (czj >= ncz) czj -= ncz;
+            zsh = (float)dcz * sz_f;
+            if (dcz != 0) gzr = dcz > 0 ? (float)dcz * sz_f - ri.z : ri.z - (float)(dcz + 1) * sz_f;
+            zshift = dcz > 0 ? 20u : 25u;
+            const float gg = fmaxf(gzr, 0.0f);
+            gz2 = gg * gg;
+            zd = dcz + 2;
+        } else {
+            czj = cz + iz;
+            if (czj >= ncz) czj -= ncz;
+            zsh = (float)iz * sz_f;
+            gz2 = 0.0f;
+            zd = iz;
+        }
+        if (gz2 >= Rg2) continue;
+        const float zo = ri.z - zsh;
+        for (int dcy = -kx; dcy <= kx; dcy++) {
+            const int cyj = cy + dcy;
+            if ((unsigned)cyj >= (unsigned)ncy) continue;
+            const float gyr = dcy > 0 ? (float)dcy * s_f - ri.y : (dcy < 0 ? ri.y - (float)(dcy + 1) * s_f : -1e30f);
+            const uint32_t yshift = dcy > 0 ? 10u : 15u;
+            const float gy = fmaxf(gyr, 0.0f);
+            const float gzy2 = fmaf(gy, gy, gz2);
+            if (gzy2 >= Rg2) continue;
+            const float yo = ri.y - (float)dcy * s_f;
+            const uint32_t lrow = cbase + ((uint32_t)czj * (uint32_t)ncy + (uint32_t)cyj) * (uint32_t)ncx + (uint32_t)cx;
+            const uint32_t kkrow = (uint32_t)(2 + 5 * (dcy + 2) + 25 * zd);
+            // a stencil of 3 reaches cells 3 away, which have no stencil code
+            const bool rowcode = K <= 2 || ((uint32_t)(dcy + 2) <= 4u && (uint32_t)zd <= 4u);
+            // one copy of the candidate loop for all x offsets (code size)
+#pragma unroll 1
+            for (int dcx = -kx; dcx <= kx; dcx++) {
+                if ((unsigned)(cx + dcx) >= (unsigned)ncx) continue;
+                const float gxr = dcx > 0 ? (float)dcx * s_f - ri.x : (dcx < 0 ? ri.x - (float)(dcx + 1) * s_f : -1e30f);
+                const float gx = fmaxf(gxr, 0.0f);
+                const float d2 = fmaf(gx, gx, gzy2);
+                if (d2 >= Rg2) continue;
+                const uint32_t lin = lrow + (uint32_t)dcx;
+                const uint4 cr = a.g.cell[lin];
+                const uint2 se = make_uint2(cr.x, cr.y);
+                if (se.x >= se.y) continue;
+                const float R = fmaxf(hf, __uint_as_float(cr.z)) * Rc + slack;
+                if (tight_gap2(cr.w, gxr, dcx > 0 ? 0u : 5u, gyr, yshift, gzr, zshift, qs, qsz) >= R * R) continue;
+                const float xo = ri.x - (float)dcx * s_f;
+                const uint32_t kk = (rowcode && (K <= 2 || (dcx >= -2 && dcx <= 2)) ? kkrow + (uint32_t)dcx : kFarCode) << kColBits;
+                // (the record array is padded past its end; slots past the cell
+                // are masked)
+                for (uint32_t jb = se.x; jb < se.y; jb += kGroup) {
+                    const float4* qp = a.r4 + jb;
+                    float4 q[kGroup];
+#pragma unroll
+                    for (int u = 0; u < kGroup; u++) q[u] = qp[u];
+                    const uint32_t rem = se.y - jb;
+                    float r2[kGroup], T[kGroup];
+                    unsigned near = 0;
+#pragma unroll
+                    for (int u = 0; u < kGroup; u++) {
+                        const float dx = xo - q[u].x, dy = yo - q[u].y;
+                        float dz = zo - q[u].z;
+                        if (ZW) dz = fmaf(-lz_f, rintf(dz * inv_lz), dz);
+                        r2[u] = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                        T[u] = fmaxf(Ti, q[u].w);
+                        if ((uint32_t)u < rem && r2[u] <= T[u] * fhi) near |= 1u << u;
+                    }
+                    if (!near) continue;
+                    const uint32_t c0 = row.mark();
+#pragma unroll
+                    for (int u = 0; u < kGroup; u++) {
+                        if (!(near & (1u << u))) continue;
+                        const uint32_t j = jb + (uint32_t)u;
+                        if (j == i32) continue;
+                        row.decide(a, P, i, j, r2[u], Ti, T[u], flo, fhi, j | kk);
+                    }
+                    row.group_end(c0);
+                }
+            }
+        }
+    }
+}
+
+// big particles keep the walk over rows (by value through an out-of-line call,
+// so that the caller's row stays in registers)
 template <class S>
+__device__ __noinline__ S walk_big_rows(const NbArgs& a, const PatchDev* P, int64_t i, RowReach R, S row)
+{
+    if (R.zw) walk_rows<S, 1, false>(a, P, i, R.kx, R.kz, R.Rg2, row);
+    else walk_rows<S, 0, false>(a, P, i, R.kx, R.kz, R.Rg2, row);
+    return row;
+}
+
+// the whole search for particle i; K = 0: by rows, K = 1, 2, 3 (the patch's
+// stencil): small particles by cells
+template <class S, int K>
 __device__ __forceinline__ void walk_all(const NbArgs& a, const PatchDev* P, int64_t i, bool big, S& row)
 {
     const RowReach R = row_reach(a, P, a.g.cellxyz[i], (float)a.h[i], big);
-    // (the boxes hold the rows as far as K cells)
-    if (R.zw) walk_rows<S, 1, false>(a, P, i, R.kx, R.kz, R.Rg2, row);
-    else if (S::kBoxes && R.kx <= P->K && use_boxes(P)) walk_rows<S, 0, S::kBoxes>(a, P, i, R.kx, R.kz, R.Rg2, row);
-    else walk_rows<S, 0, false>(a, P, i, R.kx, R.kz, R.Rg2, row);
+    if constexpr (K > 0) {
+        if (big) row = walk_big_rows<S>(a, P, i, R, row);
+        else if (R.zw) walk_cells<S, K, 1>(a, P, i, R, row);
+        else walk_cells<S, K, 0>(a, P, i, R, row);
+    } else {
+        // (the boxes hold the rows as far as K cells)
+        if (R.zw) walk_rows<S, 1, false>(a, P, i, R.kx, R.kz, R.Rg2, row);
+        else if (S::kBoxes && R.kx <= P->K && use_boxes(P)) walk_rows<S, 0, S::kBoxes>(a, P, i, R.kx, R.kz, R.Rg2, row);
+        else walk_rows<S, 0, false>(a, P, i, R.kx, R.kz, R.Rg2, row);
+    }
     if (P->nbig > 0) row = walk_coarse<S>(a, P, i, row);
 }
 
