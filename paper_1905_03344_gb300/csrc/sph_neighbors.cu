@@ -505,9 +505,12 @@ static int launch_nb(const Launch& L, const NbArgs& a)
         launch_nb_team<EXACT>(L, a);
         return 1;
     }
+    if (a.K == 1) {
+        launch_nb_thread<EXACT, 1>(L, a);
+        return 1;
+    }
     launch_nb_thread<EXACT, 0>(L, a);
-    if (a.K == 1) launch_nb_thread<EXACT, 1>(L, a);
-    else if (a.K == 2) launch_nb_thread<EXACT, 2>(L, a);
+    if (a.K == 2) launch_nb_thread<EXACT, 2>(L, a);
     else launch_nb_thread<EXACT, 3>(L, a);
     return 2;
 }

@@ -330,23 +330,34 @@ __device__ __forceinline__ bool use_boxes(const PatchDev* P)
     return (uint32_t)(P->row_inset >> 32) > kBoxInset * (uint32_t)P->row_inset;
 }
 
-// Whether a patch's lists are searched cell by cell: where h varies so much
-// from cell to cell that the one radius of a row reaches far beyond what most
-// of its cells need.  The mean over the cells of hnb / (the cell's largest h)
-// tells: above 1.06 for stencils of 1 or 2 cells, above 1.12 for 3.  Search in
-// ms, rows / cells, at a mean of 1.0 (200^3 disturbed by 4 %) 8.9 / 10.5, 1.04
-// (100^3 disturbed, h raised behind the surface) 1.10 / 1.18, 1.05 to 1.06
-// (100^3 after 20 to 50 steps) 1.41 / 1.36, 1.1 to 1.15 (64 patches of 60^3)
-// 21.4 / 19.6, 1.2 to 1.3 (of 35^3) 5.6 / 4.1, 1.5 (of 20^3) 1.8 / 1.1; with 3
-// cells 1.07 (100^3) 1.36 / 1.45, 1.11 to 1.18 (64 patches of 60^3) 22.9 / 23.9
-// and 26.4 / 26.1, more (of 35^3) 4.8 / 4.4.  On the irregular patch (1.16) h
-// varies from particle to particle and a cell's box says little, a mean inset
-// of 0.03 where the others have 0.09 or more: 1.29 / 1.41.
+// Whether a patch's lists are searched cell by cell.  A row has one radius and
+// its chord ends at a cell's face; a cell has a radius of its own.  So rows
+// lose where h varies so much from cell to cell that their one radius reaches
+// far beyond what most of the cells need, which the mean over the cells of
+// hnb / (the cell's largest h) tells, and where cells are large.  Search, rows /
+// cells, with stencils of 2 cells of edge h_s (ms):
+//   mean 1.0   200^3 disturbed by 4 %                        8.6 / 10.1
+//   1.04       100^3 disturbed, h raised behind the surface  1.10 / 1.18
+//   1.05-1.06  100^3 after 20 to 50 steps                    1.41 / 1.36
+//   1.1-1.15   64 patches of 60^3                            21.4 / 19.6
+//   1.2-1.3    of 35^3                                       5.6 / 4.1
+//   1.5        of 20^3                                       1.8 / 1.1
+// so above 1.06; but on the irregular patch (1.16) h varies from particle to
+// particle and a cell's box says little, a mean inset of 0.03 where the others
+// have 0.09 or more: 1.25 / 1.33.  With edges of 1.2 h_s, 100^3 at 1.05: 1.21 /
+// 1.13, of 1.4 h_s 1.31 / 1.12 and the irregular patch with adapting h 1.10 /
+// 0.93 (disturbed, h even: 0.72 / 0.76); of 1.9 h_s rows lose on all of these
+// (1.05 / 0.97 to 1.84 / 1.57), and with stencils of one cell, whose edges are
+// 2 h_s and more.  With 3 cells 100^3 (1.07) 1.36 / 1.45, 64 patches of 60^3
+// (1.11 to 1.18) 22.9 / 23.9 and 26.4 / 26.1, of 35^3 4.8 / 4.4.
 constexpr uint32_t kCellsInset = 1020u / 16u;
 __device__ __forceinline__ bool use_cells(const PatchDev* P)
 {
+    const float edge = P->s_f * __fdividef(1.0f, P->hs_f);      // in h_s
+    if (P->K == 1 || edge > 1.75f) return true;
     const uint32_t over = (uint32_t)(P->h_spread >> 32), n = (uint32_t)P->h_spread;   // of the mean - 1, in 1/256
-    return over > (P->K <= 2 ? 15u : 30u) * n && (uint32_t)(P->row_inset >> 32) > kCellsInset * (uint32_t)P->row_inset;
+    const uint32_t least = P->K == 3 ? 30u : edge > 1.15f ? 10u : 15u;
+    return over > least * n && ((P->K == 2 && edge > 1.3f) || (uint32_t)(P->row_inset >> 32) > kCellsInset * (uint32_t)P->row_inset);
 }
 
 // the z plane iz of the walk
@@ -581,7 +592,7 @@ __device__ __forceinline__ float tight_gap2(uint32_t box, float gxr, uint32_t xs
 // and 16.2; 64 patches 7.6 and 7.3, 11.6 and 11.4): they have no registers to
 // spare for the rows' boxes.
 template <class S, int K, int ZW>
-__device__ __forceinline__ void walk_cells(const NbArgs& a, const PatchDev* P, int64_t i, const RowReach& R, S& row)
+__device__ __forceinline__ void walk_cells(const NbArgs& a, const PatchDev* P, int64_t i, S& row)
 {
     const float s_f = P->s_f, sz_f = P->sz_f, lz_f = P->lz_f, inv_lz = 1.0f / P->lz_f;
     const int ncx = P->ncx, ncy = P->ncy, ncz = P->ncz;
@@ -591,6 +602,7 @@ __device__ __forceinline__ void walk_cells(const NbArgs& a, const PatchDev* P, i
     const uint32_t cc = a.g.cellxyz[i];
     const int cx = cc & 255, cy = (cc >> 8) & 255, cz = cc >> 16;
     const float hf = (float)a.h[i];
+    const RowReach R = row_reach(a, P, cc, hf, false);
     const float Ti = ri.w, Rg2 = R.Rg2;
     // a stencil of at most 2 cells keeps its compile-time bounds
     const int kx = K <= 2 ? K : R.kx, kz = K <= 2 ? K : R.kz;
@@ -695,8 +707,9 @@ __device__ __forceinline__ void walk_cells(const NbArgs& a, const PatchDev* P, i
 // big particles keep the walk over rows (by value through an out-of-line call,
 // so that the caller's row stays in registers)
 template <class S>
-__device__ __noinline__ S walk_big_rows(const NbArgs& a, const PatchDev* P, int64_t i, RowReach R, S row)
+__device__ __noinline__ S walk_big_rows(const NbArgs& a, const PatchDev* P, int64_t i, S row)
 {
+    const RowReach R = row_reach(a, P, a.g.cellxyz[i], (float)a.h[i], true);
     if (R.zw) walk_rows<S, 1, false>(a, P, i, R.kx, R.kz, R.Rg2, row);
     else walk_rows<S, 0, false>(a, P, i, R.kx, R.kz, R.Rg2, row);
     return row;
@@ -707,12 +720,12 @@ __device__ __noinline__ S walk_big_rows(const NbArgs& a, const PatchDev* P, int6
 template <class S, int K>
 __device__ __forceinline__ void walk_all(const NbArgs& a, const PatchDev* P, int64_t i, bool big, S& row)
 {
-    const RowReach R = row_reach(a, P, a.g.cellxyz[i], (float)a.h[i], big);
     if constexpr (K > 0) {
-        if (big) row = walk_big_rows<S>(a, P, i, R, row);
-        else if (R.zw) walk_cells<S, K, 1>(a, P, i, R, row);
-        else walk_cells<S, K, 0>(a, P, i, R, row);
+        if (big) row = walk_big_rows<S>(a, P, i, row);
+        else if (P->zmode) walk_cells<S, K, 1>(a, P, i, row);
+        else walk_cells<S, K, 0>(a, P, i, row);
     } else {
+        const RowReach R = row_reach(a, P, a.g.cellxyz[i], (float)a.h[i], big);
         // (the boxes hold the rows as far as K cells)
         if (R.zw) walk_rows<S, 1, false>(a, P, i, R.kx, R.kz, R.Rg2, row);
         else if (S::kBoxes && R.kx <= P->K && use_boxes(P)) walk_rows<S, 0, S::kBoxes>(a, P, i, R.kx, R.kz, R.Rg2, row);
