@@ -116,7 +116,7 @@ struct sph_ctx {
     uint32_t* perm[2] = {nullptr, nullptr};
     uint16_t* patch_of = nullptr;
     uint32_t *keys = nullptr, *vals = nullptr, *keys_alt = nullptr, *vals_alt = nullptr;
-    float* hnb_tmp = nullptr;   // one float per cell: the x-y pass of the grid's hnb
+    float* hnb_tmp = nullptr;   // one float per cell: the maxima along x of the grid's hnb
     uint32_t* hist = nullptr;      // the radix sort's work words
     Grid grid{};
     Recs rec{};

@@ -8,7 +8,7 @@
 // covers the bounding box in x, y and the period lz in z; a small particle
 // searches the (2K+1)^3 cells around its own (K = 1 for cell_factor >= 1,
 // 2 for >= 1/2, 3 below) for small neighbours, row by row, pruned by the
-// largest h around its cell.  Big
+// largest h around its cell, or cell by cell, pruned by each cell's own.  Big
 // particles are indexed separately by coarse cells (aligned blocks of 2^kc
 // fine cells with edge >= 2 h_max), which every particle searches for big
 // neighbours; a big particle searches the fine grid as far as its own 2 h.

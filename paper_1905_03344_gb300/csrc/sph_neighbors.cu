@@ -153,12 +153,13 @@ void launch_nb_thread(const Launch& L, const NbArgs& a)
 // would write.
 //
 // Bound by instruction issue: about 1600 warp instructions a particle against
-// 870 of the thread walk, so the line lies where the chip fills up.  Search
-// in us, thread / team: lattice 20^3 95 / 28, 33^3 100 / 70, 45^3 139 / 168; h
-// raised behind the surface 20^3 143 / 53, 33^3 171 / 136, 45^3 200 / 298;
-// irregular 20^3 182 / 66, 33^3 408 / 152, 45^3 473 / 421.  A team whose lanes
-// take whole rows instead (hits collected in shared memory) took 33 us at
-// 20^3, 101 at 33^3 and 424 on the irregular 33^3.
+// 870 of the thread walk, so the line lies where 152 SMs fill up; on the
+// irregular patch, whose threads wait for the longest row of their warp, that
+// is past 91,000 particles.  Search in us, thread / team: lattice 20^3 95 / 28,
+// 33^3 100 / 70, 45^3 139 / 168; h raised behind the surface 20^3 143 / 53,
+// 33^3 171 / 136, 45^3 200 / 298; irregular 20^3 182 / 66, 33^3 408 / 152, 45^3
+// 473 / 421.  A team whose lanes take whole rows instead (hits collected in
+// shared memory) took 33 us at 20^3, 101 at 33^3 and 424 on the irregular 33^3.
 constexpr int kTeam = 8;
 constexpr int kTeams = 32 / kTeam;      // particles a warp searches for at a time
 constexpr int kTeamRuns = 32;           // runs written down at a time
@@ -392,11 +393,11 @@ __global__ void __launch_bounds__(32 * kNbtWarps, 5) k_nb_team(const __grid_cons
         const int64_t begin = U.begin + (part & ((1 << sub_log) - 1)) * width;
         const int n = (int)min((int64_t)width, U.end - begin);
         if (n <= 0) continue;
-        // lane l holds particle begin + l's row: words reserved, their place
-        // in the warp's reservation, words and n_i found
+        // lane l holds particle begin + l's row: words reserved, words and n_i
+        // found
         const bool act = lane < n;
         const uint32_t hint = act ? a.rowcap[begin + lane] : 0u;
-        uint32_t res = 0, off = 0, cnt = 0, own = 0;
+        uint32_t res = 0, cnt = 0, own = 0;
         unsigned long long r0 = 0;
         bool ok = true;
         // pass 0 counts the rows (without hints), 1 writes them, 2 writes the

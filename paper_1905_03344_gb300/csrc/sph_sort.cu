@@ -115,8 +115,7 @@ __global__ void __launch_bounds__(256) k_reset_red(int npatch, PatchRed* red, So
 // ---------------------------------------------------------------------------
 // A1a': per patch, a histogram of h / h_max in kHBins bins (integer counts,
 // so independent of the order of the atomics); it sets the class threshold.
-// Lanes of a warp that fall into the same bin (on a lattice, all of them)
-// add their count with one atomic.
+// One atomic on shared memory per particle, one on the patch's bin per block.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_h_hist(State s, const WorkItem* items, int nitems, PatchRed* red)
 {
@@ -495,8 +494,11 @@ int launch_scan_u32_to_u64(const Launch& L, int64_t n, const uint32_t* in, uint6
 }
 
 // ---------------------------------------------------------------------------
-// Stable LSD radix sort, 8-bit digits, one kernel per pass.  The digits of
-// all passes are counted while the keys are made.  A block takes the next
+// Stable LSD radix sort, 8-bit digits, one kernel per pass, after Adinets and
+// Merrill, "Onesweep: a faster least significant digit radix sort for GPUs",
+// 2022, with the decoupled look-back of Merrill and Garland, "Single-pass
+// parallel prefix scan with decoupled look-back", 2016.  The digits of all
+// passes are counted while the keys are made.  A block takes the next
 // tile (in the order of a ticket), ranks its keys stably (warp match +
 // per-warp counters, warps in tile order), publishes the tile's digit counts
 // and looks back over the tiles before it for their sum, each of which is
@@ -510,8 +512,8 @@ int launch_scan_u32_to_u64(const Launch& L, int64_t n, const uint32_t* in, uint6
 // stage, write), so by how many tiles are resident: five blocks on an SM with
 // 12 keys a thread, 48 registers and 35 KB; 16 keys at 128 registers, two
 // blocks, took 100 us a pass at 8 M where this takes 72, votes per digit bit
-// in place of the match 75, 8 keys 73.  Up to 622,592 keys (four tiles an SM)
-// the tiles have 1024 keys, which keeps more SMs busy.  The pass per digit of
+// in place of the match 75, 8 keys 73.  Up to 622,592 keys (four tiles on each
+// of 152 SMs) the tiles have 1024 keys, which keeps more SMs busy.  The pass per digit of
 // a histogram, a three-kernel scan and a scatter (with a copy back after an
 // odd number of passes) that this replaces took 15 launches where this takes
 // 3: 460 -> 216 us at 8 M, 126 -> 51 us at 1 M, 102 -> 21 us at 8000.
@@ -661,8 +663,7 @@ int launch_radix_sort(const Launch& L, int64_t n, int passes, const RadixSort& r
 
 // ---------------------------------------------------------------------------
 // Row-length bins of the pair sums: key = octave of |N(i)|, sorted stably by
-// one radix pass; the bin starts are the scanned digit offsets of the first
-// tile.
+// one radix pass; the bin starts are the scanned digit counts.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_octave_keys(int64_t n, const uint32_t* cnt, uint32_t* keys, uint32_t* vals, uint32_t* hist)
 {

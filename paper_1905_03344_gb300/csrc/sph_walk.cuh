@@ -235,14 +235,15 @@ __device__ __forceinline__ uint32_t stencil_code(const PatchDev* P, int dcx, int
 // (2 kx + 1) x (2 kz + 1) rows around i's cell (every z plane with ZW), each
 // clipped to the chord of the search sphere, whose distance from the row is
 // that from the row's particles (row_gap2) where these lie in layers: one run
-// of the row copy.  Bound by instruction issue (70 % of cycles) and by the
-// L1's gathers (71 %).  A walk over cells, pruned by each cell's tight box, tested about as many
-// candidates but paid ~35 instructions for each of ~82 cells and ended a
-// group of four in every one of them; the rows come to 13-21 runs.  Search of
+// of the row copy.  Bound by instruction issue (75 % of cycles) and by the
+// L1's gathers (72 %).  The walk over cells tests about as many candidates but
+// pays ~35 instructions for each of ~82 cells and ends a group of four in
+// every one of them; the rows come to 13-21 runs.  From cells to rows, search of
 // 8 M particles (a 200^3 lattice disturbed by 4 %) 10.24 -> 8.63 ms, of the
 // 64-patch batch 7.66 -> 5.90, of the 80^3 irregular patch 1.41 -> 1.25, of
 // 45^3 176 -> 137 us; 100^3 with h raised by a third behind the surface 1.12
-// (unchanged: its cells are 1.3 times as wide).  Slower: lanes that leave the
+// (unchanged: its cells are 1.3 times as wide).  Where cells are still the
+// better, use_cells() says.  Slower: lanes that leave the
 // lockstep of the rows for their own runs (L1 77-90 % busy), hits without
 // branches, ids loaded only for hits, groups of 3 or 5.
 //
@@ -321,9 +322,10 @@ __device__ __forceinline__ float row_gap2(uint32_t b, float y, float z, float s_
 // of a sheared one, leave 0.2 to 0.35, random positions 0.02.  Search of the
 // 200^3 patch, without / with boxes: undisturbed 7.9 / 6.9 ms, over 50 steps
 // 8.32 / 7.49; 33^3 72 / 64 us; 100^3 disturbed, h raised behind the surface
-// 1121 / 1072 us; 200^3 disturbed by 4 %, which leaves 0.26 but fewer rows that
-// a whole warp skips, 8.57 / 8.76 ms.  The irregular patch, where they are not
-// used, would take 6 % longer with them.
+// (0.19) 1121 / 1072 us.  The irregular patch, where they are not used, would
+// take 6 % longer with them.  The line does not separate everything: a 200^3
+// lattice disturbed by 4 % (0.26) has as large an inset but fewer rows that a
+// whole warp skips, and pays 2 % for its boxes, 8.57 / 8.76 ms.
 constexpr uint32_t kBoxInset = 1020u / 8u;   // of the four insets' sum, 4 x 255
 __device__ __forceinline__ bool use_boxes(const PatchDev* P)
 {
