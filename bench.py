@@ -62,8 +62,9 @@ NB_BYTES_PER_PARTICLE = 48
 # profiles/launches_square_patch_200cubed.md), scaled to the benchmark's
 # launch by its entries.  None once the kernel has changed since; the
 # momentum figure is that of its 2-lanes-per-particle instantiation, the
-# search's that of both its 2- and 3-cell stencils (5.99 and 6.02 B).
-NB_DRAM_BYTES_PER_ENTRY = 5.99
+# search's that of its walk over rows with 2- and 3-cell stencils (5.97 and 6.00
+# B; cell by cell, as most of the 64 patches after 20 steps, 6.35 B).
+NB_DRAM_BYTES_PER_ENTRY = 5.97
 MOMENTUM_DRAM_BYTES_PER_ENTRY = 7.90
 MOMENTUM_DRAM_TPP = 2
 
